@@ -19,6 +19,7 @@
 #include <utility>
 
 #include "internal.h"
+#include "project.cuh"
 
 namespace nrv {
 
@@ -76,7 +77,7 @@ nrv_status launch_clear_keys(const RViews& views, cudaStream_t s) {
     return NRV_OK;
 }
 
-// Tiles of the culling variant: TILE x TILE pixels; bound[t] holds the largest
+// Tiles of the chunk-culling variants: TILE x TILE pixels; bound[t] holds the largest
 // depth word (key >> 32) over the tile's pixels after a first pass over a
 // subset of the points.  Keys only decrease afterwards, so a point whose depth
 // word exceeds its tile's bound can never win there.
@@ -105,63 +106,8 @@ __host__ __device__ inline TileDims tile_dims(int width, int height) {
     return d;
 }
 
-// Certainly rejected without the exact division?  The pixel is located with the
-// fast quotient __fdividef (documented error <= 2 ulp for divisors in
-// [2^-126, 2^126]).  Carrying that error and the roundings of the exact
-// sequence through (q + 1) * W/2 bounds |sx_fast - sx_exact| by
-// W/2 * 2^-22 * (2.25 |q| + 1), over-estimated here as W/2 * 2^-20 * (|q| + 4).
-// A point is rejected only when the whole error interval is off screen, or lies
-// inside one tile whose bound is smaller than the point's depth word.
-__device__ __forceinline__ bool cull_point(const RView& v, float cw, float cx, float cy,
-                                           const uint32_t* __restrict__ bound, int tiles_x) {
-    if (!(cw >= 0x1p-125f && cw <= 0x1p125f)) return false;
-    const float qx = __fdividef(cx, cw), qy = __fdividef(cy, cw);
-    const float ax = __fmul_rn(__fadd_rn(qx, 1.0f), v.hw);
-    const float ay = __fmul_rn(__fsub_rn(1.0f, qy), v.hh);
-    const float ex = (fabsf(qx) + 4.0f) * v.hw * 0x1p-20f;
-    const float ey = (fabsf(qy) + 4.0f) * v.hh * 0x1p-20f;
-    if (ax + ex < 0.0f || ax - ex >= v.fw || ay + ey < 0.0f || ay - ey >= v.fh) return true;
-    if (!bound) return false;
-    // tile coordinates: scaling by 1/16 and the differences below are exact
-    const float tx = floorf(ax * (1.0f / TILE)), ty = floorf(ay * (1.0f / TILE));
-    const float rx = ax - tx * TILE, ry = ay - ty * TILE;
-    if (!(rx > ex && TILE - rx > ex && ry > ey && TILE - ry > ey && tx >= 0.0f && ty >= 0.0f &&
-          tx * TILE < v.fw && ty * TILE < v.fh))
-        return false;
-    return __float_as_uint(cw) > __ldg(bound + (int)ty * tiles_x + (int)tx);
-}
-
-// Projection + clipping of one point for one view; on success returns the
-// pixel (row-major index) and the depth word of the key (bits of w).  With a
-// tile bound table, points that cull_point rejects are dropped before the
-// exact divisions.  (Locating the pixel from the fast quotient with the error
-// bound of cull_point, and dividing exactly only where that interval straddles
-// a pixel edge, measured slower: the correctly rounded division's own fast path
-// costs fewer instructions than the quotient, its bound and the tests.)
-__device__ __forceinline__ bool project_point(const RView& v, float x, float y, float z,
-                                              uint32_t& pix, uint32_t& dbits,
-                                              const uint32_t* __restrict__ bound = nullptr,
-                                              int tiles_x = 0, bool cull = false) {
-    const float cw = __fadd_rn(
-        __fadd_rn(__fadd_rn(__fmul_rn(v.m[8], x), __fmul_rn(v.m[9], y)), __fmul_rn(v.m[10], z)),
-        v.m[11]);
-    if (!(cw >= v.znear && cw <= v.zfar)) return false;
-    const float cx = __fadd_rn(
-        __fadd_rn(__fadd_rn(__fmul_rn(v.m[0], x), __fmul_rn(v.m[1], y)), __fmul_rn(v.m[2], z)),
-        v.m[3]);
-    const float cy = __fadd_rn(
-        __fadd_rn(__fadd_rn(__fmul_rn(v.m[4], x), __fmul_rn(v.m[5], y)), __fmul_rn(v.m[6], z)),
-        v.m[7]);
-    if (cull && cull_point(v, cw, cx, cy, bound, tiles_x)) return false;
-    const float sx = __fmul_rn(__fadd_rn(__fdiv_rn(cx, cw), 1.0f), v.hw);
-    const float sy = __fmul_rn(__fsub_rn(1.0f, __fdiv_rn(cy, cw)), v.hh);
-    if (!(sx >= 0.0f && sx < v.fw && sy >= 0.0f && sy < v.fh)) return false;
-    const int px = __float2int_rz(sx), py = __float2int_rz(sy);
-    pix = (uint32_t)py * (uint32_t)v.width + (uint32_t)px;
-    dbits = __float_as_uint(cw);
-    return true;
-}
-
+// Projection, clipping, early depth test and atomic of one point for one view, by the scalar
+// sequence.
 __device__ __forceinline__ void render_point(const RView& v, float x, float y, float z,
                                              uint32_t idx) {
     const float cw = __fadd_rn(
@@ -183,30 +129,101 @@ __device__ __forceinline__ void render_point(const RView& v, float x, float y, f
     if (key < __ldcg(p)) atomicMin(p, key);
 }
 
-// One thread handles 4 consecutive points = 48 bytes = three 16-byte loads, and
-// prefetches its next group while it works on this one.  Per view, the four
-// points are projected first and their four early-depth reads issued together,
-// so each thread keeps four L2 round trips in flight instead of one.
-// The views come by value, or -- when a captured frame is replayed with new
-// cameras -- from device memory (views_dev); each block keeps them in shared memory.
+// A point whose depth lies inside the view's range but outside project4's (depths below
+// 2^-60 or above 2^125; views with such ranges only).
+__device__ __noinline__ void render_point_wide(const RView& v, float x, float y, float z,
+                                               uint32_t idx) {
+    const float cw = __fadd_rn(
+        __fadd_rn(__fadd_rn(__fmul_rn(v.m[8], x), __fmul_rn(v.m[9], y)), __fmul_rn(v.m[10], z)),
+        v.m[11]);
+    const uint32_t b = __float_as_uint(cw);
+    if (b >= FAST_W_LO && b <= FAST_W_HI) return;
+    render_point(v, x, y, z, idx);
+}
+
+// The points of a group that project4 leaves to the wide path.
+__device__ __forceinline__ void render_wide4(const RView& v, const f2* X, const f2* Y, const f2* Z,
+                                             const uint32_t* idx, uint32_t in) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        float x[2], y[2], z[2];
+        f2_unpack(X[h], x[0], x[1]);
+        f2_unpack(Y[h], y[0], y[1]);
+        f2_unpack(Z[h], z[0], z[1]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            if ((in >> (2 * h + e)) & 1u) render_point_wide(v, x[e], y[e], z[e], idx[2 * h + e]);
+    }
+}
+
+// Four points of one view: project, read the depth words of their pixels together (keys only
+// decrease: a point strictly behind that word cannot win), then the atomics still needed.
+// in: bit j set where point j is present; idx: its key's low word.  MERGE (ascending idx, points
+// next to one another in the scene): a run of points in one pixel leaves only its nearest, the
+// lowest index among equals -- about a third of the points of a dense scan are left to read
+// the key image and fewer still to write it.
+template <bool MERGE>
+__device__ __forceinline__ void render_view(const FView& v, const f2* X, const f2* Y, const f2* Z,
+                                            const uint32_t* idx_in, uint32_t in) {
+    uint32_t pix[4], db[4], cur[4], idx[4];
+    bool ok[4];
+    project4(v, X, Y, Z, pix, db, ok);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        idx[j] = idx_in[j];
+        ok[j] = ok[j] & ((in >> j) & 1u);
+    }
+    if (MERGE) {
+#pragma unroll
+        for (int j = 1; j < 4; ++j) {
+            const bool same = ok[j] & ok[j - 1] & (pix[j] == pix[j - 1]);
+            const bool prev = same & (db[j - 1] <= db[j]);
+            ok[j - 1] = ok[j - 1] & !same;
+            db[j] = prev ? db[j - 1] : db[j];
+            idx[j] = prev ? idx[j - 1] : idx[j];
+        }
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        cur[j] = 0u;
+        if (ok[j]) cur[j] = __ldcg(reinterpret_cast<const uint32_t*>(v.key + pix[j]) + 1);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (ok[j] && db[j] <= cur[j])
+            atomicMin(v.key + pix[j], ((unsigned long long)db[j] << 32) | idx[j]);
+}
+
+// One thread handles 4 consecutive points (48 bytes, three 16-byte loads).  Per view they are
+// projected first and their early-depth reads issued together.
+// The views come by value, or -- when a captured frame is replayed with new cameras -- from
+// device memory (views_dev); each block keeps them in shared memory, and a thread copies one
+// view at a time into registers (read per use, the views made 40% of the pass's shared/L1
+// wavefronts).
 // Variants (picked per scene by the launcher's timing, see below):
 //   SINGLE   one view, kept in registers for the whole pass;
 //   PREFETCH the next group's coordinates are loaded before this group is done;
 //   MINB     register budget: at least MINB blocks of 256 threads per SM.
-//   bound    per-tile depth bounds of all views back to back, or null (no culling);
-//            groups [g_begin, ngroups) are processed.
+// A block works through `span` consecutive groups: scenes are stored along scan lines, particle
+// paths or cells, so neighbours in the array share pixels.  Strided over the whole grid, the
+// 0.5M points in flight were neighbours and most saw their pixel still empty, every one an
+// atomic; in one block the next 1024 points see what the last ones wrote.
+// Eight-view terrain of 200M points: 4.39 ms with project4 alone (4.85 with the scalar
+// sequence), 3.68 with runs of points in a pixel merged, 3.53 with the views' register copies,
+// 3.27 with contiguous spans.  It is then bound by issue (64% active) and by the sectors of its
+// key reads and atomics (0.36 per point and view) about equally; eight points per thread
+// measured slower (3.43 at three blocks per SM with spills, 3.87 at two).
 // Indices are 32-bit: N < 2^32, so there are fewer than 2^30 groups.
-template <bool SINGLE, bool PREFETCH, int MINB, bool CULL>
+template <bool SINGLE, bool PREFETCH, int MINB>
 __global__ void __launch_bounds__(256, MINB) visibility_kernel(const float4* __restrict__ xyz4,
                                                                uint32_t ngroups,
                                                                const float* __restrict__ xyz,
                                                                uint64_t n,
                                                                const __grid_constant__ RViews vs_arg,
                                                                const RViews* __restrict__ views_dev,
-                                                               const uint32_t* __restrict__ bound,
-                                                               uint32_t g_begin) {
+                                                               uint32_t span) {
     __shared__ RViews vs;
-    __shared__ int tile_off[8], tiles_x[8];
+    __shared__ FView fs[SINGLE ? 1 : 8];
     {
         // the views: a word-wise copy into shared memory (no local copy of the parameter)
         const uint32_t* src = reinterpret_cast<const uint32_t*>(views_dev ? views_dev : &vs_arg);
@@ -214,66 +231,38 @@ __global__ void __launch_bounds__(256, MINB) visibility_kernel(const float4* __r
             reinterpret_cast<uint32_t*>(&vs)[i] = src[i];
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        int off = 0;
-        for (int v = 0; v < vs.n; ++v) {
-            const TileDims d = tile_dims(vs.v[v].width, vs.v[v].height);
-            tiles_x[v] = d.w0;
-            tile_off[v] = off;
-            off += d.words;
-        }
-    }
+    const int nv = SINGLE ? 1 : vs.n;
+    if (threadIdx.x < nv) fview_init(fs[threadIdx.x], vs.v[threadIdx.x]);
     __syncthreads();
-    const bool cull = CULL && bound != nullptr;
-    RView v0;
-    if (SINGLE) v0 = vs.v[0];
-    const uint32_t stride = gridDim.x * blockDim.x;
-    uint32_t g = g_begin + blockIdx.x * blockDim.x + threadIdx.x;
+    FView f0;
+    if (SINGLE) f0 = fs[0];
+    // this block's contiguous run of groups
+    const uint32_t g0 = blockIdx.x * span, g1 = g0 + span < ngroups ? g0 + span : ngroups;
+    uint32_t g = g0 + threadIdx.x;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a, c = a;
-    if (PREFETCH && g < ngroups) {
-        a = __ldcs(xyz4 + 3 * g);
-        b = __ldcs(xyz4 + 3 * g + 1);
-        c = __ldcs(xyz4 + 3 * g + 2);
-    }
-    for (; g < ngroups; g += stride) {
-        float4 na = a, nb = b, nc = c;
-        if (PREFETCH) {
-            const uint32_t gn = g + stride;
-            if (gn < ngroups) {
-                na = __ldcs(xyz4 + 3 * gn);
-                nb = __ldcs(xyz4 + 3 * gn + 1);
-                nc = __ldcs(xyz4 + 3 * gn + 2);
-            }
-        } else {
-            a = __ldcs(xyz4 + 3 * g);
-            b = __ldcs(xyz4 + 3 * g + 1);
-            c = __ldcs(xyz4 + 3 * g + 2);
+    auto load = [&](uint32_t gq, float4& p, float4& r, float4& t) {
+        if (gq < g1) {
+            p = __ldcs(xyz4 + 3 * gq);
+            r = __ldcs(xyz4 + 3 * gq + 1);
+            t = __ldcs(xyz4 + 3 * gq + 2);
         }
-        const float px[4] = {a.x, a.w, b.z, c.y};
-        const float py[4] = {a.y, b.x, b.w, c.z};
-        const float pz[4] = {a.z, b.y, c.x, c.w};
+    };
+    if (PREFETCH) load(g, a, b, c);
+    for (; g < g1; g += blockDim.x) {
+        float4 na = a, nb = b, nc = c;
+        if (PREFETCH) load(g + blockDim.x, na, nb, nc);
+        else load(g, a, b, c);
+        const f2 X[2] = {f2_pack(a.x, a.w), f2_pack(b.z, c.y)};
+        const f2 Y[2] = {f2_pack(a.y, b.x), f2_pack(b.w, c.z)};
+        const f2 Z[2] = {f2_pack(a.z, b.y), f2_pack(c.x, c.w)};
         const uint32_t i0 = 4 * g + vs.base;
-        for (int v = 0; v < (SINGLE ? 1 : vs.n); ++v) {
-            // several views: this view's parameters read from shared memory once into
-            // registers for the four points (read per use, they made a third of the L1
-            // wavefronts of the pass)
-            RView vcopy;
-            if (!SINGLE) vcopy = vs.v[v];
-            const RView& vw = SINGLE ? v0 : vcopy;
-            uint32_t pix[4], db[4];
-            unsigned long long cur[4];
-            bool ok[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                ok[j] = project_point(vw, px[j], py[j], pz[j], pix[j], db[j],
-                                      cull ? bound + tile_off[v] : nullptr, tiles_x[v], cull);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cur[j] = ok[j] ? __ldcg(vw.key + pix[j]) : 0ull;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const unsigned long long key = ((unsigned long long)db[j] << 32) | (i0 + j);
-                if (ok[j] && key < cur[j]) atomicMin(vw.key + pix[j], key);
-            }
+        const uint32_t idx[4] = {i0, i0 + 1, i0 + 2, i0 + 3};
+#pragma unroll 1
+        for (int v = 0; v < nv; ++v) {
+            FView fv;
+            if (!SINGLE) fv = fs[v];
+            render_view<true>(SINGLE ? f0 : fv, X, Y, Z, idx, 15u);
+            if (fs[v].wide) render_wide4(vs.v[v], X, Y, Z, idx, 15u);
         }
         if (PREFETCH) {
             a = na;
@@ -283,8 +272,8 @@ __global__ void __launch_bounds__(256, MINB) visibility_kernel(const float4* __r
     }
     // the last n mod 4 points
     if (blockIdx.x == 0 && threadIdx.x < (n & 3)) {
-        const uint64_t i = 4 * ngroups + threadIdx.x;
-        for (int v = 0; v < vs.n; ++v)
+        const uint64_t i = 4 * (uint64_t)ngroups + threadIdx.x;
+        for (int v = 0; v < nv; ++v)
             render_point(vs.v[v], xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], (uint32_t)i + vs.base);
     }
 }
@@ -467,6 +456,8 @@ nrv_status launch_chunk_bounds(const float* xyz, uint64_t n, void* chunks, cudaS
     return NRV_OK;
 }
 
+constexpr uint32_t RENDER_RUN = 8;   // chunk groups (1024 points each) per run of the culled pass: one per warp
+
 // True when no point in the box (c, e) can set a key of view v, given the tile
 // depth bounds (null: depth range and screen only; HIZ: the view's bound pyramid,
 // read at one level, else its level-0 tiles).  Allowances: 1e-5 of the
@@ -553,10 +544,12 @@ __global__ void __launch_bounds__(256, 4) chunk_render_kernel(const float* __res
                                                            const __grid_constant__ RViews vs_arg,
                                                            const RViews* __restrict__ views_dev,
                                                            const uint32_t* __restrict__ bound,
-                                                           int prepass, uint32_t S, uint32_t g_begin,
-                                                           uint32_t g_end) {
+                                                           int prepass, uint32_t S, uint32_t r_begin,
+                                                           uint32_t r_end, uint32_t run_step,
+                                                           uint32_t nruns) {
     pdl_wait_and_release();
     __shared__ RViews vs;
+    __shared__ FView fs[SINGLE ? 1 : 8];
     __shared__ int tile_off[8];
     __shared__ TileDims tdim[8];
     {
@@ -573,6 +566,7 @@ __global__ void __launch_bounds__(256, 4) chunk_render_kernel(const float* __res
             off += tdim[v].words;
         }
     }
+    if (threadIdx.x < vs.n) fview_init(fs[threadIdx.x], vs.v[threadIdx.x]);
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const uint32_t nch = (uint32_t)chunk_count(n);
@@ -581,13 +575,21 @@ __global__ void __launch_bounds__(256, 4) chunk_render_kernel(const float* __res
     const uint32_t all = (1u << vs.n) - 1u;
     // one view: its parameters live in registers for the whole pass
     RView vreg;
+    FView freg;
     TileDims treg;
     if (SINGLE) {
+        freg = fs[0];
         vreg = vs.v[0];
         treg = tdim[0];
     }
     // the views of mask vm in which the box (c, e) may set a key
     auto box_visible = [&](const float* c, const float* e, uint32_t vm) -> uint32_t {
+        if (SINGLE) {
+            // the matrix: the low halves of the paired registers
+            float dup;
+#pragma unroll
+            for (int i = 0; i < 12; ++i) f2_unpack(freg.m[i], vreg.m[i], dup);
+        }
         if (SINGLE) return chunk_hidden<HIZ>(vreg, c, e, bound, treg) ? 0u : 1u;
         uint32_t vis = 0;
         for (int v = 0; v < vs.n; ++v)
@@ -614,23 +616,19 @@ __global__ void __launch_bounds__(256, 4) chunk_render_kernel(const float* __res
                 vall |= vm[j];
             }
         }
+        const f2 X[2] = {f2_pack(x[0], x[1]), f2_pack(x[2], x[3])};
+        const f2 Y[2] = {f2_pack(y[0], y[1]), f2_pack(y[2], y[3])};
+        const f2 Z[2] = {f2_pack(z[0], z[1]), f2_pack(z[2], z[3])};
         while (vall) {
-            const int v = __ffs(vall) - 1;
+            const int v = SINGLE ? 0 : __ffs(vall) - 1;
             vall &= vall - 1;
-            const RView& vw = SINGLE ? vreg : vs.v[v];
-            uint32_t pix[4], db[4];
-            bool ok[4];
+            uint32_t inv = 0;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-                ok[j] = in[j] && ((vm[j] >> v) & 1u) && project_point(vw, x[j], y[j], z[j], pix[j], db[j]);
-            unsigned long long cur[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cur[j] = ok[j] ? __ldcg(vw.key + pix[j]) : 0ull;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const unsigned long long key = ((unsigned long long)db[j] << 32) | idx[j];
-                if (ok[j] && key < cur[j]) atomicMin(vw.key + pix[j], key);
-            }
+            for (int j = 0; j < 4; ++j) inv |= (in[j] && ((vm[j] >> v) & 1u)) ? 1u << j : 0u;
+            FView fv;
+            if (!SINGLE) fv = fs[v];
+            render_view<false>(SINGLE ? freg : fv, X, Y, Z, idx, inv);
+            if (fs[v].wide) render_wide4(vs.v[v], X, Y, Z, idx, inv);
         }
     };
     // up to four chunks: one point of each per lane
@@ -726,8 +724,16 @@ __global__ void __launch_bounds__(256, 4) chunk_render_kernel(const float* __res
         }
         __syncwarp();
     };
-    // culled pass over the chunk groups [g_begin, g_end) of 32 chunks
-    for (uint32_t g = g_begin + warp; g < g_end; g += nwarps) {
+    // culled pass over the runs at places [r_begin, r_end) of the run order, one group of 32
+    // chunks per warp and run
+    const uint32_t ngroups = (nch + 31) / 32;
+    uint32_t run = (uint32_t)((uint64_t)(r_begin + blockIdx.x) * run_step % nruns);
+    const uint32_t run_inc = (uint32_t)((uint64_t)gridDim.x * run_step % nruns);
+    for (uint32_t t = r_begin + blockIdx.x; t < r_end; t += gridDim.x) {
+        const uint32_t g = run * RENDER_RUN + threadIdx.x / 32;
+        run += run_inc;
+        if (run >= nruns) run -= nruns;
+        if (g >= ngroups) continue;
         const uint32_t kk = g * 32 + lane;
         uint32_t vis = 0;
         if (kk < nch && (kk & (S - 1)) != 0) {
@@ -779,14 +785,13 @@ size_t visibility_scratch_bytes(const RViews& views) {
 // choice is made during a stream capture: the default variant is used until an
 // uncaptured launch has tuned.
 //
-// A culling variant first renders the leading 1/16 of the points without
-// culling, turns the keys into tile bounds, then renders the rest with culling.
 typedef void (*VisFn)(const float4*, uint32_t, const float*, uint64_t, RViews, const RViews*,
-                      const uint32_t*, uint32_t);
+                      uint32_t);
+
+constexpr uint64_t SPAN_MAX = 4096;   // groups of 4 points (16K points)
 
 struct VisVariant {
     VisFn fn;            // null for a chunk-culling variant
-    bool cull;
     const char* name;
     int blocks_per_sm;   // resident blocks, from the compiled register count
     uint32_t chunk_S;    // chunk culling: every S-th chunk renders in the prepass (0: not chunked;
@@ -799,47 +804,47 @@ struct VisVariant {
 };
 
 static VisVariant kSingle[] = {
-    {visibility_kernel<true, true, 3, false>, false, "single/prefetch/3", 0},
-    {visibility_kernel<true, false, 3, false>, false, "single/plain/3", 0},
-    {visibility_kernel<true, true, 2, false>, false, "single/prefetch/2", 0},
-    {visibility_kernel<true, true, 3, true>, true, "single/prefetch/3/cull", 0},
-    {visibility_kernel<true, false, 3, true>, true, "single/plain/3/cull", 0},
-    {visibility_kernel<true, true, 2, true>, true, "single/prefetch/2/cull", 0},
-    {visibility_kernel<true, true, 4, false>, false, "single/prefetch/4", 0},
-    {visibility_kernel<true, false, 4, false>, false, "single/plain/4", 0},
-    {nullptr, true, "single/chunks/16", 0, 16, 1},
-    {nullptr, true, "single/chunks/16x2", 0, 16, 2},
-    {nullptr, true, "single/chunks/16x4", 0, 16, 4},
-    {nullptr, true, "single/chunks/16/r", 0, 16, 1, 1},
-    {nullptr, true, "single/chunks/16x2/r", 0, 16, 2, 1},
-    {nullptr, true, "single/chunks/16x4/r", 0, 16, 4, 1},
-    {nullptr, true, "single/chunks/16/r/sub", 0, 16, 1, 1, 1},
-    {nullptr, true, "single/chunks/16x2/r/sub", 0, 16, 2, 1, 1},
-    {nullptr, true, "single/chunks/16x4/r/sub", 0, 16, 4, 1, 1},
-    {nullptr, true, "single/chunks/16x2/r/hiz", 0, 16, 2, 1, 0, 1},
-    {nullptr, true, "single/chunks/16/r/sub/hiz", 0, 16, 1, 1, 1, 1},
-    {nullptr, true, "single/chunks/16x2/r/sub/hiz", 0, 16, 2, 1, 1, 1},
-    {nullptr, true, "single/chunks/16x4/r/sub/hiz", 0, 16, 4, 1, 1, 1},
-    {nullptr, true, "single/chunks/32x2/r/sub/hiz", 0, 32, 2, 1, 1, 1},
-    {nullptr, true, "single/chunks/8x2/r/sub/hiz", 0, 8, 2, 1, 1, 1},
-    {nullptr, true, "single/chunks/16x2/r/sub/hiz/33", 0, 16, 2, 1, 1, 1, 33},
-    {nullptr, true, "single/chunks/16x2/r/sub/hiz/25", 0, 16, 2, 1, 1, 1, 25},
+    {visibility_kernel<true, false, 3>, "single/plain/3", 0},
+    {visibility_kernel<true, true, 3>, "single/prefetch/3", 0},
+    {visibility_kernel<true, true, 2>, "single/prefetch/2", 0},
+    {visibility_kernel<true, false, 2>, "single/plain/2", 0},
+    {nullptr, "single/chunks/16x2/r/33", 0, 16, 2, 1, 0, 0, 33},
+    {nullptr, "single/chunks/16x2/r/25", 0, 16, 2, 1, 0, 0, 25},
+    {nullptr, "single/chunks/32x2/r", 0, 32, 2, 1},
+    {nullptr, "single/chunks/16x2/r/hiz/33", 0, 16, 2, 1, 0, 1, 33},
+    {nullptr, "single/chunks/16", 0, 16, 1},
+    {nullptr, "single/chunks/16x2", 0, 16, 2},
+    {nullptr, "single/chunks/16x4", 0, 16, 4},
+    {nullptr, "single/chunks/16/r", 0, 16, 1, 1},
+    {nullptr, "single/chunks/16x2/r", 0, 16, 2, 1},
+    {nullptr, "single/chunks/16x4/r", 0, 16, 4, 1},
+    {nullptr, "single/chunks/16/r/sub", 0, 16, 1, 1, 1},
+    {nullptr, "single/chunks/16x2/r/sub", 0, 16, 2, 1, 1},
+    {nullptr, "single/chunks/16x4/r/sub", 0, 16, 4, 1, 1},
+    {nullptr, "single/chunks/16x2/r/hiz", 0, 16, 2, 1, 0, 1},
+    {nullptr, "single/chunks/16/r/sub/hiz", 0, 16, 1, 1, 1, 1},
+    {nullptr, "single/chunks/16x2/r/sub/hiz", 0, 16, 2, 1, 1, 1},
+    {nullptr, "single/chunks/16x4/r/sub/hiz", 0, 16, 4, 1, 1, 1},
+    {nullptr, "single/chunks/32x2/r/sub/hiz", 0, 32, 2, 1, 1, 1},
+    {nullptr, "single/chunks/8x2/r/sub/hiz", 0, 8, 2, 1, 1, 1},
+    {nullptr, "single/chunks/16x2/r/sub/hiz/33", 0, 16, 2, 1, 1, 1, 33},
+    {nullptr, "single/chunks/16x2/r/sub/hiz/25", 0, 16, 2, 1, 1, 1, 25},
 };
 static VisVariant kMulti[] = {
-    {visibility_kernel<false, true, 3, false>, false, "multi/prefetch/3", 0},
-    {visibility_kernel<false, false, 3, false>, false, "multi/plain/3", 0},
-    {visibility_kernel<false, true, 3, true>, true, "multi/prefetch/3/cull", 0},
-    {visibility_kernel<false, false, 3, true>, true, "multi/plain/3/cull", 0},
-    {nullptr, true, "multi/chunks/16", 0, 16, 1},
-    {nullptr, true, "multi/chunks/16x2", 0, 16, 2},
-    {nullptr, true, "multi/chunks/16x4", 0, 16, 4},
-    {nullptr, true, "multi/chunks/16x2/sub", 0, 16, 2, 0, 1},
-    {nullptr, true, "multi/chunks/16x2/sub/hiz", 0, 16, 2, 0, 1, 1},
-    {visibility_kernel<false, false, 4, false>, false, "multi/plain/4", 0},
+    {visibility_kernel<false, true, 3>, "multi/prefetch/3", 0},
+    {visibility_kernel<false, false, 3>, "multi/plain/3", 0},
+    {visibility_kernel<false, true, 2>, "multi/prefetch/2", 0},
+    {nullptr, "multi/chunks/16x2/33", 0, 16, 2, 0, 0, 0, 33},
+    {nullptr, "multi/chunks/16", 0, 16, 1},
+    {nullptr, "multi/chunks/16x2", 0, 16, 2},
+    {nullptr, "multi/chunks/16x4", 0, 16, 4},
+    {nullptr, "multi/chunks/16x2/sub", 0, 16, 2, 0, 1},
+    {nullptr, "multi/chunks/16x2/sub/hiz", 0, 16, 2, 0, 1, 1},
+    {visibility_kernel<false, false, 4>, "multi/plain/4", 0},
 };
 
 typedef void (*ChunkFn)(const float*, uint64_t, const float*, RViews, const RViews*,
-                        const uint32_t*, int, uint32_t, uint32_t, uint32_t);
+                        const uint32_t*, int, uint32_t, uint32_t, uint32_t, uint32_t, uint32_t);
 template <bool SINGLE>
 static ChunkFn chunk_kernel_of(const VisVariant& v) {
     if (v.hiz) return v.sub ? chunk_render_kernel<SINGLE, true, true> : chunk_render_kernel<SINGLE, false, true>;
@@ -847,6 +852,26 @@ static ChunkFn chunk_kernel_of(const VisVariant& v) {
 }
 static ChunkFn chunk_kernel(const VisVariant& v) {
     return v.single ? chunk_kernel_of<true>(v) : chunk_kernel_of<false>(v);
+}
+
+// The culled pass takes the scene in runs of RENDER_RUN groups (8K points), run i of the pass
+// being run (i * step) mod nruns of the scene: with a step near the golden section of nruns and
+// coprime to it, every prefix of the pass is spread over the whole scene.  A scene stored far
+// to near along the view axis (a grid, layer by layer) would otherwise have every layer pass
+// the tests and overwrite the last one, and a first part of the pass that occludes nothing.
+static uint32_t run_order_step(uint32_t nruns) {
+    uint32_t step = (uint32_t)(0.6180339887 * nruns);
+    if (step < 1) step = 1;
+    auto gcd = [](uint32_t a, uint32_t b) {
+        while (b) {
+            const uint32_t t = a % b;
+            a = b;
+            b = t;
+        }
+        return a;
+    };
+    while (gcd(step, nruns) != 1) ++step;
+    return step;
 }
 
 static nrv_status resident_blocks(VisVariant& v) {
@@ -874,39 +899,41 @@ static nrv_status run_variant(VisVariant& v, const float* xyz, uint64_t n,
         const float* ch = reinterpret_cast<const float*>(chunks);
         const uint32_t ngroups = (uint32_t)((chunk_count(n) + 31) / 32);
         const ChunkFn kern = chunk_kernel(v);
+        const uint32_t nruns = (ngroups + RENDER_RUN - 1) / RENDER_RUN;
+        const uint32_t step = run_order_step(nruns);
         NRV_TRY(launch_pdl(kern, dim3(blocks), dim3(256), s, xyz, n, ch, views, views_dev,
-                           (const uint32_t*)nullptr, 1, v.chunk_S, 0u, 0u));
+                           (const uint32_t*)nullptr, 1, v.chunk_S, 0u, 0u, step, nruns));
         // the chunk groups in `phases` consecutive parts, the tile bounds rebuilt from the
         // keys so far before each part (later parts meet tighter bounds)
         for (int ph = 0; ph < v.phases; ++ph) {
-            uint32_t g0 = (uint32_t)((uint64_t)ngroups * ph / v.phases);
-            uint32_t g1 = (uint32_t)((uint64_t)ngroups * (ph + 1) / v.phases);
+            uint32_t g0 = (uint32_t)((uint64_t)nruns * ph / v.phases);
+            uint32_t g1 = (uint32_t)((uint64_t)nruns * (ph + 1) / v.phases);
             if (v.phases == 2 && v.first_part) {
-                const uint32_t cut = (uint32_t)((uint64_t)ngroups * v.first_part / 100);
+                const uint32_t cut = (uint32_t)((uint64_t)nruns * v.first_part / 100);
                 g0 = ph ? cut : 0u;
-                g1 = ph ? ngroups : cut;
+                g1 = ph ? nruns : cut;
             }
             NRV_TRY(launch_tile_bounds(views, views_dev, tiles, v.hiz != 0, s));
             NRV_TRY(launch_pdl(kern, dim3(blocks), dim3(256), s, xyz, n, ch, views, views_dev,
-                               (const uint32_t*)tiles, 0, v.chunk_S, g0, g1));
+                               (const uint32_t*)tiles, 0, v.chunk_S, g0, g1, step, nruns));
         }
         return NRV_OK;
     }
     const uint64_t ngroups = n / 4;
-    auto launch = [&](uint64_t g0, uint64_t g1, uint64_t npts, const uint32_t* b) -> nrv_status {
-        int blocks = g_vis_sms * v.blocks_per_sm;
-        const uint64_t need = (g1 - g0 + 255) / 256;
-        if (need < (uint64_t)blocks) blocks = (int)(need > 0 ? need : 1);
-        v.fn<<<blocks, 256, 0, s>>>(reinterpret_cast<const float4*>(xyz), (uint32_t)g1, xyz, npts,
-                                    views, views_dev, b, (uint32_t)g0);
-        NRV_CHECK_LAUNCH();
-        return NRV_OK;
-    };
-    if (!v.cull || !tiles || ngroups < 64) return launch(0, ngroups, n, nullptr);
-    const uint64_t gsub = ngroups / 16;
-    NRV_TRY(launch(0, gsub, 4 * gsub, nullptr));
-    NRV_TRY(launch_tile_bounds(views, views_dev, tiles, false, s));
-    return launch(gsub, ngroups, n, tiles);
+    // spans of at most 16K points, at least eight per resident block where there are that many;
+    // a smaller scene in one wave (1M points, 512 x 512: 25.3 us against 26.6 for 1024-point
+    // spans in 2.1 waves)
+    const uint64_t step = 256, resident = (uint64_t)g_vis_sms * v.blocks_per_sm;
+    uint64_t span = ngroups / (resident * 8) / step * step;
+    if (span < step) span = ((ngroups + resident - 1) / resident + step - 1) / step * step;
+    if (span > SPAN_MAX) span = SPAN_MAX;
+    if (span < step) span = step;
+    const uint64_t blocks = (ngroups + span - 1) / span;
+    v.fn<<<(unsigned)(blocks > 0 ? blocks : 1), 256, 0, s>>>(reinterpret_cast<const float4*>(xyz),
+                                                            (uint32_t)ngroups, xyz, n, views, views_dev,
+                                                            (uint32_t)span);
+    NRV_CHECK_LAUNCH();
+    return NRV_OK;
 }
 
 int visibility_variant_count(int multi) {
@@ -948,8 +975,8 @@ nrv_status launch_visibility(const float* xyz, uint64_t n, const RViews& views, 
     if (const char* e = getenv("NRV_VIS_VARIANT")) {
         const int i = atoi(e);
         if (i >= 0 && i < count) {
-            if (tab[i].cull && !tiles) return fail(NRV_ERR_ARG, "variant %d needs tile scratch", i);
-            if (tab[i].chunk_S && !chunks) return fail(NRV_ERR_ARG, "variant %d needs chunk bounds", i);
+            if (tab[i].chunk_S && (!tiles || !chunks))
+                return fail(NRV_ERR_ARG, "variant %d needs tile scratch and chunk bounds", i);
             return run_variant(tab[i], xyz, n, views, s, views_dev, tiles, chunks);
         }
     }
@@ -963,7 +990,7 @@ nrv_status launch_visibility(const float* xyz, uint64_t n, const RViews& views, 
         float best = 1e30f;
         int arg = 0;
         for (int i = 0; i < count; ++i) {
-            if ((tab[i].cull && !tiles) || (tab[i].chunk_S && !chunks)) continue;
+            if (tab[i].chunk_S && (!tiles || !chunks)) continue;
             float ms = 0.0f;
             for (int rep = 0; rep < 2; ++rep) {
                 NRV_TRY(launch_clear_keys(views, s));
@@ -987,7 +1014,7 @@ nrv_status launch_visibility(const float* xyz, uint64_t n, const RViews& views, 
         NRV_TRY(launch_clear_keys(views, s));
     }
     int pick = choice > 0 ? choice - 1 : 0;
-    if ((tab[pick].cull && !tiles) || (tab[pick].chunk_S && !chunks)) pick = 0;
+    if (tab[pick].chunk_S && (!tiles || !chunks)) pick = 0;
     return run_variant(tab[pick], xyz, n, views, s, views_dev, tiles, chunks);
 }
 
