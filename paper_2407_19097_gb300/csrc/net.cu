@@ -2,6 +2,7 @@
 // re-packing, activation workspace and the forward pass.
 #include <string.h>
 
+#include "f32.h"
 #include "net.h"
 #include "net_simt.cuh"
 
@@ -60,7 +61,7 @@ static inline int padded_cin(const Net* net, int l) {
 // ------------------------------------------------------------------ weight re-packing
 // conv forward   wf[tap][c][o]  = W[o][c][tap]      (c < padded cin, zero beyond cin)
 // conv backward  wt[tap][o][c]  = W[o][c][8 - tap]  (180-degree rotation, transposed)
-// upconv         wf[a][b][c][o] = W[c][o][a][b]
+// upconv         wf[a][b][c][o] = wt[a][b][o][c] = W[c][o][a][b]
 // All layers in one launch: element i belongs to the layer whose range holds it.
 struct RepackJobs {
     int n;
@@ -92,6 +93,7 @@ __global__ void repack_f32_kernel(const float* __restrict__ P, const __grid_cons
             wt[it] = c < L.cin ? P[L.woff + ((size_t)o * L.cin + c) * 9 + (8 - tap)] : 0.0f;
         } else {
             wf[i] = P[L.woff + ((size_t)c * L.cout + o) * 4 + tap];
+            wt[((size_t)tap * L.cout + o) * cinp + c] = wf[i];
         }
     }
 }
@@ -172,10 +174,15 @@ static nrv_status simt_conv3(const Net* net, int l, TView<const T> x1, int c1, T
                              int c2, TView<T> y, const Geo& g, int level, bool relu,
                              cudaStream_t s) {
     const Layer& L = net->layers[l];
+    const float* wf = (const float*)net->wf32.p + net->wf_off[l];
+    const float* bias = (const float*)net->params.p + L.boff;
+    if constexpr (sizeof(T) == 4)
+        return f32_conv3(x1.p, c1, x2.p, c2, wf, bias, relu ? 1 : 0, nullptr, y.p, L.cout, g.n, g.h[level],
+                         g.w[level], s);
     Conv3Args<T> a;
     a.x1 = x1; a.x2 = x2; a.c1 = c1; a.c2 = c2;
-    a.w = (const float*)net->wf32.p + net->wf_off[l];
-    a.bias = (const float*)net->params.p + L.boff;
+    a.w = wf;
+    a.bias = bias;
     a.y = y;
     a.cout = L.cout;
     a.n = g.n; a.h = g.h[level]; a.w_ = g.w[level];
@@ -193,6 +200,9 @@ template <typename T>
 static nrv_status simt_upconv(const Net* net, int l, TView<const T> x, TView<T> y, int n, int hi,
                               int wi, cudaStream_t s) {
     const Layer& L = net->layers[l];
+    if constexpr (sizeof(T) == 4)
+        return f32_upconv(x.p, L.cin, (const float*)net->wf32.p + net->wf_off[l],
+                          (const float*)net->params.p + L.boff, y.p, L.cout, n, hi, wi, s);
     const size_t npx = (size_t)n * hi * wi * 4;
     dim3 grid((unsigned)((npx + 127) / 128), L.cout / 16);
     upconv2_kernel<T><<<grid, 128, (size_t)4 * L.cin * 16 * 4, s>>>(
@@ -294,8 +304,6 @@ static bool g_attr_set = false;
 
 static nrv_status set_kernel_attrs() {
     if (g_attr_set) return NRV_OK;
-    NRV_CHECK_CUDA(cudaFuncSetAttribute(conv3_simt_kernel<float>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 9 * 128 * 16 * 4));
     NRV_CHECK_CUDA(cudaFuncSetAttribute(conv3_simt_kernel<__nv_bfloat16>,
                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 9 * 128 * 16 * 4));
     g_attr_set = true;

@@ -4,6 +4,7 @@
 // Gradients of the weights are reductions over all pixels.  They are computed
 // in fixed pixel chunks whose partial sums are added in a fixed order by a
 // second kernel, so a step is bit-for-bit reproducible.
+#include "f32.h"
 #include "net.h"
 #include "net_simt.cuh"
 
@@ -549,6 +550,10 @@ struct Bwd {
                 clear_error();
             }
         }
+        if constexpr (sizeof(T) == 4)
+            return f32_conv3(gpre.p, net->layers[l].cout, nullptr, 0,
+                             (const float*)net->wtf32.p + net->wf_off[l], nullptr, 0, mask.p, out.p,
+                             net->layers[l].cin, g.n, g.h[level], g.w[level], s);
         // this translation unit has its own instance of the kernel template
         static bool attr = false;
         if (!attr) {
@@ -637,6 +642,10 @@ struct Bwd {
             if (st != NRV_ERR_UNSUPPORTED) return st;
             clear_error();
         }
+        if constexpr (sizeof(T) == 4)
+            return f32_upconv_dgrad(gout.p + gout.coff, gout.ld, L.cout,
+                                    (const float*)net->wtf32.p + net->wf_off[l], xm.p, gx.p, L.cin, g.n,
+                                    g.h[level_in], g.w[level_in], s);
         dim3 grid((unsigned)((npx + 127) / 128), L.cin / 16);
         upconv2_dgrad_kernel<T><<<grid, 128, (size_t)4 * 16 * L.cout * 4, s>>>(
             gout, L.cout, (const float*)net->wf32.p + net->wf_off[l], L.cin, xm, gx, g.n,
