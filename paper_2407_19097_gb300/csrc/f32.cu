@@ -295,7 +295,326 @@ nrv_status launch_mode(F32Args& a, cudaStream_t s) {
     return a.ncols % 32 == 0 ? launch_width<MODE, 32>(a, s) : launch_width<MODE, 16>(a, s);
 }
 
+// ------------------------------------------------------------------ weight gradients
+// dW[(tap, c)][o] = sum over pixels of x[p + tap][c] g[p][o]: a block takes 16 input channels
+// x 16 output channels x 9 taps over a contiguous run of 32 x 8 pixel tiles.  Thread (slice,
+// dy, channel pair) walks one row of the tile with 3 dx x 2 c x 16 o sums: a window of three
+// pixels slides along the row, so each step reads one new channel pair and 16 gradients for 48
+// paired FMAs (the first form read 2 quads for 16).  The eight slices are added in order.
+constexpr int WT = 192;              // 8 slices x 3 kernel rows x 8 channel pairs
+constexpr int WTW = 32, WTH = 8;     // tile
+constexpr int WXRS = (WTW + 2) * 64 + 64;   // 64 bytes off per row in the banks
+constexpr int WX_BYTES = (WTH + 2) * WXRS, WG_BYTES = WTH * WTW * 64;
+constexpr int WSTAGE = WX_BYTES + WG_BYTES;
+constexpr int WRED = WT * 96 * 4;
+constexpr int WSMEM = 2 * WSTAGE > WRED ? 2 * WSTAGE : WRED;
+
+struct F32Wgrad {
+    const float* g;
+    const float *x1, *x2;
+    int c1, c2, cout;
+    int n, h, w, tiles_x, tiles_y, ntiles, tiles_per_block;
+    float *part, *partb;
+};
+
+__global__ void __launch_bounds__(WT, 2) wgrad_f32_kernel(const __grid_constant__ F32Wgrad a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ float bred[12][16];
+    const uint32_t s0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+    const int t = threadIdx.x, slice = t / 24, u = t % 24, dy = u / 8, cp = u % 8;
+    const int og = blockIdx.y * 16, cg = blockIdx.z * 16, cin = a.c1 + a.c2;
+    const float* src = cg < a.c1 ? a.x1 + cg : a.x2 + (cg - a.c1);
+    const int ld = cg < a.c1 ? a.c1 : a.c2;
+    const int nc = cin - cg < 16 ? cin - cg : 16;      // real channels of the group
+    const int t0 = blockIdx.x * a.tiles_per_block;
+    const int t1 = t0 + a.tiles_per_block < a.ntiles ? t0 + a.tiles_per_block : a.ntiles;
+
+    auto load = [&](int tile, int buf) {
+        const int tx = tile % a.tiles_x, ty = (tile / a.tiles_x) % a.tiles_y, img = tile / (a.tiles_x * a.tiles_y);
+        const int x0 = tx * WTW, y0 = ty * WTH;
+        const uint32_t xb = s0 + buf * WSTAGE, gb = xb + WX_BYTES;
+        for (int i = t; i < (WTH + 2) * (WTW + 2) * 4; i += WT) {
+            const int q = i & 3, pp = i >> 2, r = pp / (WTW + 2), p = pp - r * (WTW + 2);
+            const int y = y0 + r - 1, x = x0 + p - 1;
+            const bool ok = (unsigned)y < (unsigned)a.h && (unsigned)x < (unsigned)a.w && 4 * q < nc;
+            const float* sp = src;
+            if (ok) sp += (((size_t)img * a.h + y) * a.w + x) * ld + 4 * q;
+            cp16(xb + r * WXRS + p * 64 + q * 16, sp, ok);
+        }
+        for (int i = t; i < WTH * WTW * 4; i += WT) {
+            const int q = i & 3, pp = i >> 2, r = pp / WTW, p = pp - r * WTW;
+            const int y = y0 + r, x = x0 + p;
+            const bool ok = y < a.h && x < a.w;
+            const float* sp = a.g;
+            if (ok) sp += (((size_t)img * a.h + y) * a.w + x) * a.cout + og + 4 * q;
+            cp16(gb + pp * 64 + q * 16, sp, ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    f2 acc[3][2][8];
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) acc[i][j][k] = 0ull;
+    float bsum = 0.0f;
+    if (t0 < t1) load(t0, 0);
+    for (int tile = t0; tile < t1; ++tile) {
+        const int buf = (tile - t0) & 1;
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (tile + 1 < t1) load(tile + 1, buf ^ 1);
+        const uint8_t* xs = smem + buf * WSTAGE + (slice + dy) * WXRS + cp * 8;
+        const uint8_t* gs = smem + buf * WSTAGE + WX_BYTES;
+        const uint8_t* gr = gs + slice * WTW * 64;
+        f2 win[3][2];
+        auto take = [&](int p, f2* d) {
+            const float2 v = *reinterpret_cast<const float2*>(xs + p * 64);
+            d[0] = f2_pack(v.x, v.x);
+            d[1] = f2_pack(v.y, v.y);
+        };
+        take(0, win[0]);
+        take(1, win[1]);
+#pragma unroll 2
+        for (int p = 0; p < WTW; ++p) {
+            take(p + 2, win[2]);
+            const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(gr + p * 64);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const ulonglong2 gv = gp[k];
+#pragma unroll
+                for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+                    for (int c = 0; c < 2; ++c) {
+                        acc[dx][c][2 * k] = f2_fma(win[dx][c], gv.x, acc[dx][c][2 * k]);
+                        acc[dx][c][2 * k + 1] = f2_fma(win[dx][c], gv.y, acc[dx][c][2 * k + 1]);
+                    }
+            }
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                win[0][c] = win[1][c];
+                win[1][c] = win[2][c];
+            }
+        }
+        if (blockIdx.z == 0)
+            for (int p = t >> 4; p < WTH * WTW; p += WT / 16)
+                bsum += *reinterpret_cast<const float*>(gs + p * 64 + (t & 15) * 4);
+    }
+    __syncthreads();
+    float* red = reinterpret_cast<float*>(smem);   // [slice][u][96]
+#pragma unroll
+    for (int dx = 0; dx < 3; ++dx)
+#pragma unroll
+        for (int c = 0; c < 2; ++c)
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                reinterpret_cast<f2*>(red)[(size_t)t * 48 + (dx * 2 + c) * 8 + k] = acc[dx][c][k];
+    bred[t >> 4][t & 15] = bsum;
+    __syncthreads();
+    for (int i = t; i < 16 * 144; i += WT) {
+        const int c = i & 15, tap = (i >> 4) % 9, o = i / 144;
+        if (c >= nc) continue;
+        const int at = ((tap / 3) * 8 + c / 2) * 96 + ((tap % 3) * 2 + (c & 1)) * 16 + o;
+        float v = red[at];
+#pragma unroll
+        for (int sl = 1; sl < 8; ++sl) v += red[sl * 24 * 96 + at];
+        a.part[((size_t)blockIdx.x * a.cout + og + o) * 9 * cin + tap * cin + cg + c] = v;
+    }
+    if (blockIdx.z == 0 && t < 16) {
+        float v = bred[0][t];
+        for (int k = 1; k < 12; ++k) v += bred[k][t];
+        a.partb[(size_t)blockIdx.x * a.cout + og + t] = v;
+    }
+}
+
+// Transposed conv: dW[c][(ab, o)] = sum over input pixels of x[p][c] g[out(p, ab)][o]: a block
+// takes 32 c x 64 (ab, o) over a contiguous run of pixels, 64 per stage; a thread 8 x 8 sums,
+// the eight warps every eighth pixel each, added in order at the end.
+constexpr int UPX = 64;
+constexpr int USTAGE = UPX * (32 + 64) * 4;
+constexpr int URED = NT * 64 * 4;
+constexpr int USMEM = 2 * USTAGE > URED ? 2 * USTAGE : URED;
+
+struct F32WgradUp {
+    const float *x, *g;
+    int cin, cout, ldg;
+    int n, h, w;             // input level
+    long long npx, px_per_block;
+    float *part, *partb;
+};
+
+__global__ void __launch_bounds__(NT, 2) wgrad_up_f32_kernel(const __grid_constant__ F32WgradUp a) {
+    extern __shared__ __align__(128) uint8_t smem[];
+    __shared__ float bred[4][64];
+    const uint32_t s0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
+    const int t = threadIdx.x, warp = t >> 5, lane = t & 31, cq = lane & 3, nq = lane >> 2;
+    const int cg = blockIdx.y * 32, ng = blockIdx.z * 64, K = 4 * a.cout;
+    const long long q0 = blockIdx.x * a.px_per_block;
+    const long long q1 = q0 + a.px_per_block < a.npx ? q0 + a.px_per_block : a.npx;
+
+    auto load = [&](long long qb, int buf) {
+        const uint32_t xb = s0 + buf * USTAGE, gb = xb + UPX * 128;
+        for (int i = t; i < UPX * 8; i += NT) {
+            const int q = i & 7, p = i >> 3;
+            const bool ok = qb + p < q1;
+            cp16(xb + i * 16, ok ? a.x + (size_t)(qb + p) * a.cin + cg + 4 * q : a.x, ok);
+        }
+        for (int i = t; i < UPX * 16; i += NT) {
+            const int q = i & 15, p = i >> 4, col = ng + 4 * q, ab = col / a.cout, o = col - ab * a.cout;
+            const long long px = qb + p;
+            const bool ok = px < q1;
+            const float* sp = a.g;
+            if (ok) {
+                const int X = (int)(px % a.w), r = (int)(px / a.w), Y = r % a.h, img = r / a.h;
+                sp += (((size_t)img * 2 * a.h + 2 * Y + (ab >> 1)) * (2 * (size_t)a.w) + 2 * X + (ab & 1)) * a.ldg + o;
+            }
+            cp16(gb + i * 16, sp, ok);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+
+    f2 acc[4][8];   // channel pairs x columns
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = 0ull;
+    float bsum = 0.0f;
+    if (q0 < q1) load(q0, 0);
+    int buf = 0;
+    for (long long qb = q0; qb < q1; qb += UPX, buf ^= 1) {
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        if (qb + UPX < q1) load(qb + UPX, buf ^ 1);
+        const uint8_t* xs = smem + buf * USTAGE;
+        const uint8_t* gs = xs + UPX * 128;
+#pragma unroll 2
+        for (int p = warp; p < UPX; p += NT / 32) {
+            const ulonglong2* xp = reinterpret_cast<const ulonglong2*>(xs + p * 128 + cq * 32);
+            const ulonglong2 xa = xp[0], xb = xp[1];
+            const f2 xv[4] = {xa.x, xa.y, xb.x, xb.y};
+            const float4* gp = reinterpret_cast<const float4*>(gs + p * 256 + nq * 32);
+            const float4 g0 = gp[0], g1 = gp[1];
+            const float gv[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const f2 gd = f2_pack(gv[j], gv[j]);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) acc[i][j] = f2_fma(xv[i], gd, acc[i][j]);
+            }
+        }
+        if (blockIdx.y == 0)
+            for (int p = t >> 6; p < UPX; p += 4) bsum += *reinterpret_cast<const float*>(gs + p * 256 + (t & 63) * 4);
+    }
+    __syncthreads();
+    float* red = reinterpret_cast<float*>(smem);   // [warp][lane][channel 8][column 8]
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float lo, hi;
+            f2_unpack(acc[i][j], lo, hi);
+            red[t * 64 + (2 * i) * 8 + j] = lo;
+            red[t * 64 + (2 * i + 1) * 8 + j] = hi;
+        }
+    bred[t >> 6][t & 63] = bsum;
+    __syncthreads();
+    for (int i = t; i < 32 * 64; i += NT) {
+        const int col = i & 63, c = i >> 6;
+        const int at = ((col >> 3) * 4 + (c >> 3)) * 64 + (c & 7) * 8 + (col & 7);
+        float v = red[at];
+#pragma unroll
+        for (int wv = 1; wv < 8; ++wv) v += red[wv * 32 * 64 + at];
+        a.part[((size_t)blockIdx.x * a.cin + cg + c) * K + ng + col] = v;
+    }
+    if (blockIdx.y == 0 && t < 64) {
+        float v = bred[0][t];
+        for (int k = 1; k < 4; ++k) v += bred[k][t];
+        a.partb[(size_t)blockIdx.x * K + ng + t] = v;
+    }
+}
+
 }  // namespace
+
+// Blocks of one weight gradient: about two per SM over all channel groups.
+static int split_blocks(long long units, int groups) {
+    long long nb = (304 + groups - 1) / groups;
+    if (nb > units) nb = units;
+    if (nb < 1) nb = 1;
+    const long long per = (units + nb - 1) / nb;
+    return (int)((units + per - 1) / per);
+}
+int f32_wgrad_splits(int cin, int cout, int n, int h, int wd) {
+    const long long tiles = (long long)((wd + WTW - 1) / WTW) * ((h + WTH - 1) / WTH) * n;
+    return split_blocks(tiles, (cout / 16) * ((cin + 15) / 16));
+}
+int f32_wgrad_up_splits(int cin, int cout, int n, int h, int wd) {
+    return split_blocks(((long long)n * h * wd + UPX - 1) / UPX, (cin / 32) * (cout / 16));
+}
+
+nrv_status f32_wgrad(const float* g, int cout, const float* x1, int c1, const float* x2, int c2, int n, int h,
+                     int wd, float* part, float* partb, cudaStream_t s) {
+    const int cin = c1 + c2;
+    if (cout % 16 || (cin % 16 && cin != 8) || (c2 && c1 % 16))
+        return fail(NRV_ERR_UNSUPPORTED, "weight gradient: channel groups");
+    F32Wgrad a;
+    memset(&a, 0, sizeof(a));
+    a.g = g;
+    a.x1 = x1;
+    a.x2 = x2;
+    a.c1 = c1;
+    a.c2 = c2;
+    a.cout = cout;
+    a.n = n;
+    a.h = h;
+    a.w = wd;
+    a.tiles_x = (wd + WTW - 1) / WTW;
+    a.tiles_y = (h + WTH - 1) / WTH;
+    if ((long long)a.tiles_x * a.tiles_y * n > 0x3FFFFFFF) return fail(NRV_ERR_UNSUPPORTED, "too many tiles");
+    a.ntiles = a.tiles_x * a.tiles_y * n;
+    const int nb = f32_wgrad_splits(cin, cout, n, h, wd);
+    a.tiles_per_block = (a.ntiles + nb - 1) / nb;
+    a.part = part;
+    a.partb = partb;
+    static bool attr = false;
+    if (!attr) {
+        NRV_CHECK_CUDA(cudaFuncSetAttribute(wgrad_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WSMEM));
+        attr = true;
+    }
+    wgrad_f32_kernel<<<dim3(nb, cout / 16, (cin + 15) / 16), WT, WSMEM, s>>>(a);
+    NRV_CHECK_LAUNCH();
+    return NRV_OK;
+}
+
+nrv_status f32_wgrad_up(const float* x, int cin, const float* g, int ldg, int cout, int n, int h, int wd,
+                        float* part, float* partb, cudaStream_t s) {
+    if (cin % 32 || cout % 16) return fail(NRV_ERR_UNSUPPORTED, "weight gradient: channel groups");
+    F32WgradUp a;
+    memset(&a, 0, sizeof(a));
+    a.x = x;
+    a.g = g;
+    a.cin = cin;
+    a.cout = cout;
+    a.ldg = ldg;
+    a.n = n;
+    a.h = h;
+    a.w = wd;
+    a.npx = (long long)n * h * wd;
+    const int nb = f32_wgrad_up_splits(cin, cout, n, h, wd);
+    const long long units = (a.npx + UPX - 1) / UPX;
+    a.px_per_block = (units + nb - 1) / nb * UPX;
+    a.part = part;
+    a.partb = partb;
+    static bool attr = false;
+    if (!attr) {
+        NRV_CHECK_CUDA(cudaFuncSetAttribute(wgrad_up_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, USMEM));
+        attr = true;
+    }
+    wgrad_up_f32_kernel<<<dim3(nb, cin / 32, cout / 16), NT, USMEM, s>>>(a);
+    NRV_CHECK_LAUNCH();
+    return NRV_OK;
+}
 
 nrv_status f32_conv3(const float* x1, int c1, const float* x2, int c2, const float* w, const float* bias,
                      int relu, const float* mask, float* y, int cout, int n, int h, int wd, cudaStream_t s) {

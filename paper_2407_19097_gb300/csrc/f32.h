@@ -17,4 +17,15 @@ nrv_status f32_upconv(const float* x, int cin, const float* w, const float* bias
 nrv_status f32_upconv_dgrad(const float* g, int ldg, int cout, const float* wt, const float* mask, float* gx,
                             int cin, int n, int h, int wd, cudaStream_t s);
 
+// Weight and bias gradient partials of a 3x3 conv: part[split][o][tap * cin + c] and
+// partb[split][o] over f32_wgrad_splits() splits of the pixels (g: [n][h][wd][cout]).
+int f32_wgrad_splits(int cin, int cout, int n, int h, int wd);
+nrv_status f32_wgrad(const float* g, int cout, const float* x1, int c1, const float* x2, int c2, int n, int h,
+                     int wd, float* part, float* partb, cudaStream_t s);
+// Of a transposed conv: part[split][c][ab * cout + o], partb[split][ab * cout + o]; g at (2h, 2wd)
+// with ldg channels per pixel, of which the first cout.
+int f32_wgrad_up_splits(int cin, int cout, int n, int h, int wd);
+nrv_status f32_wgrad_up(const float* x, int cin, const float* g, int ldg, int cout, int n, int h, int wd,
+                        float* part, float* partb, cudaStream_t s);
+
 }  // namespace nrv

@@ -61,6 +61,16 @@ struct Net {
     DevBuf grads;            // gradient tensors
     DevBuf partial;          // wgrad partial sums
     DevBuf tmaps;            // device copies of TMA descriptors (unused when passed by value)
+    // the backward pass's weight gradients run on a stream of the net's own beside the chain
+    // of data gradients; the last event is the join
+    static constexpr int SIDE_EVENTS = 24;
+    cudaStream_t side = nullptr;
+    cudaEvent_t side_ev[SIDE_EVENTS + 1] = {};
+    ~Net() {
+        if (side) cudaStreamDestroy(side);
+        for (cudaEvent_t e : side_ev)
+            if (e) cudaEventDestroy(e);
+    }
     // render-batch resources
     DevBuf batch_ws;
     DevBuf layer_ws;         // row-planar copies for nrv_net_run_layer

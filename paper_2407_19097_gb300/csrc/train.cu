@@ -136,54 +136,85 @@ struct ReduceSeg {
     float* dw;
 };
 
-__device__ __forceinline__ void reduce_item(const ReduceSeg& R, int i, int tx, int ty,
-                                            float (*red)[33]) {
+// Every segment in one launch: block b belongs to the segment whose range of 32-sum blocks
+// holds it.  Each thread reads eight chunks before it adds them, so the pass is bound by the
+// partials' bytes and not by a chain of dependent loads (a segment per launch, one load at a
+// time, took 0.2 ms of a 1.6 ms training step).
+constexpr int MAX_SEGS = 2 * NUM_LAYERS;
+struct ReduceTable {
+    int n;
+    int first[MAX_SEGS + 1];   // first block of each segment
+    ReduceSeg seg[MAX_SEGS];
+};
+
+__global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ ReduceTable T) {
+    __shared__ float red[8][33];
+    int k = 0;
+    while ((int)blockIdx.x >= T.first[k + 1]) ++k;
+    const ReduceSeg& R = T.seg[k];
+    const int tx = threadIdx.x, ty = threadIdx.y;
+    const int i = ((int)blockIdx.x - T.first[k]) * 32 + tx;
     float s = 0.0f;
     if (i < R.count)
-        for (int ch = ty; ch < R.nchunks; ch += 8) {
-            const float* pc = R.part + (size_t)ch * R.stride;
-            if (R.mode == 3) s += ((pc[i] + pc[R.cout + i]) + pc[2 * R.cout + i]) + pc[3 * R.cout + i];
-            else s += pc[i];
+        for (int c0 = ty; c0 < R.nchunks; c0 += 64) {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int ch = c0 + 8 * j;
+                v[j] = 0.0f;
+                if (ch < R.nchunks) {
+                    const float* pc = R.part + (size_t)ch * R.stride;
+                    if (R.mode == 3)
+                        v[j] = ((pc[i] + pc[R.cout + i]) + pc[2 * R.cout + i]) + pc[3 * R.cout + i];
+                    else v[j] = pc[i];
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s += v[j];
         }
     red[ty][tx] = s;
     __syncthreads();
     if (ty != 0 || i >= R.count) return;
     float t = red[0][tx];
-    for (int k = 1; k < 8; ++k) t += red[k][tx];
+    for (int j = 1; j < 8; ++j) t += red[j][tx];
     if (R.mode == 0) {
-        const int K = 9 * R.cin, o = i / K, k = i % K, tap = k / R.cin, c = k % R.cin;
+        const int K = 9 * R.cin, o = i / K, q = i % K, tap = q / R.cin, c = q % R.cin;
         if (c < R.cin_real) R.dw[((size_t)o * R.cin_real + c) * 9 + tap] = t;
     } else if (R.mode == 1) {
-        const int K = 4 * R.cout, c = i / K, k = i % K, ab = k / R.cout, o = k % R.cout;
+        const int K = 4 * R.cout, c = i / K, q = i % K, ab = q / R.cout, o = q % R.cout;
         R.dw[((size_t)c * R.cout + o) * 4 + ab] = t;
     } else {
         R.dw[i] = t;
     }
 }
 
-// Two reductions (a layer's weights and its bias) in one launch: the first segment's
-// blocks, then the second's.
-__global__ void reduce_partials_kernel(const __grid_constant__ ReduceSeg A,
-                                       const __grid_constant__ ReduceSeg B) {
-    __shared__ float red[8][33];
-    const int nba = (A.count + 31) / 32;
-    const bool first = (int)blockIdx.x < nba;
-    const int blk = first ? (int)blockIdx.x : (int)blockIdx.x - nba;
-    reduce_item(first ? A : B, blk * 32 + threadIdx.x, threadIdx.x, threadIdx.y, red);
-}
-
-static nrv_status reduce_partials(const float* part, int nchunks, size_t stride, int count, int mode,
-                                  int cout, int cin, int cin_real, float* dw, cudaStream_t s,
-                                  const ReduceSeg* second = nullptr) {
-    const ReduceSeg A{part, nchunks, stride, count, mode, cout, cin, cin_real, dw};
-    ReduceSeg B;
-    memset(&B, 0, sizeof(B));
-    if (second) B = *second;
-    const int blocks = (A.count + 31) / 32 + (B.count + 31) / 32;
-    reduce_partials_kernel<<<blocks, dim3(32, 8), 0, s>>>(A, B);
-    NRV_CHECK_LAUNCH();
-    return NRV_OK;
-}
+// The partial sums of a backward pass: one region per layer of the net's buffer, and the table
+// of the segments to reduce once every partial is written.
+struct Partials {
+    DevBuf* buf;
+    size_t used = 0;           // floats
+    ReduceTable T;
+    explicit Partials(DevBuf* b) : buf(b) { T.n = 0; T.first[0] = 0; }
+    // `floats` floats; the buffer was sized for the whole pass (reserve), so nothing moves
+    float* take(size_t floats) {
+        float* p = (float*)buf->p + used;
+        used += (floats + 31) / 32 * 32;
+        return used * sizeof(float) <= buf->bytes ? p : nullptr;
+    }
+    void add(const ReduceSeg& R) {
+        T.seg[T.n] = R;
+        T.first[T.n + 1] = T.first[T.n] + (R.count + 31) / 32;
+        ++T.n;
+    }
+    nrv_status flush(cudaStream_t s) {
+        if (T.n == 0) return NRV_OK;
+        reduce_partials_kernel<<<T.first[T.n], dim3(32, 8), 0, s>>>(T);
+        NRV_CHECK_LAUNCH();
+        T.n = 0;
+        used = 0;
+        return NRV_OK;
+    }
+};
 
 // ------------------------------------------------------------------ weight gradients, 2x2 transposed conv
 // part[chunk][c][ab*cout + o] = sum_{input px in chunk} x[q][c] * g[out(q, ab)][o]
@@ -464,14 +495,37 @@ static int blocks_for(size_t work, int per = 256) {
     return (int)(b > 0 ? b : 1);
 }
 
+// Gradient tensors of a backward pass, each with a buffer of its own: the weight gradients on
+// the side stream may read one long after the chain has gone on.
+enum Grad {
+    G_D0B, G_D0A, G_CAT0, G_E0B, G_E0A, G_D1B, G_D1A, G_CAT1, G_E1B, G_E1A, G_P0, G_D2B, G_D2A, G_CAT2,
+    G_E2B, G_E2A, G_P1, G_E3B, G_E3A, G_P2, NUM_GRADS
+};
+static const int kGradLevel[NUM_GRADS] = {0, 0, 0, 0, 0, 1, 1, 1, 1, 1, 1, 2, 2, 2, 2, 2, 2, 3, 3, 3};
+static const int kGradC[NUM_GRADS] = {16, 16, 32, 16, 16, 32, 32, 64, 32, 32, 16, 64, 64, 128, 64, 64, 32,
+                                      128, 128, 64};
+
+// The stream and events that the weight gradients run on, created on first use.
+static nrv_status net_side_stream(Net* net) {
+    if (net->side) return NRV_OK;
+    for (cudaEvent_t& e : net->side_ev)
+        if (!e) NRV_CHECK_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    NRV_CHECK_CUDA(cudaStreamCreateWithFlags(&net->side, cudaStreamNonBlocking));
+    return NRV_OK;
+}
+
 template <typename T>
 struct Bwd {
     Net* net;
     cudaStream_t s;
     const Geo& g;
     float* dparams;
-    T* W1[4];
-    T* W2[4];
+    Partials parts;
+    cudaStream_t sw;         // weight gradients (the side stream, or s itself)
+    T* G[NUM_GRADS];         // gradient tensors
+
+    Bwd(Net* net_, cudaStream_t s_, const Geo& g_, float* dp)
+        : net(net_), s(s_), g(g_), dparams(dp), parts(&net_->partial), sw(s_) {}
 
     T* A(int a) const { return reinterpret_cast<T*>((char*)net->acts.p + net->act_off[a]); }
     // saved activations: row-planar in BF16 (the tensor-core layout), NHWC in FP32
@@ -489,50 +543,102 @@ struct Bwd {
                               !x1.coff && x1.ld == c1 &&
                               (!c2 || (x2.planar && !x2.coff && x2.ld == c2));
             if (fits) {
-                const int groups = cin / 16 > 0 ? cin / 16 : 1;
-                const size_t per_split = (size_t)L.cout * 9 * cin;
-                const size_t max_split = (size_t)(304 + groups - 1) / groups;
-                NRV_TRY(net->partial.ensure((max_split * (per_split + L.cout)) * sizeof(float)));
-                float* part = (float*)net->partial.p;
-                float* partb = part + max_split * per_split;
+                const size_t per_split = (size_t)L.cout * 9 * cin, max_split = tc_splits(cin);
+                float* part = parts.take(max_split * per_split);
+                float* partb = parts.take(max_split * L.cout);
+                if (!part || !partb) return fail(NRV_ERR_STATE, "partial sums");
                 int nsplit = 0;
                 const nrv_status st = tc_wgrad(net, l, gpre.p, x1.p, c1, c2 ? x2.p : nullptr, c2, g.n,
                                                g.h[level], g.w[level], part, max_split * per_split,
-                                               partb, &nsplit, s);
+                                               partb, &nsplit, sw);
                 if (st == NRV_OK) {
-                    const ReduceSeg bias{partb, nsplit, (size_t)L.cout, L.cout, 2, L.cout, cin, L.cin,
-                                         dparams + L.boff};
-                    return reduce_partials(part, nsplit, per_split, (int)per_split, 0, L.cout, cin,
-                                           L.cin, dparams + L.woff, s, &bias);
+                    parts.add(ReduceSeg{part, nsplit, per_split, (int)per_split, 0, L.cout, cin, L.cin,
+                                        dparams + L.woff});
+                    parts.add(ReduceSeg{partb, nsplit, (size_t)L.cout, L.cout, 2, L.cout, cin, L.cin,
+                                        dparams + L.boff});
+                    return NRV_OK;
                 }
                 if (st != NRV_ERR_UNSUPPORTED) return st;
                 clear_error();
             }
         }
-        const int CG = cin < 16 ? cin : 16;
-        if (cin % CG || (c2 && c1 % CG) || L.cout % 16)
-            return fail(NRV_ERR_UNSUPPORTED, "weight gradient: channel groups");
         const int h = g.h[level], w = g.w[level];
-        const int TW = wgrad_tile_width(w), R = WG_TILE / TW;
+        const size_t per_split = (size_t)L.cout * 9 * cin;
+        int nblk, tpb = 0;
+        if (sizeof(T) == 4) nblk = f32_wgrad_splits(cin, L.cout, g.n, h, w);
+        else nblk = simt_splits(L.cout, cin, h, w, &tpb);
+        float* part = parts.take(nblk * per_split);
+        float* partb = parts.take((size_t)nblk * L.cout);
+        if (!part || !partb) return fail(NRV_ERR_STATE, "partial sums");
+        if constexpr (sizeof(T) == 4) {
+            NRV_TRY(f32_wgrad(gpre.p, L.cout, x1.p, c1, x2.p, c2, g.n, h, w, part, partb, sw));
+        } else {
+            const int CG = cin < 16 ? cin : 16;
+            if (cin % CG || (c2 && c1 % CG) || L.cout % 16)
+                return fail(NRV_ERR_UNSUPPORTED, "weight gradient: channel groups");
+            wgrad3_kernel<T><<<dim3((unsigned)nblk, L.cout / 16, cin / CG), WG_THREADS, 0, sw>>>(
+                gpre, L.cout, x1, c1, x2, c2, g.n, h, w, wgrad_tile_width(w), tpb, part, partb);
+            NRV_CHECK_LAUNCH();
+        }
+        parts.add(ReduceSeg{part, nblk, per_split, (int)per_split, 0, L.cout, cin, L.cin, dparams + L.woff});
+        parts.add(ReduceSeg{partb, nblk, (size_t)L.cout, L.cout, 2, L.cout, cin, L.cin, dparams + L.boff});
+        return NRV_OK;
+    }
+
+    // Splits of a layer's weight gradient: at most this many on the tensor cores; on the CUDA
+    // cores in BF16 about four blocks per SM in all, each a contiguous run of tpb tiles.
+    static size_t tc_splits(int cin) {
+        const int groups = cin / 16 > 0 ? cin / 16 : 1;
+        return (size_t)(304 + groups - 1) / groups;
+    }
+    int simt_splits(int cout, int cin, int h, int w, int* tpb) const {
+        const int CG = cin < 16 ? cin : 16, TW = wgrad_tile_width(w), R = WG_TILE / TW;
         const long long ntiles = (long long)g.n * ((h + R - 1) / R) * ((w + TW - 1) / TW);
-        const int groups = (L.cout / 16) * (cin / CG);
-        // about 4 blocks per SM in all, each a contiguous run of tiles
+        const int groups = (cout / 16) * (cin / CG) > 0 ? (cout / 16) * (cin / CG) : 1;
         long long nblk = (152LL * 4 + groups - 1) / groups;
         if (nblk > ntiles) nblk = ntiles;
         if (nblk < 1) nblk = 1;
-        const int tpb = (int)((ntiles + nblk - 1) / nblk);
-        nblk = (ntiles + tpb - 1) / tpb;
-        const size_t need = ((size_t)nblk * L.cout * 9 * cin + (size_t)nblk * L.cout) * sizeof(float);
-        NRV_TRY(net->partial.ensure(need));
-        float* part = (float*)net->partial.p;
-        float* partb = part + (size_t)nblk * L.cout * 9 * cin;
-        wgrad3_kernel<T><<<dim3((unsigned)nblk, L.cout / 16, cin / CG), WG_THREADS, 0, s>>>(
-            gpre, L.cout, x1, c1, x2, c2, g.n, h, w, TW, tpb, part, partb);
-        NRV_CHECK_LAUNCH();
-        NRV_TRY(reduce_partials(part, (int)nblk, (size_t)L.cout * 9 * cin, L.cout * 9 * cin, 0, L.cout,
-                                cin, L.cin, dparams + L.woff, s));
-        return reduce_partials(partb, (int)nblk, L.cout, L.cout, 2, L.cout, cin, L.cin,
-                               dparams + L.boff, s);
+        *tpb = (int)((ntiles + nblk - 1) / nblk);
+        return (int)((ntiles + *tpb - 1) / *tpb);
+    }
+    int simt_up_splits(int cin, size_t npx, size_t* chunk) const {
+        const int groups = cin / 16;
+        size_t nch = (608 + groups - 1) / groups;
+        const size_t maxch = (npx + 127) / 128;
+        if (nch > maxch) nch = maxch;
+        if (nch < 1) nch = 1;
+        *chunk = (npx + nch - 1) / nch;
+        return (int)((npx + *chunk - 1) / *chunk);
+    }
+    // Floats of partial sums layer l may take (either path), its pixels at `level` of g.
+    size_t need(int l, int level) const {
+        const Layer& L = net->layers[l];
+        const int h = g.h[level], w = g.w[level];
+        auto pad = [](size_t f) { return (f + 31) / 32 * 32; };
+        size_t per, bias, ns;
+        if (L.kind == CONV3) {
+            const int cin = l == L_E0A ? net->c0p : L.cin;
+            int tpb;
+            per = (size_t)L.cout * 9 * cin;
+            bias = L.cout;
+            if (sizeof(T) == 4) return pad(f32_wgrad_splits(cin, L.cout, g.n, h, w) * per) + pad((size_t)f32_wgrad_splits(cin, L.cout, g.n, h, w) * bias);
+            ns = simt_splits(L.cout, cin, h, w, &tpb);
+            return pad(tc_splits(cin) * per) + pad(tc_splits(cin) * bias) + pad(ns * per) + pad(ns * bias);
+        }
+        per = (size_t)L.cin * 4 * L.cout;
+        bias = 4 * L.cout;
+        if (sizeof(T) == 4) {
+            ns = f32_wgrad_up_splits(L.cin, L.cout, g.n, h, w);
+            return pad(ns * per) + pad(ns * bias);
+        }
+        size_t chunk;
+        ns = simt_up_splits(L.cin, g.px(level), &chunk);
+        const size_t tc = up_splits(L.cout);
+        return pad(tc * per) + pad(tc * bias) + pad(ns * per) + pad(ns * bias);
+    }
+    static size_t up_splits(int cout) {
+        const int groups = 4 * cout <= 128 ? 1 : 2;
+        return (size_t)(304 + groups - 1) / groups;
     }
 
     nrv_status dgrad_conv(int l, TView<const T> gpre, TView<T> out, TView<const T> mask,
@@ -588,45 +694,46 @@ struct Bwd {
         if (sizeof(T) == 2 && x.planar && !x.coff && x.ld == L.cin && gout.planar &&
             gout.ld % 8 == 0 && gout.coff % 8 == 0 && gout.coff + L.cout <= gout.ld) {
             // BF16: on the tensor cores, the bias gradient beside it
-            const int groups = 4 * L.cout <= 128 ? 1 : 2;
-            const size_t per_split = (size_t)L.cin * 4 * L.cout;
-            const size_t max_split = (size_t)(304 + groups - 1) / groups;
-            NRV_TRY(net->partial.ensure((max_split * (per_split + 4 * L.cout)) * sizeof(float)));
-            float* part = (float*)net->partial.p;
-            float* partb = part + max_split * per_split;
+            const size_t per_split = (size_t)L.cin * 4 * L.cout, max_split = up_splits(L.cout);
+            float* part = parts.take(max_split * per_split);
+            float* partb = parts.take(max_split * 4 * L.cout);
+            if (!part || !partb) return fail(NRV_ERR_STATE, "partial sums");
             int nsplit = 0;
             const nrv_status st = tc_wgrad_up(net, l, gout.p, gout.ld, gout.coff, x.p, g.n,
                                               g.h[level_in], g.w[level_in], part,
-                                              max_split * per_split, partb, &nsplit, s);
+                                              max_split * per_split, partb, &nsplit, sw);
             if (st == NRV_OK) {
                 // bias, per split: the four kernel positions' sums of each channel
-                const ReduceSeg bias{partb, nsplit, (size_t)4 * L.cout, L.cout, 3, L.cout, L.cin,
-                                     L.cin, dparams + L.boff};
-                return reduce_partials(part, nsplit, per_split, (int)per_split, 1, L.cout, L.cin,
-                                       L.cin, dparams + L.woff, s, &bias);
+                parts.add(ReduceSeg{part, nsplit, per_split, (int)per_split, 1, L.cout, L.cin, L.cin,
+                                    dparams + L.woff});
+                parts.add(ReduceSeg{partb, nsplit, (size_t)4 * L.cout, L.cout, 3, L.cout, L.cin, L.cin,
+                                    dparams + L.boff});
+                return NRV_OK;
             }
             if (st != NRV_ERR_UNSUPPORTED) return st;
             clear_error();
         }
         const size_t npx = g.px(level_in);
-        const int groups = L.cin / 16;
-        size_t nch = (608 + groups - 1) / groups;
-        const size_t maxch = (npx + 127) / 128;
-        if (nch > maxch) nch = maxch;
-        if (nch < 1) nch = 1;
-        const size_t chunk = (npx + nch - 1) / nch;
-        nch = (npx + chunk - 1) / chunk;
         const int K = 4 * L.cout;
-        NRV_TRY(net->partial.ensure((nch * L.cin * K + nch * K) * sizeof(float)));
-        float* part = (float*)net->partial.p;
-        float* partb = part + nch * L.cin * K;
-        wgrad_up_kernel<T><<<dim3((unsigned)nch, groups), 256, 0, s>>>(
-            x, L.cin, gout, L.cout, g.n, g.h[level_in], g.w[level_in], chunk, part, partb);
-        NRV_CHECK_LAUNCH();
-        NRV_TRY(reduce_partials(part, (int)nch, (size_t)L.cin * K, L.cin * K, 1, L.cout, L.cin, L.cin,
-                                dparams + L.woff, s));
-        return reduce_partials(partb, (int)nch, K, L.cout, 3, L.cout, L.cin, L.cin,
-                               dparams + L.boff, s);
+        int nch;
+        size_t chunk = 0;
+        if (sizeof(T) == 4) nch = f32_wgrad_up_splits(L.cin, L.cout, g.n, g.h[level_in], g.w[level_in]);
+        else nch = simt_up_splits(L.cin, npx, &chunk);
+        float* part = parts.take((size_t)nch * L.cin * K);
+        float* partb = parts.take((size_t)nch * K);
+        if (!part || !partb) return fail(NRV_ERR_STATE, "partial sums");
+        if constexpr (sizeof(T) == 4) {
+            NRV_TRY(f32_wgrad_up(x.p, L.cin, gout.p + gout.coff, gout.ld, L.cout, g.n, g.h[level_in],
+                                 g.w[level_in], part, partb, sw));
+        } else {
+            wgrad_up_kernel<T><<<dim3((unsigned)nch, L.cin / 16), 256, 0, sw>>>(
+                x, L.cin, gout, L.cout, g.n, g.h[level_in], g.w[level_in], chunk, part, partb);
+            NRV_CHECK_LAUNCH();
+        }
+        parts.add(ReduceSeg{part, nch, (size_t)L.cin * K, L.cin * K, 1, L.cout, L.cin, L.cin,
+                            dparams + L.woff});
+        parts.add(ReduceSeg{partb, nch, (size_t)K, L.cout, 3, L.cout, L.cin, L.cin, dparams + L.boff});
+        return NRV_OK;
     }
 
     // data gradient of transposed conv l at level_in, zeroed where the layer's input xm (a
@@ -654,11 +761,6 @@ struct Bwd {
         return NRV_OK;
     }
 
-    nrv_status upconv_bwd(int l, int xin, TView<const T> gout, TView<T> gx, int level_in) {
-        NRV_TRY(wgrad_up(l, CA(xin), gout, level_in));
-        return dgrad_up(l, gout, CA(xin), gx, level_in);
-    }
-
     nrv_status pool_bwd(TView<const T> gp, TView<const T> gs, int e, TView<T> ge, int level) {
         const int c = net->act_c[e];
         pool_bwd_kernel<T><<<blocks_for(g.px(level) * c / 8), 256, 0, s>>>(
@@ -675,72 +777,132 @@ struct Bwd {
         return TView<const T>{p, ld, kPlanar, coff};
     }
 
+    // The data gradients form a chain on s; each weight gradient needs one link of it and
+    // nothing needs the weight gradients until the end, so they run beside it on sw: point()
+    // lets sw go on once what s holds so far is done.
+    int npoint = 0;
+    nrv_status point() {
+        if (sw == s) return NRV_OK;
+        if (npoint >= Net::SIDE_EVENTS) return fail(NRV_ERR_STATE, "backward events");
+        NRV_CHECK_CUDA(cudaEventRecord(net->side_ev[npoint], s));
+        NRV_CHECK_CUDA(cudaStreamWaitEvent(sw, net->side_ev[npoint], 0));
+        ++npoint;
+        return NRV_OK;
+    }
+    // s continues after everything on sw
+    nrv_status join() {
+        if (sw == s) return NRV_OK;
+        NRV_CHECK_CUDA(cudaEventRecord(net->side_ev[Net::SIDE_EVENTS], sw));
+        NRV_CHECK_CUDA(cudaStreamWaitEvent(s, net->side_ev[Net::SIDE_EVENTS], 0));
+        return NRV_OK;
+    }
+
     nrv_status run(const float* drgb, const T* netin) {
+        // every layer's partial sums side by side, reduced by one launch at the end
+        static const int lvl[NUM_LAYERS] = {0, 0, 1, 1, 2, 2, 3, 3, 3, 2, 2, 2, 1, 1, 1, 0, 0, 0};
+        const size_t tot = (size_t)g.n * net->geo_H * net->geo_W;
+        size_t hch = 608, hchunk = (tot + hch - 1) / hch;
+        if (hchunk < 64) hchunk = 64;
+        hch = (tot + hchunk - 1) / hchunk;
+        size_t floats = (hch * 51 + 31) / 32 * 32;
+        for (int l = 0; l < L_HEAD; ++l) floats += need(l, lvl[l]);
+        NRV_TRY(net->partial.ensure(floats * sizeof(float)));
+        NRV_TRY(net_side_stream(net));
+        sw = net->side;
+        NRV_TRY(point());
+        const nrv_status st = layers_bwd(drgb, netin, hch, hchunk);
+        const nrv_status fs = st == NRV_OK ? parts.flush(sw) : st;
+        const nrv_status js = join();   // also after a failure: nothing runs on past this call
+        return fs != NRV_OK ? fs : js;
+    }
+
+    nrv_status layers_bwd(const float* drgb, const T* netin, size_t hch, size_t hchunk) {
         const TView<const T> none{nullptr, 0};
         const int H = net->geo_H, Wd = net->geo_W;
         // head
         const Layer& Lh = net->layers[L_HEAD];
-        head_dgrad_kernel<T><<<blocks_for(g.px(0)), 256, 0, s>>>(
-            drgb, (const float*)net->params.p + Lh.woff, CA(A_D0B), V(W1[0], 16), g.n, g.h[0],
-            g.w[0], H, Wd);
-        NRV_CHECK_LAUNCH();
         {
-            const size_t tot = (size_t)g.n * H * Wd;
-            size_t nch = 608;
-            size_t chunk = (tot + nch - 1) / nch;
-            if (chunk < 64) chunk = 64;
-            nch = (tot + chunk - 1) / chunk;
-            NRV_TRY(net->partial.ensure(nch * 51 * sizeof(float)));
-            head_wgrad_kernel<T><<<(unsigned)nch, 256, 0, s>>>(drgb, CA(A_D0B), g.n, g.h[0], g.w[0],
-                                                               H, Wd, chunk, (float*)net->partial.p);
+            float* part = parts.take(hch * 51);
+            if (!part) return fail(NRV_ERR_STATE, "partial sums");
+            head_wgrad_kernel<T><<<(unsigned)hch, 256, 0, sw>>>(drgb, CA(A_D0B), g.n, g.h[0], g.w[0], H, Wd,
+                                                               hchunk, part);
             NRV_CHECK_LAUNCH();
             // weight (48) and bias (3) are consecutive in the parameter vector
             if (Lh.boff != Lh.woff + 48) return fail(NRV_ERR_STATE, "head parameter layout");
-            NRV_TRY(reduce_partials((const float*)net->partial.p, (int)nch, 51, 51, 2, 3, 16, 16,
-                                    dparams + Lh.woff, s));
+            parts.add(ReduceSeg{part, (int)hch, 51, 51, 2, 3, 16, 16, dparams + Lh.woff});
         }
+        head_dgrad_kernel<T><<<blocks_for(g.px(0)), 256, 0, s>>>(
+            drgb, (const float*)net->params.p + Lh.woff, CA(A_D0B), V(G[G_D0B], 16), g.n, g.h[0],
+            g.w[0], H, Wd);
+        NRV_CHECK_LAUNCH();
+        NRV_TRY(point());
         // level 0 decoder
-        NRV_TRY(wgrad_conv(L_D0B, C(W1[0], 16), CA(A_D0A), 16, none, 0, 0));
-        NRV_TRY(dgrad_conv(L_D0B, C(W1[0], 16), V(W2[0], 16), CA(A_D0A), 0));
-        NRV_TRY(wgrad_conv(L_D0A, C(W2[0], 16), CA(A_UP1), 16, CA(A_E0B), 16, 0));
-        NRV_TRY(dgrad_conv(L_D0A, C(W2[0], 16), V(W1[0], 32), none, 0));
-        NRV_TRY(upconv_bwd(L_UP1, A_D1B, C(W1[0], 32), V(W1[1], 32), 1));
+        NRV_TRY(wgrad_conv(L_D0B, C(G[G_D0B], 16), CA(A_D0A), 16, none, 0, 0));
+        NRV_TRY(dgrad_conv(L_D0B, C(G[G_D0B], 16), V(G[G_D0A], 16), CA(A_D0A), 0));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_D0A, C(G[G_D0A], 16), CA(A_UP1), 16, CA(A_E0B), 16, 0));
+        NRV_TRY(dgrad_conv(L_D0A, C(G[G_D0A], 16), V(G[G_CAT0], 32), none, 0));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_up(L_UP1, CA(A_D1B), C(G[G_CAT0], 32), 1));
+        NRV_TRY(dgrad_up(L_UP1, C(G[G_CAT0], 32), CA(A_D1B), V(G[G_D1B], 32), 1));
+        NRV_TRY(point());
         // level 1 decoder
-        NRV_TRY(wgrad_conv(L_D1B, C(W1[1], 32), CA(A_D1A), 32, none, 0, 1));
-        NRV_TRY(dgrad_conv(L_D1B, C(W1[1], 32), V(W2[1], 32), CA(A_D1A), 1));
-        NRV_TRY(wgrad_conv(L_D1A, C(W2[1], 32), CA(A_UP2), 32, CA(A_E1B), 32, 1));
-        NRV_TRY(dgrad_conv(L_D1A, C(W2[1], 32), V(W1[1], 64), none, 1));
-        NRV_TRY(upconv_bwd(L_UP2, A_D2B, C(W1[1], 64), V(W1[2], 64), 2));
+        NRV_TRY(wgrad_conv(L_D1B, C(G[G_D1B], 32), CA(A_D1A), 32, none, 0, 1));
+        NRV_TRY(dgrad_conv(L_D1B, C(G[G_D1B], 32), V(G[G_D1A], 32), CA(A_D1A), 1));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_D1A, C(G[G_D1A], 32), CA(A_UP2), 32, CA(A_E1B), 32, 1));
+        NRV_TRY(dgrad_conv(L_D1A, C(G[G_D1A], 32), V(G[G_CAT1], 64), none, 1));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_up(L_UP2, CA(A_D2B), C(G[G_CAT1], 64), 2));
+        NRV_TRY(dgrad_up(L_UP2, C(G[G_CAT1], 64), CA(A_D2B), V(G[G_D2B], 64), 2));
+        NRV_TRY(point());
         // level 2 decoder
-        NRV_TRY(wgrad_conv(L_D2B, C(W1[2], 64), CA(A_D2A), 64, none, 0, 2));
-        NRV_TRY(dgrad_conv(L_D2B, C(W1[2], 64), V(W2[2], 64), CA(A_D2A), 2));
-        NRV_TRY(wgrad_conv(L_D2A, C(W2[2], 64), CA(A_UP3), 64, CA(A_E2B), 64, 2));
-        NRV_TRY(dgrad_conv(L_D2A, C(W2[2], 64), V(W1[2], 128), none, 2));
-        NRV_TRY(upconv_bwd(L_UP3, A_E3B, C(W1[2], 128), V(W1[3], 128), 3));
+        NRV_TRY(wgrad_conv(L_D2B, C(G[G_D2B], 64), CA(A_D2A), 64, none, 0, 2));
+        NRV_TRY(dgrad_conv(L_D2B, C(G[G_D2B], 64), V(G[G_D2A], 64), CA(A_D2A), 2));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_D2A, C(G[G_D2A], 64), CA(A_UP3), 64, CA(A_E2B), 64, 2));
+        NRV_TRY(dgrad_conv(L_D2A, C(G[G_D2A], 64), V(G[G_CAT2], 128), none, 2));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_up(L_UP3, CA(A_E3B), C(G[G_CAT2], 128), 3));
+        NRV_TRY(dgrad_up(L_UP3, C(G[G_CAT2], 128), CA(A_E3B), V(G[G_E3B], 128), 3));
+        NRV_TRY(point());
         // bottom level
-        NRV_TRY(wgrad_conv(L_E3B, C(W1[3], 128), CA(A_E3A), 128, none, 0, 3));
-        NRV_TRY(dgrad_conv(L_E3B, C(W1[3], 128), V(W2[3], 128), CA(A_E3A), 3));
-        NRV_TRY(wgrad_conv(L_E3A, C(W2[3], 128), CA(A_P2), 64, none, 0, 3));
-        NRV_TRY(dgrad_conv(L_E3A, C(W2[3], 128), V(W1[3], 64), none, 3));
-        // level 2 encoder: skip gradient sits in channels 64..127 of W1[2]
-        NRV_TRY(pool_bwd(C(W1[3], 64), C(W1[2], 128, 64), A_E2B, V(W2[2], 64), 2));
-        NRV_TRY(wgrad_conv(L_E2B, C(W2[2], 64), CA(A_E2A), 64, none, 0, 2));
-        NRV_TRY(dgrad_conv(L_E2B, C(W2[2], 64), V(W1[2], 64), CA(A_E2A), 2));
-        NRV_TRY(wgrad_conv(L_E2A, C(W1[2], 64), CA(A_P1), 32, none, 0, 2));
-        NRV_TRY(dgrad_conv(L_E2A, C(W1[2], 64), V(W2[2], 32), none, 2));
-        // level 1 encoder: skip gradient in channels 32..63 of W1[1]
-        NRV_TRY(pool_bwd(C(W2[2], 32), C(W1[1], 64, 32), A_E1B, V(W2[1], 32), 1));
-        NRV_TRY(wgrad_conv(L_E1B, C(W2[1], 32), CA(A_E1A), 32, none, 0, 1));
-        NRV_TRY(dgrad_conv(L_E1B, C(W2[1], 32), V(W1[1], 32), CA(A_E1A), 1));
-        NRV_TRY(wgrad_conv(L_E1A, C(W1[1], 32), CA(A_P0), 16, none, 0, 1));
-        NRV_TRY(dgrad_conv(L_E1A, C(W1[1], 32), V(W2[1], 16), none, 1));
-        // level 0 encoder: skip gradient in channels 16..31 of W1[0]
-        NRV_TRY(pool_bwd(C(W2[1], 16), C(W1[0], 32, 16), A_E0B, V(W2[0], 16), 0));
-        NRV_TRY(wgrad_conv(L_E0B, C(W2[0], 16), CA(A_E0A), 16, none, 0, 0));
-        NRV_TRY(dgrad_conv(L_E0B, C(W2[0], 16), V(W1[0], 16), CA(A_E0A), 0));
-        NRV_TRY(wgrad_conv(L_E0A, C(W1[0], 16), C(const_cast<T*>(netin), net->c0p), net->c0p, none,
-                           0, 0));
-        return NRV_OK;
+        NRV_TRY(wgrad_conv(L_E3B, C(G[G_E3B], 128), CA(A_E3A), 128, none, 0, 3));
+        NRV_TRY(dgrad_conv(L_E3B, C(G[G_E3B], 128), V(G[G_E3A], 128), CA(A_E3A), 3));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_E3A, C(G[G_E3A], 128), CA(A_P2), 64, none, 0, 3));
+        NRV_TRY(dgrad_conv(L_E3A, C(G[G_E3A], 128), V(G[G_P2], 64), none, 3));
+        // level 2 encoder: the skip gradient is channels 64..127 of the concatenation's
+        NRV_TRY(pool_bwd(C(G[G_P2], 64), C(G[G_CAT2], 128, 64), A_E2B, V(G[G_E2B], 64), 2));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_E2B, C(G[G_E2B], 64), CA(A_E2A), 64, none, 0, 2));
+        NRV_TRY(dgrad_conv(L_E2B, C(G[G_E2B], 64), V(G[G_E2A], 64), CA(A_E2A), 2));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_E2A, C(G[G_E2A], 64), CA(A_P1), 32, none, 0, 2));
+        NRV_TRY(dgrad_conv(L_E2A, C(G[G_E2A], 64), V(G[G_P1], 32), none, 2));
+        // level 1 encoder: channels 32..63
+        NRV_TRY(pool_bwd(C(G[G_P1], 32), C(G[G_CAT1], 64, 32), A_E1B, V(G[G_E1B], 32), 1));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_E1B, C(G[G_E1B], 32), CA(A_E1A), 32, none, 0, 1));
+        NRV_TRY(dgrad_conv(L_E1B, C(G[G_E1B], 32), V(G[G_E1A], 32), CA(A_E1A), 1));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_E1A, C(G[G_E1A], 32), CA(A_P0), 16, none, 0, 1));
+        NRV_TRY(dgrad_conv(L_E1A, C(G[G_E1A], 32), V(G[G_P0], 16), none, 1));
+        // level 0 encoder: channels 16..31
+        NRV_TRY(pool_bwd(C(G[G_P0], 16), C(G[G_CAT0], 32, 16), A_E0B, V(G[G_E0B], 16), 0));
+        NRV_TRY(point());
+        NRV_TRY(wgrad_conv(L_E0B, C(G[G_E0B], 16), CA(A_E0A), 16, none, 0, 0));
+        NRV_TRY(dgrad_conv(L_E0B, C(G[G_E0B], 16), V(G[G_E0A], 16), CA(A_E0A), 0));
+        NRV_TRY(point());
+        return wgrad_conv(L_E0A, C(G[G_E0A], 16), C(const_cast<T*>(netin), net->c0p), net->c0p, none, 0, 0);
+    }
+
+    // one layer's weight gradient alone, on s
+    template <typename Fn>
+    nrv_status alone(int l, Fn fn) {
+        NRV_TRY(net->partial.ensure(need(l, 0) * sizeof(float)));
+        NRV_TRY(fn());
+        return parts.flush(s);
     }
 };
 
@@ -759,9 +921,11 @@ nrv_status net_layer_wgrad(Net* net, int l, const void* dy, const void* x1, cons
         g.w[0] = w;
         if (prec == NRV_PREC_F32) {
             using T = float;
-            Bwd<T> b{net, s, g, dgrad, {}, {}};
-            return b.wgrad_up(l, TView<const T>{(const T*)x1, L.cin},
-                              TView<const T>{(const T*)dy, L.cout}, 0);
+            Bwd<T> b(net, s, g, dgrad);
+            return b.alone(l, [&] {
+                return b.wgrad_up(l, TView<const T>{(const T*)x1, L.cin},
+                                  TView<const T>{(const T*)dy, L.cout}, 0);
+            });
         }
         if (prec != NRV_PREC_BF16) return fail(NRV_ERR_UNSUPPORTED, "weight gradients in F32 or BF16");
         using T = __nv_bfloat16;
@@ -773,8 +937,10 @@ nrv_status net_layer_wgrad(Net* net, int l, const void* dy, const void* x1, cons
         T *pg = (T*)ws, *px = (T*)(ws + bg);
         NRV_TRY(relayout(dy, pg, 2 * rows, 2 * w, L.cout, 2, true, s));
         NRV_TRY(relayout(x1, px, rows, w, L.cin, 2, true, s));
-        Bwd<T> b{net, s, g, dgrad, {}, {}};
-        return b.wgrad_up(l, TView<const T>{px, L.cin, 1}, TView<const T>{pg, L.cout, 1}, 0);
+        Bwd<T> b(net, s, g, dgrad);
+        return b.alone(l, [&] {
+            return b.wgrad_up(l, TView<const T>{px, L.cin, 1}, TView<const T>{pg, L.cout, 1}, 0);
+        });
     }
     if (L.kind != CONV3) return fail(NRV_ERR_ARG, "layer %s has no weight gradient here", L.name);
     int c1 = l == L_E0A ? net->c0p : L.cin, c2 = 0;
@@ -788,9 +954,11 @@ nrv_status net_layer_wgrad(Net* net, int l, const void* dy, const void* x1, cons
     g.w[0] = w;
     if (prec == NRV_PREC_F32) {
         using T = float;
-        Bwd<T> b{net, s, g, dgrad, {}, {}};
-        return b.wgrad_conv(l, TView<const T>{(const T*)dy, L.cout}, TView<const T>{(const T*)x1, c1},
-                            c1, TView<const T>{(const T*)x2, c2}, c2, 0);
+        Bwd<T> b(net, s, g, dgrad);
+        return b.alone(l, [&] {
+            return b.wgrad_conv(l, TView<const T>{(const T*)dy, L.cout}, TView<const T>{(const T*)x1, c1},
+                                c1, TView<const T>{(const T*)x2, c2}, c2, 0);
+        });
     }
     if (prec != NRV_PREC_BF16) return fail(NRV_ERR_UNSUPPORTED, "weight gradients in F32 or BF16");
     // BF16: row-planar copies, as the backward pass keeps its tensors
@@ -804,9 +972,11 @@ nrv_status net_layer_wgrad(Net* net, int l, const void* dy, const void* x1, cons
     NRV_TRY(relayout(dy, pg, rows, w, L.cout, 2, true, s));
     NRV_TRY(relayout(x1, p1, rows, w, c1, 2, true, s));
     if (c2) NRV_TRY(relayout(x2, p2, rows, w, c2, 2, true, s));
-    Bwd<T> b{net, s, g, dgrad, {}, {}};
-    return b.wgrad_conv(l, TView<const T>{pg, L.cout, 1}, TView<const T>{p1, c1, 1}, c1,
-                        TView<const T>{p2, c2, 1}, c2, 0);
+    Bwd<T> b(net, s, g, dgrad);
+    return b.alone(l, [&] {
+        return b.wgrad_conv(l, TView<const T>{pg, L.cout, 1}, TView<const T>{p1, c1, 1}, c1,
+                            TView<const T>{p2, c2, 1}, c2, 0);
+    });
 }
 
 nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, int n, int h, int w,
@@ -822,7 +992,7 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
         g.w[0] = w;
         if (prec == NRV_PREC_F32) {
             using T = float;
-            Bwd<T> b{net, s, g, nullptr, {}, {}};
+            Bwd<T> b(net, s, g, nullptr);
             return b.dgrad_up(l, TView<const T>{(const T*)dy, L.cout}, TView<const T>{(const T*)mask, L.cin},
                               TView<T>{(T*)dx, L.cin}, 0);
         }
@@ -837,7 +1007,7 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
         T *pg = (T*)ws, *pm = (T*)(ws + bg), *po = (T*)(ws + bg + bm);
         NRV_TRY(relayout(dy, pg, 2 * rows, 2 * w, L.cout, 2, true, s));
         NRV_TRY(relayout(mask, pm, rows, w, L.cin, 2, true, s));
-        Bwd<T> b{net, s, g, nullptr, {}, {}};
+        Bwd<T> b(net, s, g, nullptr);
         NRV_TRY(b.dgrad_up(l, TView<const T>{pg, L.cout, 1}, TView<const T>{pm, L.cin, 1},
                            TView<T>{po, L.cin, 1}, 0));
         return relayout(po, dx, rows, w, L.cin, 2, false, s);
@@ -851,7 +1021,7 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
     g.w[0] = w;
     if (prec == NRV_PREC_F32) {
         using T = float;
-        Bwd<T> b{net, s, g, nullptr, {}, {}};
+        Bwd<T> b(net, s, g, nullptr);
         return b.dgrad_conv(l, TView<const T>{(const T*)dy, L.cout}, TView<T>{(T*)dx, L.cin},
                             TView<const T>{(const T*)mask, mask ? L.cin : 0}, 0);
     }
@@ -866,7 +1036,7 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
     T *pg = (T*)ws, *pm = mask ? (T*)(ws + bg) : nullptr, *po = (T*)(ws + bg + bm);
     NRV_TRY(relayout(dy, pg, rows, w, L.cout, 2, true, s));
     if (mask) NRV_TRY(relayout(mask, pm, rows, w, L.cin, 2, true, s));
-    Bwd<T> b{net, s, g, nullptr, {}, {}};
+    Bwd<T> b(net, s, g, nullptr);
     NRV_TRY(b.dgrad_conv(l, TView<const T>{pg, L.cout, 1}, TView<T>{po, L.cin, 1},
                          TView<const T>{pm, mask ? L.cin : 0, mask ? 1 : 0}, 0));
     return relayout(po, dx, rows, w, L.cin, 2, false, s);
@@ -876,29 +1046,20 @@ nrv_status net_backward(Net* net, const float* drgb, float* dparams, cudaStream_
     if (!net->saved) return fail(NRV_ERR_STATE, "backward without a preceding training forward");
     const Geo& g = net->geo;
     const size_t es = elem_size(net->act_prec);
-    size_t off[9], tot = 0;
-    const int chans[4] = {32, 64, 128, 128};
-    for (int l = 0; l < 4; ++l) {
-        off[2 * l] = tot;
-        tot += (g.px(l) * chans[l] * es + 1023) / 1024 * 1024;
-        off[2 * l + 1] = tot;
-        tot += (g.px(l) * chans[l] * es + 1023) / 1024 * 1024;
+    size_t off[NUM_GRADS], tot = 0;
+    for (int k = 0; k < NUM_GRADS; ++k) {
+        off[k] = tot;
+        tot += (g.px(kGradLevel[k]) * kGradC[k] * es + 1023) / 1024 * 1024;
     }
     NRV_TRY(net->grads.ensure(tot));
     if (net->act_prec == NRV_PREC_F32) {
-        Bwd<float> b{net, s, g, dparams, {}, {}};
-        for (int l = 0; l < 4; ++l) {
-            b.W1[l] = (float*)((char*)net->grads.p + off[2 * l]);
-            b.W2[l] = (float*)((char*)net->grads.p + off[2 * l + 1]);
-        }
+        Bwd<float> b(net, s, g, dparams);
+        for (int k = 0; k < NUM_GRADS; ++k) b.G[k] = (float*)((char*)net->grads.p + off[k]);
         return b.run(drgb, (const float*)net->saved_in);
     }
     if (net->act_prec == NRV_PREC_BF16) {
-        Bwd<__nv_bfloat16> b{net, s, g, dparams, {}, {}};
-        for (int l = 0; l < 4; ++l) {
-            b.W1[l] = (__nv_bfloat16*)((char*)net->grads.p + off[2 * l]);
-            b.W2[l] = (__nv_bfloat16*)((char*)net->grads.p + off[2 * l + 1]);
-        }
+        Bwd<__nv_bfloat16> b(net, s, g, dparams);
+        for (int k = 0; k < NUM_GRADS; ++k) b.G[k] = (__nv_bfloat16*)((char*)net->grads.p + off[k]);
         return b.run(drgb, (const __nv_bfloat16*)net->saved_in);
     }
     return fail(NRV_ERR_UNSUPPORTED, "backward is available for FP32 and BF16 only");
