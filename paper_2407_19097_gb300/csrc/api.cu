@@ -243,10 +243,12 @@ extern "C" nrv_status nrv_rasterize(nrv_scene* s, const nrv_view* views, int n,
     }
     cudaStream_t st = (cudaStream_t)stream;
     NRV_TRY(raster_views(s, views, n, keys, st));
+    ResolveArgs ra[8];
+    memset(ra, 0, sizeof(ra));
+    int nr = 0;
     for (int i = 0; i < n; ++i) {
         if (!gb[i].d_depth && !gb[i].d_mask && !gb[i].d_attr) continue;
-        ResolveArgs a;
-        memset(&a, 0, sizeof(a));
+        ResolveArgs& a = ra[nr++];
         a.key = reinterpret_cast<const unsigned long long*>(gb[i].d_key);
         a.attr = s->d.d_attr;
         a.base = (uint32_t)s->d.index_base;
@@ -258,9 +260,8 @@ extern "C" nrv_status nrv_rasterize(nrv_scene* s, const nrv_view* views, int n,
         a.depth = gb[i].d_depth;
         a.mask = gb[i].d_mask;
         a.gattr = gb[i].d_attr;
-        NRV_TRY(launch_resolve(a, st));
     }
-    return NRV_OK;
+    return nr ? launch_resolve(ra, nr, st) : NRV_OK;
 }
 
 extern "C" nrv_status nrv_pack(const nrv_gbuffer* gb, int h, int w, const nrv_pack_desc* d,
@@ -303,7 +304,7 @@ extern "C" nrv_status nrv_resolve(nrv_scene* s, const nrv_view* view, const uint
     a.depth = gb->d_depth;
     a.mask = gb->d_mask;
     a.gattr = gb->d_attr;
-    return launch_resolve(a, (cudaStream_t)stream);
+    return launch_resolve(&a, 1, (cudaStream_t)stream);
 }
 
 extern "C" nrv_status nrv_keys_flip_sign(uint64_t* key, int64_t n, nrv_stream stream) {
@@ -338,7 +339,7 @@ extern "C" nrv_status nrv_resolve_pack(nrv_scene* s, const nrv_view* view, const
     a.netin = netin;
     fill_pack(a, d, prec, inv);
     fill_derived(a, d, *view, s->d.d_xyz);
-    return launch_resolve(a, (cudaStream_t)stream);
+    return launch_resolve(&a, 1, (cudaStream_t)stream);
 }
 
 // --------------------------------------------------------------------- network
@@ -752,9 +753,10 @@ extern "C" nrv_status nrv_render_batch(nrv_scene* s, nrv_net* net, const nrv_pac
             NRV_TRY(launch_visibility(s->d.d_xyz, s->d.n_points, rv, q, views_dev,
                                       (uint32_t*)(base + tiles_off), s->chunks.p));
         if (ev) prof_mark(*ev, q);
+        ResolveArgs ra[8];
+        memset(ra, 0, sizeof(ra));
         for (int i = 0; i < n; ++i) {
-            ResolveArgs a;
-            memset(&a, 0, sizeof(a));
+            ResolveArgs& a = ra[i];
             a.key = reinterpret_cast<const unsigned long long*>(base + key_off[i]);
             a.attr = s->d.d_attr;
             a.base = (uint32_t)s->d.index_base;
@@ -770,8 +772,8 @@ extern "C" nrv_status nrv_render_batch(nrv_scene* s, nrv_net* net, const nrv_pac
             fill_derived(a, d, views[i], s->d.d_xyz);
             // replays take the cameras of the call from the device copy of the views
             if (views_dev) a.view_dev = &views_dev->v[i];
-            NRV_TRY(launch_resolve(a, q));
         }
+        NRV_TRY(launch_resolve(ra, n, q));
         if (ev) prof_mark(*ev, q);
         for (int g = 0; g < ngroups; ++g) {
             const int i0 = group_first[g];
