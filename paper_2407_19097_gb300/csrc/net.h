@@ -111,11 +111,19 @@ struct TcHead {
     RgbTab tab;      // per-image destinations (tab.on), else rgb + img * h * w_px * 3
 };
 
+// Conversions fused into a 3x3 conv at the borders of the mixed FP8 network (0: none):
+// pool_inv: the pool of a BF16 conv stored as E4M3 codes of mean * pool_inv; dec_scale: the
+// output of an E4M3 conv stored as BF16 of code * dec_scale.
+struct TcExtra {
+    float pool_inv, dec_scale;
+};
+
 // tensor-core convolution (tc.cu); returns NRV_ERR_UNSUPPORTED when a shape is not covered
 nrv_status tc_conv3(const Net* net, int layer, const void* x1, int c1, const void* x2, int c2,
                     void* y, const Geo& g, int level, nrv_prec prec, cudaStream_t s,
                     float inv_out = 1.0f, const TcHead* head = nullptr,
-                    void* pool_y = nullptr);   // pool_y: also the 2x2 average pool of y
+                    void* pool_y = nullptr,    // pool_y: also the 2x2 average pool of y
+                    const TcExtra* extra = nullptr);
 nrv_status tc_upconv(const Net* net, int layer, const void* x, void* y, const Geo& g, int level_in,
                      nrv_prec prec, cudaStream_t s, float inv_out = 1.0f);
 nrv_status tc_repack_fp8(Net* net, cudaStream_t s);

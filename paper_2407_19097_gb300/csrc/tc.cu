@@ -69,6 +69,7 @@
 #include <algorithm>
 
 #include "net.h"
+#include "project.cuh"
 #include "tcgen05.cuh"
 
 namespace nrv {
@@ -139,7 +140,11 @@ struct TcParams {
     int store_y;
     // optional 2x2 average pool of the stored output (mode 0, even h and w, two rows per
     // tile): row-planar [n][h/2][out_nch][w/2][16 bytes]
-    void* pool_y;            // (BF16 only)
+    void* pool_y;            // (E4M3 with row streaming only)
+    float pool_inv;          // row streaming, BF16: nonzero: the pool is stored as E4M3 codes of
+                             // mean * pool_inv, [n][h/2][out_nch / 2][w/2][16 bytes]
+    float dec_scale;         // row streaming, FP8: nonzero: the output is stored as BF16 of
+                             // code * dec_scale (a BF16 layer reads it)
     uint32_t stash_off;      // pool: shared-memory copy of the tile's even row as stored,
                              // [16-byte word][128 lanes][16 bytes], after the ring
     // Row streaming (mode 0): the weights of the three kernel rows side by side as B,
@@ -181,41 +186,6 @@ struct TileWalk {
                 ++img;
             }
         }
-    }
-};
-
-// Row streaming: the output row held by each ring slot in turn.  A CTA's run of tiles splits
-// into segments (one tile column each); a segment of R output rows streams R + 2 input rows,
-// and its slots hold output rows y0 - 2 .. y0 + R - 1, the first two belonging to no one.
-struct SlotCursor {
-    int t, seg_left, y0, r, img, x;
-    bool vx;
-    __device__ __forceinline__ void init(int t_begin) {
-        t = t_begin;
-        seg_left = 0;
-        y0 = r = img = x = 0;
-        vx = false;
-    }
-    __device__ __forceinline__ void next(const TcParams& P, int t_end, int m, bool& real, int& si,
-                                         int& sx, bool& sv, int& sy) {
-        if (seg_left == 0) {
-            const int col = t / P.hr;
-            const int te = t_end < (col + 1) * P.hr ? t_end : (col + 1) * P.hr;
-            y0 = (t - col * P.hr) * P.rpt;
-            seg_left = (te - t) * P.rpt + 2;
-            r = 0;
-            img = col / P.tiles_x;
-            x = (col - img * P.tiles_x) * P.tile_w + m;
-            vx = m < P.tile_w && x < P.w;
-            t = te;
-        }
-        real = r >= 2;
-        si = img;
-        sx = x;
-        sy = y0 + r - 2;
-        sv = vx && sy < P.h;
-        ++r;
-        --seg_left;
     }
 };
 
@@ -263,7 +233,10 @@ __device__ __forceinline__ void head_store(const TcParams& P, const float* hw, i
     }
 }
 
-template <bool FP8, bool STREAM, bool GATED>
+// What the row-streaming epilogue does besides storing (the tile form decides at run time).
+enum { EPI_PLAIN, EPI_POOL, EPI_HEAD };
+
+template <bool FP8, bool STREAM, bool GATED, int EPI>
 __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4)
     conv3_tc_kernel(const __grid_constant__ CUtensorMap tm1, const __grid_constant__ CUtensorMap tm2,
                     const __grid_constant__ TcParams P) {
@@ -275,6 +248,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
     __shared__ __align__(16) float bias_s[256];
     __shared__ __align__(16) float colscale_s[256];
     __shared__ __align__(16) float head_ws[52];
+    __shared__ __align__(16) float2 head_w2[EPI == EPI_HEAD ? 48 : 1];   // {w, w}
     __shared__ uint32_t alo_s[MAX_KS + 1];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
@@ -334,6 +308,10 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
     for (int i = threadIdx.x; i <= MAX_KS; i += NT) alo_s[i] = i < P.nks ? P.a_lo[i] : 0u;
     if (P.head_w && threadIdx.x < 51)
         head_ws[threadIdx.x] = threadIdx.x < 48 ? P.head_w[threadIdx.x] : P.head_b[threadIdx.x - 48];
+    if (EPI == EPI_HEAD && threadIdx.x < 48) {
+        const float w = P.head_w[threadIdx.x];
+        head_w2[threadIdx.x] = make_float2(w, w);
+    }
     if (warp == 1) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                          smem_u32(&tmem_slot)),
@@ -818,191 +796,18 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 }
             }
         };
-        // Two consecutive output rows of this thread's pixel from two TMEM blocks (BF16, not
-        // gated, row streaming): row a and row b, either absent (ra / rb false: a slot that
-        // holds no output row of this CTA) -- processed together, 8 output channels (one
-        // plane) at a time, so that the two rows' loads and arithmetic overlap.  With the
-        // fused pool the pair is an even and the following odd row, pooled from registers.
-        auto emit_pair = [&](uint32_t ta, bool ra, int imga, int xa, bool va, int ya, uint32_t tb,
-                             bool rb, int imgb, int xb, bool vb, int yb) {
-            // 8-output-channel chunks (one plane each); gated: features and gates of 8 channels
-            const int nchunk = GATED ? P.n_slice / 16 : P.n_slice / 8;
-            const int oc0 = (slice * P.n_slice) >> (GATED ? 1 : 0);   // first output channel
-            const int plane0 = oc0 / 8;                                    // (BF16 planes)
-            const size_t pstride = (size_t)P.w * 16;   // bytes between planes of a row
-            // this pixel's 16-byte word in plane 0 of rows a and b
-            uint8_t* const pya = (uint8_t*)P.y + (((size_t)imga * P.h + ya) * P.out_nch * P.w + xa) * 16;
-            uint8_t* const pyb = (uint8_t*)P.y + (((size_t)imgb * P.h + yb) * P.out_nch * P.w + xb) * 16;
-            const bool sa = P.store_y && ra && va, sb = P.store_y && rb && vb;
-            const bool relu = P.relu != 0;
-            const bool pool = P.pool_y && ra && rb;
-            const bool vp = va && vb;
-            float ha[3] = {0.0f, 0.0f, 0.0f}, hb[3] = {0.0f, 0.0f, 0.0f};
-            if (P.head_w) {
-#pragma unroll
-                for (int o = 0; o < 3; ++o) ha[o] = hb[o] = head_ws[48 + o];
-            }
-#pragma unroll 1
-            for (int ch = 0; ch < nchunk; ++ch) {
-                const int cf = GATED ? (ch >> 1) * 32 + (ch & 1) * 8 : ch * 8;
-                uint32_t fa[8], fb[8], ga[8], gb[8];
-                if (ra) tmem_ld8_nowait(ta + (uint32_t)cf, fa);
-                if (rb) tmem_ld8_nowait(tb + (uint32_t)cf, fb);
-                if (GATED) {
-                    if (ra) tmem_ld8_nowait(ta + (uint32_t)(cf + 16), ga);
-                    if (rb) tmem_ld8_nowait(tb + (uint32_t)(cf + 16), gb);
-                }
-                tmem_ld_wait();
-                tmem_tie8(fa);
-                tmem_tie8(fb);
-                if (GATED) {
-                    tmem_tie8(ga);
-                    tmem_tie8(gb);
-                }
-                const float4* b4 = reinterpret_cast<const float4*>(bias_s + cf);
-                const float4 bb0 = b4[0], bb1 = b4[1];
-                const float bq[8] = {bb0.x, bb0.y, bb0.z, bb0.w, bb1.x, bb1.y, bb1.z, bb1.w};
-                float gq[8];
-                if (GATED) {
-                    const float4 g0 = b4[4], g1 = b4[5];   // the gate columns' biases, 16 on
-                    gq[0] = g0.x; gq[1] = g0.y; gq[2] = g0.z; gq[3] = g0.w;
-                    gq[4] = g1.x; gq[5] = g1.y; gq[6] = g1.z; gq[7] = g1.w;
-                }
-                // scale, bias, activation and the stored form: BF16 pairs, or E4M3 codes of
-                // v / s_out (8 channels = 8 bytes, half of a 16-channel plane)
-                uint32_t pa[4], pb[4];
-                uint32_t qa[2] = {0u, 0u}, qb[2] = {0u, 0u};
-                if (FP8) {
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float sc = colscale_s[cf + j];
-                        float u = fmaf(__uint_as_float(fa[j]), sc, bq[j]);
-                        float w = fmaf(__uint_as_float(fb[j]), sc, bq[j]);
-                        if (relu) {
-                            u = fmaxf(u, 0.0f);
-                            w = fmaxf(w, 0.0f);
-                        }
-                        const uint32_t ca = __nv_cvt_float_to_fp8(u * P.inv_out, __NV_SATFINITE, __NV_E4M3);
-                        const uint32_t cb = __nv_cvt_float_to_fp8(w * P.inv_out, __NV_SATFINITE, __NV_E4M3);
-                        qa[j >> 2] |= ca << (8 * (j & 3));
-                        qb[j >> 2] |= cb << (8 * (j & 3));
-                    }
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        float u0 = __uint_as_float(fa[2 * j]) + bq[2 * j];
-                        float u1 = __uint_as_float(fa[2 * j + 1]) + bq[2 * j + 1];
-                        float w0 = __uint_as_float(fb[2 * j]) + bq[2 * j];
-                        float w1 = __uint_as_float(fb[2 * j + 1]) + bq[2 * j + 1];
-                        if (GATED) {
-                            // ELU(f) * sigmoid(g), as in the per-row epilogue
-                            auto gate = [](float f, float g) {
-                                const float e = __expf(fminf(f, 0.0f));
-                                return __fdividef(f > 0.0f ? f : e - 1.0f, 1.0f + __expf(-g));
-                            };
-                            u0 = gate(u0, __uint_as_float(ga[2 * j]) + gq[2 * j]);
-                            u1 = gate(u1, __uint_as_float(ga[2 * j + 1]) + gq[2 * j + 1]);
-                            w0 = gate(w0, __uint_as_float(gb[2 * j]) + gq[2 * j]);
-                            w1 = gate(w1, __uint_as_float(gb[2 * j + 1]) + gq[2 * j + 1]);
-                        }
-                        if (!GATED && relu) {
-                            pa[j] = bf16x2_relu(u0, u1);
-                            pb[j] = bf16x2_relu(w0, w1);
-                        } else {
-                            pa[j] = bf16x2(u0, u1);
-                            pb[j] = bf16x2(w0, w1);
-                        }
-                    }
-                }
-                if (FP8) {
-                    const int oc = oc0 + 8 * ch;
-                    const size_t poff = (size_t)(oc / 16) * pstride + (size_t)(oc & 15);
-                    if (sa) *reinterpret_cast<uint2*>(pya + poff) = make_uint2(qa[0], qa[1]);
-                    if (sb) *reinterpret_cast<uint2*>(pyb + poff) = make_uint2(qb[0], qb[1]);
-                } else {
-                    const size_t poff = (size_t)(plane0 + ch) * pstride;
-                    if (sa) *reinterpret_cast<uint4*>(pya + poff) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
-                    if (sb) *reinterpret_cast<uint4*>(pyb + poff) = make_uint4(pb[0], pb[1], pb[2], pb[3]);
-                }
-                if (P.head_w || pool) {
-                    // the values as stored (BF16-rounded, or E4M3 decoded), for the head and pool
-                    float a8[8], b8[8];
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (FP8) {
-                            __nv_fp8_e4m3 x8, y8;
-                            x8.__x = (uint8_t)(qa[j >> 2] >> (8 * (j & 3)));
-                            y8.__x = (uint8_t)(qb[j >> 2] >> (8 * (j & 3)));
-                            a8[j] = float(x8) * P.head_s;
-                            b8[j] = float(y8) * P.head_s;
-                        } else {
-                            const __nv_bfloat162 x2 = *reinterpret_cast<const __nv_bfloat162*>(&pa[j >> 1]);
-                            const __nv_bfloat162 y2 = *reinterpret_cast<const __nv_bfloat162*>(&pb[j >> 1]);
-                            a8[j] = (j & 1) ? __high2float(x2) : __low2float(x2);
-                            b8[j] = (j & 1) ? __high2float(y2) : __low2float(y2);
-                        }
-                    }
-                    if (P.head_w) {
-                        // the 1x1 head: channels in order, one fused multiply-add each
-#pragma unroll
-                        for (int o = 0; o < 3; ++o) {
-                            const float4* h4 =
-                                reinterpret_cast<const float4*>(head_ws + o * 16 + 8 * ch);
-                            const float4 w0 = h4[0], w1 = h4[1];
-                            const float wq[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w};
-#pragma unroll
-                            for (int j = 0; j < 8; ++j) {
-                                ha[o] = fmaf(wq[j], a8[j], ha[o]);
-                                hb[o] = fmaf(wq[j], b8[j], hb[o]);
-                            }
-                        }
-                    }
-                    if (pool) {
-                        // 2x2 average of rows a (even) and b (odd), pixels x and x + 1 (next lane)
-                        float rr[8];
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            const float av = vp ? a8[j] : 0.0f, cv = vp ? b8[j] : 0.0f;
-                            const float bv = __shfl_down_sync(0xffffffffu, av, 1);
-                            const float dv = __shfl_down_sync(0xffffffffu, cv, 1);
-                            rr[j] = 0.25f * ((av + bv) + (cv + dv));
-                        }
-                        if (vp && !(m & 1)) {
-                            uint32_t pk[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                __nv_bfloat162 h2 = __floats2bfloat162_rn(rr[2 * j], rr[2 * j + 1]);
-                                pk[j] = *reinterpret_cast<uint32_t*>(&h2);
-                            }
-                            const int wp = P.w >> 1;
-                            *reinterpret_cast<uint4*>((uint8_t*)P.pool_y +
-                                ((((size_t)imga * (P.h >> 1) + (ya >> 1)) * P.out_nch + plane0 + ch) *
-                                     wp + (xa >> 1)) * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        }
-                    }
-                }
-            }
-            if (P.head_w) {
-                if (ra && va && ya < P.rgb_h && xa < P.rgb_w) {
-                    float* out = rgb_image(P.rgb, P.rgb_tab, (size_t)imga, (size_t)P.rgb_h * P.rgb_w) +
-                                 ((size_t)ya * P.rgb_w + xa) * 3;
-                    out[0] = ha[0];
-                    out[1] = ha[1];
-                    out[2] = ha[2];
-                }
-                if (rb && vb && yb < P.rgb_h && xb < P.rgb_w) {
-                    float* out = rgb_image(P.rgb, P.rgb_tab, (size_t)imgb, (size_t)P.rgb_h * P.rgb_w) +
-                                 ((size_t)yb * P.rgb_w + xb) * 3;
-                    out[0] = hb[0];
-                    out[1] = hb[1];
-                    out[2] = hb[2];
-                }
-            }
-        };
-        if (STREAM) {
-            // the issuer's slot sequence: slot q is final once group q / grp has committed;
-            // slots 0 and 1 of a segment hold the two rows above it (not its own rows)
+        if constexpr (STREAM) {
+            // Row streaming.  The issuer's slot sequence: slot q is final once group q / grp has
+            // committed; a segment of R output rows (one tile column) has R + 2 slots, the first
+            // two belonging to no one.  Two groups of epilogue warps (2-5 and 6-9) take alternate
+            // slot groups, two rows (adjacent TMEM blocks) and 16 columns at a time.
+            //
+            // This loop paces the narrow layers (level 0: about 450 of the 500 cycles that an SM
+            // has per 128-pixel row), so the row cursor only adds, each fused operation is
+            // compiled on its own (EPI), a block is zeroed as soon as its loads have landed, and
+            // biases, sums and the head run on pairs of channels or rows (f32x2).
             const uint32_t lanes = (uint32_t)(32 * q) << 16;
+            const uint32_t ns = (uint32_t)P.n_slice;
             int S = 0;
             for (int tt = t_begin; tt < t_end;) {
                 const int col = tt / P.hr;
@@ -1010,21 +815,291 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 S += (te - tt) * P.rpt + 2;
                 tt = te;
             }
-            SlotCursor cur;
-            cur.init(t_begin);
-            // two groups of epilogue warps (2-5 and 6-9) take alternate slot groups
+            const int oc0 = (slice * P.n_slice) >> (GATED ? 1 : 0);   // first output channel
+            const bool dec = FP8 && P.dec_scale != 0.0f;                // BF16 output of an FP8 layer
+            const int nch = dec ? 2 * P.out_nch : P.out_nch;            // planes of the stored output
+            const size_t pstride = (size_t)P.w * 16;                    // bytes between planes of a row
+            const size_t rstride = pstride * nch;                       // and between rows
+            const int plane0 = oc0 / (FP8 && !dec ? 16 : 8);
+            // the cursor: segment, row and this thread's word of plane0 in that row
+            int ct = t_begin, left = 0, r = 0, y = 0, img = 0, x = 0;
+            bool vx = false;
+            uint8_t* py = nullptr;
+            auto segment = [&]() {
+                const int col = ct / P.hr;
+                const int te = t_end < (col + 1) * P.hr ? t_end : (col + 1) * P.hr;
+                y = (ct - col * P.hr) * P.rpt - 2;
+                left = (te - ct) * P.rpt + 2;
+                r = 0;
+                img = col / P.tiles_x;
+                x = (col - img * P.tiles_x) * P.tile_w + m;
+                vx = m < P.tile_w && x < P.w;
+                py = (uint8_t*)P.y + (size_t)img * P.h * rstride + plane0 * pstride + (size_t)x * 16 +
+                     (long long)y * (long long)rstride;
+                ct = te;
+            };
+            auto skip = [&](int cnt) {
+                while (cnt > 0) {
+                    if (left == 0) segment();
+                    const int k = cnt < left ? cnt : left;
+                    y += k;
+                    r += k;
+                    py += (size_t)k * rstride;
+                    left -= k;
+                    cnt -= k;
+                }
+            };
+            struct Row {
+                bool real, st;     // an output row of this CTA; and this thread's pixel exists
+                uint8_t* p;
+                int img, x, y;
+            };
+            auto next = [&]() {
+                if (left == 0) segment();
+                const Row o{r >= 2, r >= 2 && vx && y < P.h, py, img, x, y};
+                ++y;
+                ++r;
+                py += rstride;
+                --left;
+                return o;
+            };
+            // head sums {row a, row b} per colour
+            f2 hs[3] = {0ull, 0ull, 0ull};
+            // v: the stored values {row a, row b} of channel c
+            auto head_add = [&](int c, f2 v) {
+#pragma unroll
+                for (int o = 0; o < 3; ++o)
+                    hs[o] = f2_fma(*reinterpret_cast<const f2*>(&head_w2[o * 16 + c]), v, hs[o]);
+            };
+            // pooled means of channels 2j, 2j + 1 from this pixel's and the next lane's BF16 pairs
+            auto pool_pair = [&](uint32_t a, uint32_t b) -> f2 {
+                const uint32_t na = __shfl_down_sync(0xffffffffu, a, 1), nb = __shfl_down_sync(0xffffffffu, b, 1);
+                auto up = [](uint32_t w) { return f2_pack(__uint_as_float(w << 16), __uint_as_float(w & 0xFFFF0000u)); };
+                return f2_mul(f2_add(f2_add(up(a), up(na)), f2_add(up(b), up(nb))), f2_pack(0.25f, 0.25f));
+            };
+            // Eight output channels of rows a and b as BF16 pairs in plane k of the slice: store,
+            // and the head or the pool of the values as stored.
+            auto finish8 = [&](const Row& ra, const Row& rb, bool sa, bool sb, int k, const uint32_t* pa,
+                               const uint32_t* pb, float* mean) {
+                if (sa) *reinterpret_cast<uint4*>(ra.p + k * pstride) = make_uint4(pa[0], pa[1], pa[2], pa[3]);
+                if (sb) *reinterpret_cast<uint4*>(rb.p + k * pstride) = make_uint4(pb[0], pb[1], pb[2], pb[3]);
+                if (EPI == EPI_HEAD) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        head_add(8 * k + 2 * j, f2_pack(__uint_as_float(pa[j] << 16), __uint_as_float(pb[j] << 16)));
+                        head_add(8 * k + 2 * j + 1, f2_pack(__uint_as_float(pa[j] & 0xFFFF0000u),
+                                                            __uint_as_float(pb[j] & 0xFFFF0000u)));
+                    }
+                }
+                if (EPI == EPI_POOL)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) f2_unpack(pool_pair(pa[j], pb[j]), mean[2 * j], mean[2 * j + 1]);
+            };
+            // this thread's word of pooled plane 0 of the slice, for the row pair's output row
+            auto pool_word = [&](const Row& ra, int planes, int pl) {
+                const size_t wp = (size_t)(P.w >> 1);
+                return (uint8_t*)P.pool_y +
+                       ((((size_t)ra.img * (P.h >> 1) + (ra.y >> 1)) * planes + pl) * wp + (ra.x >> 1)) * 16;
+            };
+            auto codes4 = [](const float* v) -> uint32_t {   // four E4M3 codes
+                const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(v[0], v[1]), __NV_SATFINITE, __NV_E4M3);
+                const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(v[2], v[3]), __NV_SATFINITE, __NV_E4M3);
+                return lo | (hi << 16);
+            };
+            auto decode4 = [](uint32_t w, float* v) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const __half2 d = __half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)(w >> (16 * h)), __NV_E4M3));
+                    const float2 f = __half22float2(d);
+                    v[2 * h] = f.x;
+                    v[2 * h + 1] = f.y;
+                }
+            };
+            // sixteen columns from c0 on of the blocks at ta (row a) and ta + ns (row b)
+            auto unit = [&](uint32_t ta, int c0, const Row& ra, const Row& rb) {
+                const bool sa = ra.st && (EPI != EPI_HEAD || P.store_y), sb = rb.st && (EPI != EPI_HEAD || P.store_y);
+                const bool pool = EPI == EPI_POOL && ra.st && rb.st && !(m & 1);
+                if constexpr (GATED) {
+                    // columns c0 .. c0 + 15: features, the next 16 their gates (c0 steps by 32)
+#pragma unroll 1
+                    for (int h = 0; h < 2; ++h) {
+                        const int cf = c0 + 8 * h, k = c0 / 16 + h;
+                        uint32_t fa[8], fb[8], ga[8], gb[8];
+                        tmem_ld8_nowait(ta + (uint32_t)cf, fa);
+                        tmem_ld8_nowait(ta + ns + (uint32_t)cf, fb);
+                        tmem_ld8_nowait(ta + (uint32_t)(cf + 16), ga);
+                        tmem_ld8_nowait(ta + ns + (uint32_t)(cf + 16), gb);
+                        tmem_ld_wait();
+                        tmem_tie8(fa);
+                        tmem_tie8(fb);
+                        tmem_tie8(ga);
+                        tmem_tie8(gb);
+                        const float4* b4 = reinterpret_cast<const float4*>(bias_s + cf);
+                        const float4 f0 = b4[0], f1 = b4[1], g0 = b4[4], g1 = b4[5];
+                        const float bq[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+                        const float gq[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+                        // ELU(f) * sigmoid(g), as in the per-row epilogue
+                        auto gate = [](float f, float g) {
+                            const float e = __expf(fminf(f, 0.0f));
+                            return __fdividef(f > 0.0f ? f : e - 1.0f, 1.0f + __expf(-g));
+                        };
+                        uint32_t pa[4], pb[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            float u[2], w[2];
+#pragma unroll
+                            for (int e = 0; e < 2; ++e) {
+                                const int i = 2 * j + e;
+                                u[e] = gate(__uint_as_float(fa[i]) + bq[i], __uint_as_float(ga[i]) + gq[i]);
+                                w[e] = gate(__uint_as_float(fb[i]) + bq[i], __uint_as_float(gb[i]) + gq[i]);
+                            }
+                            pa[j] = bf16x2(u[0], u[1]);
+                            pb[j] = bf16x2(w[0], w[1]);
+                        }
+                        float mean[8];
+                        finish8(ra, rb, sa, sb, k, pa, pb, mean);
+                        if (EPI == EPI_POOL && pool) {
+                            uint32_t pk[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) pk[j] = bf16x2(mean[2 * j], mean[2 * j + 1]);
+                            *reinterpret_cast<uint4*>(pool_word(ra, P.out_nch, plane0 + k)) =
+                                make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                        }
+                    }
+                    tmem_zero16(ta + (uint32_t)c0);
+                    tmem_zero16(ta + (uint32_t)(c0 + 16));
+                    tmem_zero16(ta + ns + (uint32_t)c0);
+                    tmem_zero16(ta + ns + (uint32_t)(c0 + 16));
+                } else {
+                    uint32_t fa[16], fb[16];
+                    tmem_ld16_nowait(ta + (uint32_t)c0, fa);
+                    tmem_ld16_nowait(ta + ns + (uint32_t)c0, fb);
+                    tmem_ld_wait();
+                    tmem_tie8(fa);
+                    tmem_tie8(fa + 8);
+                    tmem_tie8(fb);
+                    tmem_tie8(fb + 8);
+                    tmem_zero16(ta + (uint32_t)c0);   // for their next output rows
+                    tmem_zero16(ta + ns + (uint32_t)c0);
+                    const f2* b2 = reinterpret_cast<const f2*>(bias_s + c0);
+                    auto pair = [](const uint32_t* f, int j) {
+                        return f2_pack(__uint_as_float(f[2 * j]), __uint_as_float(f[2 * j + 1]));
+                    };
+                    if constexpr (!FP8) {
+                        uint32_t pa[8], pb[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            float u0, u1, w0, w1;
+                            f2_unpack(f2_add(pair(fa, j), b2[j]), u0, u1);
+                            f2_unpack(f2_add(pair(fb, j), b2[j]), w0, w1);
+                            pa[j] = bf16x2_relu(u0, u1);
+                            pb[j] = bf16x2_relu(w0, w1);
+                        }
+                        const int k = c0 / 8;
+                        float mean[16];
+                        finish8(ra, rb, sa, sb, k, pa, pb, mean);
+                        finish8(ra, rb, sa, sb, k + 1, pa + 4, pb + 4, mean + 8);
+                        if (EPI == EPI_POOL && pool) {
+                            if (P.pool_inv != 0.0f) {
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) mean[j] *= P.pool_inv;
+                                *reinterpret_cast<uint4*>(pool_word(ra, P.out_nch / 2, (plane0 + k) / 2)) =
+                                    make_uint4(codes4(mean), codes4(mean + 4), codes4(mean + 8), codes4(mean + 12));
+                            } else {
+                                uint32_t pk[8];
+#pragma unroll
+                                for (int j = 0; j < 8; ++j) pk[j] = bf16x2(mean[2 * j], mean[2 * j + 1]);
+                                uint8_t* d = pool_word(ra, P.out_nch, plane0 + k);
+                                *reinterpret_cast<uint4*>(d) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                                *reinterpret_cast<uint4*>(d + (size_t)(P.w >> 1) * 16) =
+                                    make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                            }
+                        }
+                    } else {
+                        // acc * scale + bias, ReLU, and the E4M3 code of that / s_out
+                        const f2* s2 = reinterpret_cast<const f2*>(colscale_s + c0);
+                        const f2 inv = f2_pack(P.inv_out, P.inv_out);
+                        uint32_t qa[4], qb[4];
+#pragma unroll
+                        for (int g = 0; g < 4; ++g) {
+                            float u[4], w[4];
+#pragma unroll
+                            for (int j = 0; j < 2; ++j) {
+                                float u0, u1, w0, w1;
+                                f2_unpack(f2_fma(pair(fa, 2 * g + j), s2[2 * g + j], b2[2 * g + j]), u0, u1);
+                                f2_unpack(f2_fma(pair(fb, 2 * g + j), s2[2 * g + j], b2[2 * g + j]), w0, w1);
+                                f2_unpack(f2_mul(f2_pack(fmaxf(u0, 0.0f), fmaxf(u1, 0.0f)), inv), u[2 * j], u[2 * j + 1]);
+                                f2_unpack(f2_mul(f2_pack(fmaxf(w0, 0.0f), fmaxf(w1, 0.0f)), inv), w[2 * j], w[2 * j + 1]);
+                            }
+                            qa[g] = codes4(u);
+                            qb[g] = codes4(w);
+                        }
+                        const int k = c0 / 16;
+                        if (dec) {
+                            // BF16 of the decoded codes, two planes
+                            auto put = [&](uint8_t* d, const uint32_t* qc) {
+                                uint32_t pk[8];
+#pragma unroll
+                                for (int g = 0; g < 4; ++g) {
+                                    float v[4];
+                                    decode4(qc[g], v);
+                                    pk[2 * g] = bf16x2(v[0] * P.dec_scale, v[1] * P.dec_scale);
+                                    pk[2 * g + 1] = bf16x2(v[2] * P.dec_scale, v[3] * P.dec_scale);
+                                }
+                                *reinterpret_cast<uint4*>(d + (size_t)(2 * k) * pstride) =
+                                    make_uint4(pk[0], pk[1], pk[2], pk[3]);
+                                *reinterpret_cast<uint4*>(d + (size_t)(2 * k + 1) * pstride) =
+                                    make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                            };
+                            if (sa) put(ra.p, qa);
+                            if (sb) put(rb.p, qb);
+                        } else {
+                            if (sa) *reinterpret_cast<uint4*>(ra.p + k * pstride) = make_uint4(qa[0], qa[1], qa[2], qa[3]);
+                            if (sb) *reinterpret_cast<uint4*>(rb.p + k * pstride) = make_uint4(qb[0], qb[1], qb[2], qb[3]);
+                        }
+                        if (EPI == EPI_HEAD) {
+                            // the decoded codes, as a separate head kernel would read them
+#pragma unroll
+                            for (int g = 0; g < 4; ++g) {
+                                float u[4], w[4];
+                                decode4(qa[g], u);
+                                decode4(qb[g], w);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+                                    head_add(4 * g + j, f2_pack(u[j] * P.head_s, w[j] * P.head_s));
+                            }
+                        }
+                        if (EPI == EPI_POOL) {
+                            uint32_t pq[4];
+#pragma unroll
+                            for (int g = 0; g < 4; ++g) {
+                                const uint32_t na = __shfl_down_sync(0xffffffffu, qa[g], 1);
+                                const uint32_t nb = __shfl_down_sync(0xffffffffu, qb[g], 1);
+                                float u[4], un[4], w[4], wn[4], mean[4];
+                                decode4(qa[g], u);
+                                decode4(na, un);
+                                decode4(qb[g], w);
+                                decode4(nb, wn);
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) mean[j] = 0.25f * ((u[j] + un[j]) + (w[j] + wn[j]));
+                                pq[g] = codes4(mean);
+                            }
+                            if (pool)
+                                *reinterpret_cast<uint4*>(pool_word(ra, P.out_nch, plane0 + k)) =
+                                    make_uint4(pq[0], pq[1], pq[2], pq[3]);
+                        }
+                    }
+                }
+            };
             const int wg = warp >= 6 ? 1 : 0;
             int blk = 0, k = 0;
             for (int q0 = 0; q0 < S; q0 += P.grp, ++k) {
+                const int cnt = S - q0 < P.grp ? S - q0 : P.grp;
+                const int blk0 = blk;
+                blk += P.grp;
+                if (blk >= P.nb) blk -= P.nb;
                 if ((k & 1) != wg) {
-                    // the other warp group's slots: step the cursor and the ring past them
-                    const int qe = q0 + P.grp < S ? q0 + P.grp : S;
-                    for (int qq = q0; qq < qe; ++qq) {
-                        bool rr = false, vv = false;
-                        int ii = 0, xx = 0, yy = 0;
-                        cur.next(P, t_end, m, rr, ii, xx, vv, yy);
-                        if (++blk == P.nb) blk = 0;
-                    }
+                    skip(cnt);
                     continue;
                 }
                 int okw = 1;
@@ -1033,27 +1108,37 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 okw = __shfl_sync(0xffffffffu, okw, 0);
                 if (!okw) break;
                 tc_fence_after();
-                const int qe = q0 + P.grp < S ? q0 + P.grp : S;
-                for (int qq = q0; qq < qe; qq += 2) {
-                    bool ra = false, rb = false, va = false, vb = false;
-                    int ia = 0, xa = 0, ya = 0, ib = 0, xb = 0, yb = 0;
-                    cur.next(P, t_end, m, ra, ia, xa, va, ya);
-                    const uint32_t ta = tmem + lanes + (uint32_t)(blk * P.n_slice);
-                    if (++blk == P.nb) blk = 0;
-                    const bool hasb = qq + 1 < qe;
-                    uint32_t tb = ta;
-                    if (hasb) {
-                        cur.next(P, t_end, m, rb, ib, xb, vb, yb);
-                        tb = tmem + lanes + (uint32_t)(blk * P.n_slice);
-                        if (++blk == P.nb) blk = 0;
+                int bl = blk0;
+                for (int i = 0; i < cnt; i += 2) {
+                    const Row ra = next();
+                    Row rb{false, false, nullptr, 0, 0, 0};
+                    if (i + 1 < cnt) rb = next();
+                    const uint32_t ta = tmem + lanes + (uint32_t)bl * ns;
+                    bl += 2;
+                    if (bl >= P.nb) bl -= P.nb;
+                    if (EPI == EPI_HEAD) {
+#pragma unroll
+                        for (int o = 0; o < 3; ++o) hs[o] = f2_pack(head_ws[48 + o], head_ws[48 + o]);
                     }
-                    emit_pair(ta, ra, ia, xa, va, ya, tb, rb, ib, xb, vb, yb);
-                    // zero the blocks for their next output rows
-                    for (int c = 0; c < P.n_slice; c += 16) tmem_zero16(ta + (uint32_t)c);
-                    if (hasb)
-                        for (int c = 0; c < P.n_slice; c += 16) tmem_zero16(tb + (uint32_t)c);
+#pragma unroll 1
+                    for (int c0 = 0; c0 < (int)ns; c0 += GATED ? 32 : 16) unit(ta, c0, ra, rb);
+                    if (EPI == EPI_HEAD) {
+                        float va[3], vb[3];
+#pragma unroll
+                        for (int o = 0; o < 3; ++o) f2_unpack(hs[o], va[o], vb[o]);
+                        auto rgb = [&](const Row& w, const float* v) {
+                            if (!w.st || w.y >= P.rgb_h || w.x >= P.rgb_w) return;
+                            float* out = rgb_image(P.rgb, P.rgb_tab, (size_t)w.img, (size_t)P.rgb_h * P.rgb_w) +
+                                         ((size_t)w.y * P.rgb_w + w.x) * 3;
+                            out[0] = v[0];
+                            out[1] = v[1];
+                            out[2] = v[2];
+                        };
+                        rgb(ra, va);
+                        rgb(rb, vb);
+                    }
                 }
-                if (qe - q0 == P.grp) {
+                if (cnt == P.grp) {
                     tmem_st_wait();
                     tc_fence_before();
                     __syncwarp();
@@ -1662,7 +1747,7 @@ static nrv_status tc_launch(const Net* net, const TcLayerCfg& c, const uint8_t* 
                             int c1, const void* x2, int c2, void* y, int n, int H, int W,
                             cudaStream_t s, int fp8, float inv_out, const TcHead* head = nullptr,
                             void* pool_y = nullptr, int g_ld = 0, int g_off = 0,
-                            const float* bias2 = nullptr) {
+                            const float* bias2 = nullptr, const TcExtra* extra = nullptr) {
     if (!c.ok || c.c1 != c1 || c.c2 != c2) return fail(NRV_ERR_UNSUPPORTED, "layer not configured");
     if (fp8 && !net->fp8_ready) return fail(NRV_ERR_STATE, "FP8 needs activation scales");
     if (n <= 0 || H <= 0 || W <= 0) return fail(NRV_ERR_ARG, "empty tensor");
@@ -1729,24 +1814,30 @@ static nrv_status tc_launch(const Net* net, const TcLayerCfg& c, const uint8_t* 
         while (cols < need) cols *= 2;
         return cols;
     };
-    // kernel variant: operand type, row streaming, gated epilogue (BF16 only)
-    const int kv = fp8 ? 4 + P.stream : 2 * P.stream + (P.gated ? 1 : 0);
-    auto kern = fp8 ? (P.stream ? conv3_tc_kernel<true, true, false>
-                                : conv3_tc_kernel<true, false, false>)
-                    : (P.stream ? (P.gated ? conv3_tc_kernel<false, true, true>
-                                           : conv3_tc_kernel<false, true, false>)
-                                : (P.gated ? conv3_tc_kernel<false, false, true>
-                                           : conv3_tc_kernel<false, false, false>));
-    static bool attr_set[6] = {false, false, false, false, false, false};
+    // kernel variant: operand type, row streaming (with what its epilogue fuses), gated (BF16 only)
+    const int epi = !P.stream ? EPI_PLAIN : head ? EPI_HEAD : pool_y ? EPI_POOL : EPI_PLAIN;
+    typedef void (*Kern)(CUtensorMap, CUtensorMap, TcParams);
+    static const Kern kerns[12] = {
+        conv3_tc_kernel<false, false, false, EPI_PLAIN>, conv3_tc_kernel<true, false, false, EPI_PLAIN>,
+        conv3_tc_kernel<false, false, true, EPI_PLAIN>,
+        conv3_tc_kernel<false, true, false, EPI_PLAIN>, conv3_tc_kernel<false, true, false, EPI_POOL>,
+        conv3_tc_kernel<false, true, false, EPI_HEAD>,
+        conv3_tc_kernel<true, true, false, EPI_PLAIN>, conv3_tc_kernel<true, true, false, EPI_POOL>,
+        conv3_tc_kernel<true, true, false, EPI_HEAD>,
+        conv3_tc_kernel<false, true, true, EPI_PLAIN>, conv3_tc_kernel<false, true, true, EPI_POOL>,
+        conv3_tc_kernel<false, true, true, EPI_HEAD>};
+    const int kv = !P.stream ? (fp8 ? 1 : P.gated ? 2 : 0) : (fp8 ? 6 : P.gated ? 9 : 3) + epi;
+    const Kern kern = kerns[kv];
+    static bool attr_set[12] = {};
     if (!attr_set[kv]) {
         NRV_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                             220 * 1024));
         attr_set[kv] = true;
     }
     // resident CTAs per SM from registers, threads, shared memory and TMEM columns
-    static cudaFuncAttributes fa_k[6];
+    static cudaFuncAttributes fa_k[12];
     static cudaDeviceProp prop;
-    static bool have_fa[6] = {false, false, false, false, false, false}, have_prop = false;
+    static bool have_fa[12] = {}, have_prop = false;
     if (!have_prop) {
         int dev = 0;
         NRV_CHECK_CUDA(cudaGetDevice(&dev));
@@ -1774,8 +1865,8 @@ static nrv_status tc_launch(const Net* net, const TcLayerCfg& c, const uint8_t* 
     // when the 2x2 pool is fused, whose row pairs a tile then holds), two accumulator buffers,
     // two ring rows of read-ahead -- one where that admits more CTAs per SM (BF16) -- and then
     // as many more as keep that occupancy, within 215 KB.
-    // pool: one 16-byte word per 16 stored bytes of a lane, 128 lanes
-    const uint32_t stash_bytes = pool_y ? (uint32_t)(c.n_slice * es / 16) * TILE_M * 16 : 0u;
+    // pool (tile form): one 16-byte word per 16 stored bytes of a lane, 128 lanes
+    const uint32_t stash_bytes = pool_y && !P.stream ? (uint32_t)(c.n_slice * es / 16) * TILE_M * 16 : 0u;
     auto smem_for = [&](int ns) { return P.w_region + (uint32_t)ns * P.slot_bytes + stash_bytes; };
     const int rpt0 = pool_y ? 2 : 1, nacc0 = 2;
     const uint32_t cols0 = cols_for(rpt0, nacc0);
@@ -1808,10 +1899,18 @@ static nrv_status tc_launch(const Net* net, const TcLayerCfg& c, const uint8_t* 
     P.inv_out = inv_out;
     P.store_y = 1;
     if (pool_y) {
-        if (!conv || fp8 || (H & 1) || (W & 1) || mask || head)
+        if (!conv || (fp8 && !P.stream) || (H & 1) || (W & 1) || mask || head)
             return fail(NRV_ERR_UNSUPPORTED, "the fused pool needs a 3x3 conv on an even grid");
         P.pool_y = pool_y;
     }
+    if (extra) {
+        if (!P.stream || (extra->pool_inv != 0.0f && (fp8 || P.gated || !pool_y || P.out_nch % 2)) ||
+            (extra->dec_scale != 0.0f && (!fp8 || epi != EPI_PLAIN)))
+            return fail(NRV_ERR_UNSUPPORTED, "conversion fused into a 3x3 conv");
+        P.pool_inv = extra->pool_inv;
+        P.dec_scale = extra->dec_scale;
+    }
+    if (P.stream && !P.gated && !relu) return fail(NRV_ERR_UNSUPPORTED, "row streaming applies ReLU");
     if (head) {
         if (!conv || c.nslices != 1 || c.n_slice != (c.gated ? 32 : 16) || cout != 16 ||
             !(relu || c.gated))
@@ -2100,7 +2199,7 @@ nrv_status tc_generic_run(const TcPacked* st, int l, const float* params, const 
 
 nrv_status tc_conv3(const Net* net, int l, const void* x1, int c1, const void* x2, int c2, void* y,
                     const Geo& g, int level, nrv_prec prec, cudaStream_t s, float inv_out,
-                    const TcHead* head, void* pool_y) {
+                    const TcHead* head, void* pool_y, const TcExtra* extra) {
     if (prec != NRV_PREC_BF16 && prec != NRV_PREC_FP8_E4M3)
         return fail(NRV_ERR_UNSUPPORTED, "tensor-core path is BF16 or FP8");
     const Layer& L = net->layers[l];
@@ -2109,7 +2208,7 @@ nrv_status tc_conv3(const Net* net, int l, const void* x1, int c1, const void* x
     const TcLayerCfg& c = g_cfg[fp8][l];
     const uint8_t* w = (const uint8_t*)(fp8 ? net->wfp8.p : net->wbf16.p) + c.w_off;
     return tc_launch(net, c, w, (const float*)net->params.p + L.boff, 1, nullptr, L.cout, x1, c1,
-                     x2, c2, y, g.n, g.h[level], g.w[level], s, fp8, inv_out, head, pool_y);
+                     x2, c2, y, g.n, g.h[level], g.w[level], s, fp8, inv_out, head, pool_y, 0, 0, nullptr, extra);
 }
 
 nrv_status tc_dgrad(const Net* net, int l, const void* gin, void* out, const void* mask, int n, int H,
