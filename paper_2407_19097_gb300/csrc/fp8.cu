@@ -189,6 +189,25 @@ nrv_status net_calibrate(Net* net, const void* netin, int n, int H, int W, cudaS
     return NRV_OK;
 }
 
+// An E4M3 3x3 conv and the pool of its output to the next level, in the conv's epilogue where
+// the conv streams its rows, else by a kernel of its own.
+static nrv_status fp8_conv_pool(Net* net, int l, int in, int c1, int out, int level, int pooled,
+                                cudaStream_t s) {
+    const Geo& g = net->geo;
+    auto A = [&](int a) { return (uint8_t*)net->acts.p + net->act_off[a]; };
+    const float inv = 1.0f / net->act_scale[1 + out];
+    const nrv_status st = tc_conv3(net, l, A(in), c1, nullptr, 0, A(out), g, level, NRV_PREC_FP8_E4M3, s, inv,
+                                   nullptr, A(pooled));
+    if (st != NRV_ERR_UNSUPPORTED) return st;
+    clear_error();
+    NRV_TRY(tc_conv3(net, l, A(in), c1, nullptr, 0, A(out), g, level, NRV_PREC_FP8_E4M3, s, inv));
+    const int c = net->act_c[out];
+    pool2_fp8_kernel<<<blocks_for(g.px(level + 1) * c / 16), 256, 0, s>>>(A(out), A(pooled), c, g.n,
+                                                                        g.h[level + 1], g.w[level + 1]);
+    NRV_CHECK_LAUNCH();
+    return NRV_OK;
+}
+
 nrv_status forward_fp8(Net* net, const uint8_t* netin, float* rgb, cudaStream_t s, bool keep_acts) {
     if (!net->fp8_ready) return fail(NRV_ERR_STATE, "FP8 needs activation scales (calibrate first)");
     const Geo& g = net->geo;
@@ -199,22 +218,13 @@ nrv_status forward_fp8(Net* net, const uint8_t* netin, float* rgb, cudaStream_t 
         net->backend[l] = 1;
         return tc_conv3(net, l, x1, c1, x2, c2, A(out), g, level, NRV_PREC_FP8_E4M3, s, inv(out));
     };
-    auto pool = [&](int in, int out, int level_out) -> nrv_status {
-        const int c = net->act_c[in];
-        pool2_fp8_kernel<<<blocks_for(g.px(level_out) * c / 16), 256, 0, s>>>(
-            A(in), A(out), c, g.n, g.h[level_out], g.w[level_out]);
-        NRV_CHECK_LAUNCH();
-        return NRV_OK;
-    };
     auto up = [&](int l, int in, int out, int level_in) -> nrv_status {
         net->backend[l] = 1;
         return tc_upconv(net, l, A(in), A(out), g, level_in, NRV_PREC_FP8_E4M3, s, inv(out));
     };
-    // a 3x3 conv and the pool of its output to the next level (separate kernels: at level 0
-    // the FP8 epilogue is the bottleneck and a fused pool measured slower)
     auto conv_pool = [&](int l, int in, int c1, int out, int level, int pooled) -> nrv_status {
-        NRV_TRY(conv(l, A(in), c1, nullptr, 0, out, level));
-        return pool(out, pooled, level + 1);
+        net->backend[l] = 1;
+        return fp8_conv_pool(net, l, in, c1, out, level, pooled, s);
     };
     NRV_TRY(conv(L_E0A, netin, 16, nullptr, 0, A_E0A, 0));
     NRV_TRY(conv_pool(L_E0B, A_E0A, 16, A_E0B, 0, A_P0));
@@ -263,30 +273,29 @@ nrv_status forward_fp8_mixed(Net* net, const void* netin, float* rgb, cudaStream
                      int level) -> nrv_status {
         return tc_conv3(net, l, x1, c1, x2, c2, A(out), g, level, NRV_PREC_FP8_E4M3, s, inv(out));
     };
-    auto pool8 = [&](int in, int out, int level_out) -> nrv_status {
-        const int c = net->act_c[in];
-        pool2_fp8_kernel<<<blocks_for(g.px(level_out) * c / 16), 256, 0, s>>>(
-            A(in), A(out), c, g.n, g.h[level_out], g.w[level_out]);
-        NRV_CHECK_LAUNCH();
-        return NRV_OK;
-    };
     auto up8 = [&](int l, int in, int out, int level_in) -> nrv_status {
         return tc_upconv(net, l, A(in), A(out), g, level_in, NRV_PREC_FP8_E4M3, s, inv(out));
     };
     // level 0 encoder in BF16 from the BF16 input
     NRV_TRY(tc_conv3(net, L_E0A, netin, net->c0p, nullptr, 0, A(A_E0A), g, 0, NRV_PREC_BF16, s));
-    NRV_TRY(tc_conv3(net, L_E0B, A(A_E0A), 16, nullptr, 0, A(A_E0B), g, 0, NRV_PREC_BF16, s));
-    // pooled to level 1 and quantised with the scale of e0b's output
-    pool2_bf16_to_fp8_kernel<<<blocks_for(g.px(1)), 256, 0, s>>>(
-        (const __nv_bfloat16*)A(A_E0B), A(A_P0), 16, g.n, g.h[1], g.w[1], inv(A_P0));
-    NRV_CHECK_LAUNCH();
+    // pooled to level 1 and quantised with the scale of e0b's output, in e0b's epilogue
+    const TcExtra quant{inv(A_P0), 0.0f};
+    nrv_status st = tc_conv3(net, L_E0B, A(A_E0A), 16, nullptr, 0, A(A_E0B), g, 0, NRV_PREC_BF16, s, 1.0f,
+                             nullptr, A(A_P0), &quant);
+    if (st == NRV_ERR_UNSUPPORTED) {
+        clear_error();
+        NRV_TRY(tc_conv3(net, L_E0B, A(A_E0A), 16, nullptr, 0, A(A_E0B), g, 0, NRV_PREC_BF16, s));
+        pool2_bf16_to_fp8_kernel<<<blocks_for(g.px(1)), 256, 0, s>>>(
+            (const __nv_bfloat16*)A(A_E0B), A(A_P0), 16, g.n, g.h[1], g.w[1], inv(A_P0));
+        NRV_CHECK_LAUNCH();
+    } else {
+        NRV_TRY(st);
+    }
     // levels 1-3 in E4M3
     NRV_TRY(conv8(L_E1A, A(A_P0), 16, nullptr, 0, A_E1A, 1));
-    NRV_TRY(conv8(L_E1B, A(A_E1A), 32, nullptr, 0, A_E1B, 1));
-    NRV_TRY(pool8(A_E1B, A_P1, 2));
+    NRV_TRY(fp8_conv_pool(net, L_E1B, A_E1A, 32, A_E1B, 1, A_P1, s));
     NRV_TRY(conv8(L_E2A, A(A_P1), 32, nullptr, 0, A_E2A, 2));
-    NRV_TRY(conv8(L_E2B, A(A_E2A), 64, nullptr, 0, A_E2B, 2));
-    NRV_TRY(pool8(A_E2B, A_P2, 3));
+    NRV_TRY(fp8_conv_pool(net, L_E2B, A_E2A, 64, A_E2B, 2, A_P2, s));
     NRV_TRY(conv8(L_E3A, A(A_P2), 64, nullptr, 0, A_E3A, 3));
     NRV_TRY(conv8(L_E3B, A(A_E3A), 128, nullptr, 0, A_E3B, 3));
     NRV_TRY(up8(L_UP3, A_E3B, A_UP3, 3));
@@ -294,13 +303,25 @@ nrv_status forward_fp8_mixed(Net* net, const void* netin, float* rgb, cudaStream
     NRV_TRY(conv8(L_D2B, A(A_D2A), 64, nullptr, 0, A_D2B, 2));
     NRV_TRY(up8(L_UP2, A_D2B, A_UP2, 2));
     NRV_TRY(conv8(L_D1A, A(A_UP2), 32, A(A_E1B), 32, A_D1A, 1));
-    NRV_TRY(conv8(L_D1B, A(A_D1A), 32, nullptr, 0, A_D1B, 1));
-    // back to BF16 for level 0: d1b's output decoded into d1a's slot (no longer read)
-    const size_t rows1 = (size_t)g.n * g.h[1];
-    fp8_to_bf16_kernel<<<blocks_for(rows1 * g.w[1] * 4), 256, 0, s>>>(
-        A(A_D1B), (__nv_bfloat16*)A(A_D1A), 32, rows1, g.w[1], net->act_scale[1 + A_D1B]);
-    NRV_CHECK_LAUNCH();
-    NRV_TRY(tc_upconv(net, L_UP1, A(A_D1A), A(A_UP1), g, 1, NRV_PREC_BF16, s));
+    // back to BF16 for level 0: d1b's codes decoded in its epilogue (d1b's own slot holds them as
+    // BF16: elem_size sizes it for two bytes a value)
+    const TcExtra decode{0.0f, net->act_scale[1 + A_D1B]};
+    void* d1b = A(A_D1B);
+    st = tc_conv3(net, L_D1B, A(A_D1A), 32, nullptr, 0, d1b, g, 1, NRV_PREC_FP8_E4M3, s, inv(A_D1B), nullptr,
+                  nullptr, &decode);
+    if (st == NRV_ERR_UNSUPPORTED) {
+        // decoded into d1a's slot (no longer read)
+        clear_error();
+        NRV_TRY(conv8(L_D1B, A(A_D1A), 32, nullptr, 0, A_D1B, 1));
+        d1b = A(A_D1A);
+        const size_t rows1 = (size_t)g.n * g.h[1];
+        fp8_to_bf16_kernel<<<blocks_for(rows1 * g.w[1] * 4), 256, 0, s>>>(
+            A(A_D1B), (__nv_bfloat16*)d1b, 32, rows1, g.w[1], net->act_scale[1 + A_D1B]);
+        NRV_CHECK_LAUNCH();
+    } else {
+        NRV_TRY(st);
+    }
+    NRV_TRY(tc_upconv(net, L_UP1, d1b, A(A_UP1), g, 1, NRV_PREC_BF16, s));
     NRV_TRY(tc_conv3(net, L_D0A, A(A_UP1), 16, A(A_E0B), 16, A(A_D0A), g, 0, NRV_PREC_BF16, s));
     const Layer& Lh = net->layers[L_HEAD];
     const float* P = (const float*)net->params.p;

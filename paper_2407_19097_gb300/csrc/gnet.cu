@@ -63,36 +63,33 @@ int64_t gnet_layers(int c0, GLayer* L) {
     return off;
 }
 
-// g[o] = b[o] + sum_c W[o][c] x[c] for o < c0, zero for c0 <= o < 8: the 1x1 projection of the
-// packed G-buffers (8 BF16 channels per pixel in and out), FP32 accumulation.
-__global__ void inj_kernel(const uint4* __restrict__ x, uint4* __restrict__ g, size_t npx, int c0,
-                           const float* __restrict__ w, const float* __restrict__ b) {
-    // the weights in registers (channels from c0 on are neither read nor written but as zero)
-    float wr[8][8], br[8];
+// The 1x1 projection of the packed G-buffers (8 BF16 channels per pixel in and out; channels
+// from c0 on zero), FP32 accumulation: g[o] = b[o] + sum_c W[o][c] x[c].
+struct InjWeights {
+    float w[8][8], b[8];
+    __device__ __forceinline__ void load(int c0, const float* __restrict__ wp, const float* __restrict__ bp) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        br[k] = k < c0 ? b[k] : 0.0f;
+        for (int k = 0; k < 8; ++k) {
+            b[k] = k < c0 ? bp[k] : 0.0f;
 #pragma unroll
-        for (int c = 0; c < 8; ++c) wr[k][c] = (k < c0 && c < c0) ? w[k * c0 + c] : 0.0f;
+            for (int c = 0; c < 8; ++c) w[k][c] = (k < c0 && c < c0) ? wp[k * c0 + c] : 0.0f;
+        }
     }
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < npx;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const uint4 raw = x[i];
+    __device__ __forceinline__ uint4 pixel(const uint4 raw, int c0) const {
         const uint32_t rw[4] = {raw.x, raw.y, raw.z, raw.w};
         float in[8];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&rw[j]);
-            in[2 * j] = __low2float(h2);
-            in[2 * j + 1] = __high2float(h2);
+            in[2 * j] = __uint_as_float(rw[j] << 16);
+            in[2 * j + 1] = __uint_as_float(rw[j] & 0xFFFF0000u);
         }
         float o[8];
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-            float acc = br[k];
+            float acc = b[k];
 #pragma unroll
             for (int c = 0; c < 8; ++c)
-                if (c < c0) acc = fmaf(wr[k][c], in[c], acc);
+                if (c < c0) acc = fmaf(w[k][c], in[c], acc);
             o[k] = acc;
         }
         uint32_t pk[4];
@@ -101,7 +98,79 @@ __global__ void inj_kernel(const uint4* __restrict__ x, uint4* __restrict__ g, s
             __nv_bfloat162 h2 = __floats2bfloat162_rn(o[2 * j], o[2 * j + 1]);
             pk[j] = *reinterpret_cast<uint32_t*>(&h2);
         }
-        g[i] = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        return make_uint4(pk[0], pk[1], pk[2], pk[3]);
+    }
+};
+
+__global__ void inj_kernel(const uint4* __restrict__ x, uint4* __restrict__ g, size_t npx, int c0,
+                           const float* __restrict__ w, const float* __restrict__ b) {
+    InjWeights W;
+    W.load(c0, w, b);
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < npx;
+         i += (size_t)gridDim.x * blockDim.x)
+        g[i] = W.pixel(x[i], c0);
+}
+
+// The projection and its whole pyramid in one pass (four launches took 45 us at 1080p, most of
+// it re-reading): a warp takes 32 x 8 pixels -- lane x of every row, so loads and stores of a row
+// are 512 contiguous bytes -- and pools them in registers and shuffles, with the pool kernel's
+// arithmetic on the stored (BF16) values of each level.  h, wd: multiples of 8.
+__device__ __forceinline__ uint4 pool4(const uint4 a, const uint4 b, const uint4 c, const uint4 d) {
+    const uint32_t aw[4] = {a.x, a.y, a.z, a.w}, bw[4] = {b.x, b.y, b.z, b.w}, cw[4] = {c.x, c.y, c.z, c.w},
+                   dw[4] = {d.x, d.y, d.z, d.w};
+    uint32_t r[4];
+    auto lo = [](uint32_t v) { return __uint_as_float(v << 16); };
+    auto hi = [](uint32_t v) { return __uint_as_float(v & 0xFFFF0000u); };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        __nv_bfloat162 h2 = __floats2bfloat162_rn(0.25f * ((lo(aw[j]) + lo(bw[j])) + (lo(cw[j]) + lo(dw[j]))),
+                                                  0.25f * ((hi(aw[j]) + hi(bw[j])) + (hi(cw[j]) + hi(dw[j]))));
+        r[j] = *reinterpret_cast<uint32_t*>(&h2);
+    }
+    return make_uint4(r[0], r[1], r[2], r[3]);
+}
+__device__ __forceinline__ uint4 shfl4(const uint4 v, int off) {
+    return make_uint4(__shfl_down_sync(0xffffffffu, v.x, off), __shfl_down_sync(0xffffffffu, v.y, off),
+                      __shfl_down_sync(0xffffffffu, v.z, off), __shfl_down_sync(0xffffffffu, v.w, off));
+}
+__global__ void __launch_bounds__(256) inj_pyramid_kernel(const uint4* __restrict__ x, uint4* __restrict__ g0,
+                                                          uint4* __restrict__ g1, uint4* __restrict__ g2,
+                                                          uint4* __restrict__ g3, int n, int h, int wd, int c0,
+                                                          const float* __restrict__ w,
+                                                          const float* __restrict__ b) {
+    InjWeights W;
+    W.load(c0, w, b);
+    const int lane = threadIdx.x & 31, tx = (wd + 31) / 32, ty = h / 8;
+    const int tiles = n * ty * tx, nwarps = (gridDim.x * blockDim.x) / 32;
+    for (int t = (blockIdx.x * blockDim.x + threadIdx.x) / 32; t < tiles; t += nwarps) {
+        const int xt = t % tx, yt = (t / tx) % ty, img = t / (tx * ty);
+        const int px = xt * 32 + lane;
+        const bool in = px < wd;
+        uint4 p2[2];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {          // four rows: one row of level 2
+            uint4 p1[2];
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {      // two rows: one row of level 1
+                uint4 v[2];
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const size_t at = ((size_t)img * h + yt * 8 + q * 4 + k * 2 + r) * wd + px;
+                    v[r] = make_uint4(0u, 0u, 0u, 0u);
+                    if (in) {
+                        v[r] = W.pixel(x[at], c0);
+                        g0[at] = v[r];
+                    }
+                }
+                p1[k] = pool4(v[0], shfl4(v[0], 1), v[1], shfl4(v[1], 1));
+                if (in && !(lane & 1))
+                    g1[((size_t)img * (h / 2) + yt * 4 + q * 2 + k) * (wd / 2) + px / 2] = p1[k];
+            }
+            p2[q] = pool4(p1[0], shfl4(p1[0], 2), p1[1], shfl4(p1[1], 2));
+            if (in && !(lane & 3)) g2[((size_t)img * (h / 4) + yt * 2 + q) * (wd / 4) + px / 4] = p2[q];
+        }
+        const uint4 p3 = pool4(p2[0], shfl4(p2[0], 4), p2[1], shfl4(p2[1], 4));
+        if (in && !(lane & 7)) g3[((size_t)img * (h / 8) + yt) * (wd / 8) + px / 8] = p3;
     }
 }
 
@@ -236,15 +305,11 @@ extern "C" nrv_status nrv_gnet_shade(nrv_gnet* g, const void* netin, int n, int 
     char* A = (char*)g->acts.p;
     const float* P = (const float*)g->params.p;
     // injection: the 1x1 projection and its pyramid
-    inj_kernel<<<blocks(px(0)), 256, 0, s>>>((const uint4*)netin, (uint4*)(A + o_g[0]), px(0),
-                                             g->c_in, P + g->L[G_INJ].woff, P + g->L[G_INJ].boff);
+    if (px(0) / 8 > 0x7FFFFFFFull) return fail(NRV_ERR_UNSUPPORTED, "too many pixels");
+    inj_pyramid_kernel<<<blocks((size_t)n * (H[0] / 8) * ((W[0] + 31) / 32) * 32), 256, 0, s>>>(
+        (const uint4*)netin, (uint4*)(A + o_g[0]), (uint4*)(A + o_g[1]), (uint4*)(A + o_g[2]),
+        (uint4*)(A + o_g[3]), n, H[0], W[0], g->c_in, P + g->L[G_INJ].woff, P + g->L[G_INJ].boff);
     NRV_CHECK_LAUNCH();
-    using T = __nv_bfloat16;
-    for (int l = 1; l < 4; ++l) {
-        pool2_kernel<T><<<blocks(px(l)), 256, 0, s>>>(TView<const T>{(const T*)(A + o_g[l - 1]), 8, 1},
-                                                      TView<T>{(T*)(A + o_g[l]), 8, 1}, 8, n, H[l], W[l]);
-        NRV_CHECK_LAUNCH();
-    }
     const TcPacked* tc = g->tc;
     // encoder (pools fused into e0..e2)
     NRV_TRY(tc_generic_run(tc, T_E0, P, A + o_g[0], nullptr, A + o_e[0], n, H[0], W[0], s, nullptr,
