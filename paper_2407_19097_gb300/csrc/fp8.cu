@@ -279,7 +279,8 @@ nrv_status forward_fp8_mixed(Net* net, const void* netin, float* rgb, cudaStream
     // level 0 encoder in BF16 from the BF16 input
     NRV_TRY(tc_conv3(net, L_E0A, netin, net->c0p, nullptr, 0, A(A_E0A), g, 0, NRV_PREC_BF16, s));
     // pooled to level 1 and quantised with the scale of e0b's output, in e0b's epilogue
-    const TcExtra quant{inv(A_P0), 0.0f};
+    TcExtra quant;
+    quant.pool_inv = inv(A_P0);
     nrv_status st = tc_conv3(net, L_E0B, A(A_E0A), 16, nullptr, 0, A(A_E0B), g, 0, NRV_PREC_BF16, s, 1.0f,
                              nullptr, A(A_P0), &quant);
     if (st == NRV_ERR_UNSUPPORTED) {
@@ -305,7 +306,8 @@ nrv_status forward_fp8_mixed(Net* net, const void* netin, float* rgb, cudaStream
     NRV_TRY(conv8(L_D1A, A(A_UP2), 32, A(A_E1B), 32, A_D1A, 1));
     // back to BF16 for level 0: d1b's codes decoded in its epilogue (d1b's own slot holds them as
     // BF16: elem_size sizes it for two bytes a value)
-    const TcExtra decode{0.0f, net->act_scale[1 + A_D1B]};
+    TcExtra decode;
+    decode.dec_scale = net->act_scale[1 + A_D1B];
     void* d1b = A(A_D1B);
     st = tc_conv3(net, L_D1B, A(A_D1A), 32, nullptr, 0, d1b, g, 1, NRV_PREC_FP8_E4M3, s, inv(A_D1B), nullptr,
                   nullptr, &decode);

@@ -360,16 +360,15 @@ extern "C" nrv_status nrv_gnet_run_layer(nrv_gnet* g, int layer, const void* x1,
     if (layer == G_E0) c1 = 8;
     if (layer == G_E1 || layer == G_E2 || layer == G_E3) { c1 = L.cin - g->c_in; c2 = 8; }
     if (layer == G_D2 || layer == G_D1 || layer == G_D0) { c1 = L.cin / 2; c2 = L.cin / 2; }
-    const bool up = L.kind == UPCONV2;
-    const size_t rows = (size_t)n * h, rows_out = up ? 2 * rows : rows;
-    const int w_out = up ? 2 * w : w;
+    const size_t rows = (size_t)n * h;
     auto al = [](size_t b) { return (b + 255) / 256 * 256; };
-    const size_t b1 = al(rows * w * c1 * 2), b2 = al(rows * w * c2 * 2), by = al(rows_out * w_out * L.cout * 2);
-    NRV_TRY(g->layer_ws.ensure(b1 + b2 + by));
+    const size_t b1 = al(rows * w * c1 * 2), b2 = al(rows * w * c2 * 2);
+    NRV_TRY(g->layer_ws.ensure(b1 + b2));
     char* ws = (char*)g->layer_ws.p;
-    NRV_TRY(relayout(x1, ws, rows, w, c1, 2, true, s));
-    if (c2) NRV_TRY(relayout(x2, ws + b1, rows, w, c2, 2, true, s));
-    NRV_TRY(tc_generic_run(g->tc, t, (const float*)g->params.p, ws, c2 ? ws + b1 : nullptr,
-                           ws + b1 + b2, n, h, w, s));
-    return relayout(ws + b1 + b2, y, rows_out, w_out, L.cout, 2, false, s);
+    const RelayoutJob jobs[2] = {{x1, ws, rows, w, c1}, {x2, ws + b1, rows, w, c2}};
+    NRV_TRY(relayout_in(jobs, 2, 2, s));
+    TcExtra direct;
+    direct.nhwc = true;
+    return tc_generic_run(g->tc, t, (const float*)g->params.p, ws, c2 ? ws + b1 : nullptr, y, n, h, w, s,
+                          nullptr, nullptr, &direct);
 }

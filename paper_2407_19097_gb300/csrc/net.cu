@@ -355,9 +355,60 @@ nrv_status relayout(const void* src, void* dst, size_t rows, int w, int c, size_
     return NRV_OK;
 }
 
+// Several tensors in one launch.  A block writes 1024 consecutive 16-byte chunks, four per
+// thread with their reads in flight together; one 64-bit division per block, 32 bits after that.
+struct RelayoutTable {
+    int n;
+    unsigned first[4];   // first block of each job
+    size_t total[3];     // chunks
+    const uint4* src[3];
+    uint4* dst[3];
+    uint32_t w[3], nch[3];
+};
+__global__ void __launch_bounds__(256) relayout_in_kernel(const __grid_constant__ RelayoutTable T) {
+    int k = 0;
+    if (T.n > 1 && blockIdx.x >= T.first[1]) k = 1;
+    if (T.n > 2 && blockIdx.x >= T.first[2]) k = 2;
+    const uint32_t w = T.w[k], nch = T.nch[k], per = w * nch;
+    const size_t b0 = (size_t)(blockIdx.x - T.first[k]) * 1024, total = T.total[k];
+    const size_t row0 = b0 / per;
+    const uint32_t l0 = (uint32_t)(b0 - row0 * per) + threadIdx.x;
+    const uint4* const src = T.src[k] + row0 * per;
+    uint4 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        // planar index: pixels fastest
+        const uint32_t l = l0 + 256 * j, row = l / per, q = l - row * per, ch = q / w, x = q - ch * w;
+        if (b0 + threadIdx.x + 256 * j < total) v[j] = __ldg(src + (size_t)row * per + (size_t)x * nch + ch);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+        if (b0 + threadIdx.x + 256 * j < total) T.dst[k][b0 + threadIdx.x + 256 * j] = v[j];
+}
+
+nrv_status relayout_in(const RelayoutJob* jobs, int n, size_t es, cudaStream_t s) {
+    RelayoutTable T;
+    memset(&T, 0, sizeof(T));
+    for (int k = 0; k < n; ++k) {
+        const RelayoutJob& j = jobs[k];
+        if (!j.src || j.c == 0) continue;
+        const int at = T.n++;
+        T.src[at] = (const uint4*)j.src;
+        T.dst[at] = (uint4*)j.dst;
+        T.w[at] = (uint32_t)j.w;
+        T.nch[at] = (uint32_t)(j.c * es / 16);
+        T.total[at] = j.rows * T.w[at] * T.nch[at];
+        T.first[at + 1] = T.first[at] + (unsigned)((T.total[at] + 1023) / 1024);
+    }
+    if (T.n == 0) return NRV_OK;
+    relayout_in_kernel<<<T.first[T.n], 256, 0, s>>>(T);
+    NRV_CHECK_LAUNCH();
+    return NRV_OK;
+}
+
 // One layer alone (nrv_net_run_layer): same kernels and dispatch as the forward
-// pass.  The caller's tensors are NHWC; BF16 and FP8 layers run on row-planar
-// copies in the handle's scratch, as inside the network.
+// pass.  The caller's tensors are NHWC; BF16 and FP8 layers read row-planar copies in the
+// handle's scratch, as inside the network; a BF16 layer stores its NHWC output itself.
 nrv_status net_run_layer(Net* net, int l, const void* x1, const void* x2, int n, int h, int w,
                          nrv_prec prec, void* y, cudaStream_t s) {
     NRV_TRY(set_kernel_attrs());
@@ -398,8 +449,18 @@ nrv_status net_run_layer(Net* net, int l, const void* x1, const void* x2, int n,
     NRV_TRY(net->layer_ws.ensure(b1 + b2 + by));
     char* ws = (char*)net->layer_ws.p;
     void *p1 = ws, *p2 = c2 ? ws + b1 : nullptr, *py = ws + b1 + b2;
-    NRV_TRY(relayout(x1, p1, rows_in, w, c1, es, true, s));
-    if (c2) NRV_TRY(relayout(x2, p2, rows_in, w, c2, es, true, s));
+    const RelayoutJob jobs[2] = {{x1, p1, rows_in, w, c1}, {x2, p2, rows_in, w, c2}};
+    NRV_TRY(relayout_in(jobs, 2, es, s));
+    if (prec == NRV_PREC_BF16) {
+        TcExtra direct;
+        direct.nhwc = true;
+        const nrv_status st = up ? tc_upconv(net, l, p1, y, g, 0, prec, s, 1.0f, &direct)
+                                 : tc_conv3(net, l, p1, c1, p2, c2, y, g, 0, prec, s, 1.0f, nullptr, nullptr,
+                                            &direct);
+        net->backend[l] = 1;
+        if (st != NRV_ERR_UNSUPPORTED) return st;
+        clear_error();
+    }
     float inv_out = 1.0f;
     if (prec == NRV_PREC_FP8_E4M3) {
         int in1, in2, out;

@@ -92,6 +92,14 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
 // channels of es bytes
 nrv_status relayout(const void* src, void* dst, size_t rows, int w, int c, size_t es,
                     bool to_planar, cudaStream_t s);
+// up to three tensors from NHWC to row-planar in one launch (entries with a null source skipped)
+struct RelayoutJob {
+    const void* src;
+    void* dst;
+    size_t rows;
+    int w, c;
+};
+nrv_status relayout_in(const RelayoutJob* jobs, int n, size_t es, cudaStream_t s);
 nrv_status net_repack(Net* net, cudaStream_t s);
 // parameters in and out (netio.cu): Xavier-uniform draw into d_params, file save / load
 nrv_status net_init_params(const Net* net, uint64_t seed, float* d_params, cudaStream_t s);
@@ -111,11 +119,13 @@ struct TcHead {
     RgbTab tab;      // per-image destinations (tab.on), else rgb + img * h * w_px * 3
 };
 
-// Conversions fused into a 3x3 conv at the borders of the mixed FP8 network (0: none):
-// pool_inv: the pool of a BF16 conv stored as E4M3 codes of mean * pool_inv; dec_scale: the
-// output of an E4M3 conv stored as BF16 of code * dec_scale.
+// Conversions fused into a layer's epilogue.  pool_inv: the pool of a BF16 conv stored as E4M3
+// codes of mean * pool_inv; dec_scale: the output of an E4M3 conv stored as BF16 of code *
+// dec_scale (0: none; both at the borders of the mixed FP8 network).  nhwc: the BF16 output, and
+// the mask of a data gradient, in NHWC (single layers called with NHWC tensors).
 struct TcExtra {
-    float pool_inv, dec_scale;
+    float pool_inv = 0.0f, dec_scale = 0.0f;
+    bool nhwc = false;
 };
 
 // tensor-core convolution (tc.cu); returns NRV_ERR_UNSUPPORTED when a shape is not covered
@@ -125,7 +135,8 @@ nrv_status tc_conv3(const Net* net, int layer, const void* x1, int c1, const voi
                     void* pool_y = nullptr,    // pool_y: also the 2x2 average pool of y
                     const TcExtra* extra = nullptr);
 nrv_status tc_upconv(const Net* net, int layer, const void* x, void* y, const Geo& g, int level_in,
-                     nrv_prec prec, cudaStream_t s, float inv_out = 1.0f);
+                     nrv_prec prec, cudaStream_t s, float inv_out = 1.0f,
+                     const TcExtra* extra = nullptr);
 nrv_status tc_repack_fp8(Net* net, cudaStream_t s);
 // TMA map of a row-planar tensor [n][h][nch][w][16 bytes] (tc.cu): boxes of 128 pixels x
 // box_planes planes of one row
@@ -156,12 +167,12 @@ nrv_status tc_wgrad(const Net* net, int l, const void* g, const void* x1, int c1
 // the output gradient gin with the flipped, transposed kernel, zeroed where mask <= 0 (mask
 // may be null); NRV_ERR_UNSUPPORTED when the layer has no such path
 nrv_status tc_dgrad(const Net* net, int l, const void* gin, void* out, const void* mask, int n, int H,
-                    int W, cudaStream_t s);
+                    int W, cudaStream_t s, const TcExtra* extra = nullptr);
 // data gradient of transposed conv l on the tensor cores (BF16, row-planar): out (C_in at the
 // input level (n, H, W)) from the output gradient g at (2H, 2W), which holds g_ld channels of
 // which C_out from g_off on, zeroed where mask (shaped like out) is not positive
 nrv_status tc_updgrad(const Net* net, int l, const void* g, int g_ld, int g_off, const void* mask,
-                      void* out, int n, int H, int W, cudaStream_t s);
+                      void* out, int n, int H, int W, cudaStream_t s, const TcExtra* extra = nullptr);
 // A layer of another network on the tensor-core conv kernel (tc.cu): a 3x3 conv (plain or
 // gated) or a 2x2 stride-2 transposed conv, BF16 row-planar in and out.  c1, c2: the stored
 // channels of the sources (multiples of 8; c2 = 0 without a second source), cin_real: the
@@ -177,7 +188,8 @@ nrv_status tc_generic_prepare(const TcGeneric* L, int n, const float* params, Tc
                               cudaStream_t s);
 nrv_status tc_generic_run(const TcPacked* st, int l, const float* params, const void* x1,
                           const void* x2, void* y, int n, int H, int W, cudaStream_t s,
-                          const TcHead* head = nullptr, void* pool_y = nullptr);
+                          const TcHead* head = nullptr, void* pool_y = nullptr,
+                          const TcExtra* extra = nullptr);
 void tc_generic_free(TcPacked* st);
 nrv_status forward_fp8(Net* net, const uint8_t* netin, float* rgb, cudaStream_t s, bool keep_acts);
 // levels 1-3 in E4M3, level 0 in BF16 (fp8.cu); netin is the BF16 packed input

@@ -102,6 +102,7 @@ struct TcParams {
                              // buffer i mod nacc, so the issuers run up to nacc tiles ahead
     int cout;                // output channels
     int out_nch;             // 16-byte planes per output row
+    int nhwc;                // BF16: the output (and the mask) NHWC instead of row-planar
     int mode;                // 0: 3x3 conv (+ bias, ReLU); 1: 2x2 stride-2 transposed conv + bias;
                              // 2: data gradient of the transposed conv (stored like mode 0)
     int parity_plane0;       // mode 2: first plane of the output gradient's channels
@@ -674,8 +675,11 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         xo = 2 * x + (abi & 1);
                         wo = 2 * P.w;
                     }
+                    // 16-byte word of these channels, and from it to the next plane's
                     uint8_t* dst = (uint8_t*)P.y +
-                                   ((row * P.out_nch + (size_t)(o / ce)) * wo + xo) * 16;
+                                   (P.nhwc ? (row * wo + xo) * P.out_nch + (size_t)(o / ce)
+                                           : (row * P.out_nch + (size_t)(o / ce)) * wo + xo) * 16;
+                    const size_t pnext = P.nhwc ? 16 : (size_t)wo * 16;
                     if (FP8) {
                         uint32_t wd[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
@@ -702,7 +706,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                             const size_t off = (size_t)(dst - (uint8_t*)P.y);
                             const uint4 m0 = *reinterpret_cast<const uint4*>(P.mask + off);
                             const uint4 m1 =
-                                *reinterpret_cast<const uint4*>(P.mask + off + (size_t)wo * 16);
+                                *reinterpret_cast<const uint4*>(P.mask + off + pnext);
                             const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
                             for (int j = 0; j < 16; ++j) {
@@ -722,7 +726,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         if (P.store_y) {
                             *reinterpret_cast<uint4*>(dst) =
                                 make_uint4(packed[0], packed[1], packed[2], packed[3]);
-                            *reinterpret_cast<uint4*>(dst + (size_t)wo * 16) =
+                            *reinterpret_cast<uint4*>(dst + pnext) =
                                 make_uint4(packed[4], packed[5], packed[6], packed[7]);
                         }
                         if (P.pool_y && !(yy & 1)) {
@@ -818,8 +822,10 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
             const int oc0 = (slice * P.n_slice) >> (GATED ? 1 : 0);   // first output channel
             const bool dec = FP8 && P.dec_scale != 0.0f;                // BF16 output of an FP8 layer
             const int nch = dec ? 2 * P.out_nch : P.out_nch;            // planes of the stored output
-            const size_t pstride = (size_t)P.w * 16;                    // bytes between planes of a row
-            const size_t rstride = pstride * nch;                       // and between rows
+            // bytes between the planes of a pixel, the pixels of a plane and the rows
+            const size_t pstride = P.nhwc ? 16 : (size_t)P.w * 16;
+            const size_t xstride = P.nhwc ? (size_t)nch * 16 : 16;
+            const size_t rstride = (size_t)P.w * nch * 16;
             const int plane0 = oc0 / (FP8 && !dec ? 16 : 8);
             // the cursor: segment, row and this thread's word of plane0 in that row
             int ct = t_begin, left = 0, r = 0, y = 0, img = 0, x = 0;
@@ -834,7 +840,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 img = col / P.tiles_x;
                 x = (col - img * P.tiles_x) * P.tile_w + m;
                 vx = m < P.tile_w && x < P.w;
-                py = (uint8_t*)P.y + (size_t)img * P.h * rstride + plane0 * pstride + (size_t)x * 16 +
+                py = (uint8_t*)P.y + (size_t)img * P.h * rstride + plane0 * pstride + (size_t)x * xstride +
                      (long long)y * (long long)rstride;
                 ct = te;
             };
@@ -1153,10 +1159,12 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
         // contiguous bytes.
         auto emit_up = [&](uint32_t tbase, int img, int x, bool valid, int yy) {
             const size_t wo = 2 * (size_t)P.w;
+            // in 16-byte words: to the next plane of a pixel, to the next pixel of a plane
+            const size_t pw = P.nhwc ? 1 : wo, xw = P.nhwc ? (size_t)P.out_nch : 1;
 #pragma unroll 1
             for (int a = 0; a < 2; ++a) {
-                uint8_t* const prow =
-                    (uint8_t*)P.y + ((((size_t)img * 2 * P.h + 2 * yy + a) * P.out_nch) * wo + 2 * x) * 16;
+                uint8_t* const prow = (uint8_t*)P.y +
+                    ((((size_t)img * 2 * P.h + 2 * yy + a) * P.out_nch) * wo + 2 * x * xw) * 16;
 #pragma unroll 1
                 for (int o8 = 0; o8 < P.cout; o8 += 8) {
                     const int c0 = 2 * a * P.cout + o8, c1 = c0 + P.cout;   // b = 0 and b = 1
@@ -1185,9 +1193,9 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         p1[j] = P.relu ? bf16x2_relu(v[0], v[1]) : bf16x2(v[0], v[1]);
                     }
                     if (valid) {
-                        uint4* dst = reinterpret_cast<uint4*>(prow + (size_t)(o8 / 8) * wo * 16);
+                        uint4* dst = reinterpret_cast<uint4*>(prow + (size_t)(o8 / 8) * pw * 16);
                         dst[0] = make_uint4(p0[0], p0[1], p0[2], p0[3]);
-                        dst[1] = make_uint4(p1[0], p1[1], p1[2], p1[3]);
+                        dst[xw] = make_uint4(p1[0], p1[1], p1[2], p1[3]);
                     }
                 }
             }
@@ -1903,7 +1911,11 @@ static nrv_status tc_launch(const Net* net, const TcLayerCfg& c, const uint8_t* 
             return fail(NRV_ERR_UNSUPPORTED, "the fused pool needs a 3x3 conv on an even grid");
         P.pool_y = pool_y;
     }
-    if (extra) {
+    if (extra && extra->nhwc) {
+        if (fp8 || head || pool_y) return fail(NRV_ERR_UNSUPPORTED, "NHWC output");
+        P.nhwc = 1;
+    }
+    if (extra && (extra->pool_inv != 0.0f || extra->dec_scale != 0.0f)) {
         if (!P.stream || (extra->pool_inv != 0.0f && (fp8 || P.gated || !pool_y || P.out_nch % 2)) ||
             (extra->dec_scale != 0.0f && (!fp8 || epi != EPI_PLAIN)))
             return fail(NRV_ERR_UNSUPPORTED, "conversion fused into a 3x3 conv");
@@ -2188,13 +2200,13 @@ void tc_generic_free(TcPacked* st) { delete st; }
 
 nrv_status tc_generic_run(const TcPacked* st, int l, const float* params, const void* x1,
                           const void* x2, void* y, int n, int H, int W, cudaStream_t s,
-                          const TcHead* head, void* pool_y) {
+                          const TcHead* head, void* pool_y, const TcExtra* extra) {
     if (!st || l < 0 || l >= (int)st->cfg.size()) return fail(NRV_ERR_ARG, "bad layer");
     const TcLayerCfg& c = st->cfg[l];
     const TcGeneric& L = st->spec[l];
     return tc_launch(nullptr, c, (const uint8_t*)st->w.p + c.w_off, params + L.boff,
                      (c.kind == CONV3 && !c.gated) ? 1 : 0, nullptr, L.cout, x1, c.c1, x2, c.c2, y,
-                     n, H, W, s, 0, 1.0f, head, pool_y, 0, 0, c.gated ? params + L.boff2 : nullptr);
+                     n, H, W, s, 0, 1.0f, head, pool_y, 0, 0, c.gated ? params + L.boff2 : nullptr, extra);
 }
 
 nrv_status tc_conv3(const Net* net, int l, const void* x1, int c1, const void* x2, int c2, void* y,
@@ -2212,13 +2224,13 @@ nrv_status tc_conv3(const Net* net, int l, const void* x1, int c1, const void* x
 }
 
 nrv_status tc_dgrad(const Net* net, int l, const void* gin, void* out, const void* mask, int n, int H,
-                    int W, cudaStream_t s) {
+                    int W, cudaStream_t s, const TcExtra* extra) {
     const Layer& L = net->layers[l];
     const TcLayerCfg& c = g_cfg_dg[l];
     if (L.kind != CONV3 || !c.ok) return fail(NRV_ERR_UNSUPPORTED, "no tensor-core data gradient");
     const uint8_t* w = (const uint8_t*)net->wtbf16.p + c.w_off;
     return tc_launch(net, c, w, nullptr, 0, mask, L.cin, gin, L.cout, nullptr, 0, out, n, H, W, s, 0,
-                     1.0f);
+                     1.0f, nullptr, nullptr, 0, 0, nullptr, extra);
 }
 
 nrv_status tc_planar_map(CUtensorMap* map, const void* base, int n, int h, int w, int nch,
@@ -2247,18 +2259,18 @@ nrv_status tc_parity_map(CUtensorMap* map, const void* base, int rows, int w, in
 }
 
 nrv_status tc_updgrad(const Net* net, int l, const void* g, int g_ld, int g_off, const void* mask,
-                      void* out, int n, int H, int W, cudaStream_t s) {
+                      void* out, int n, int H, int W, cudaStream_t s, const TcExtra* extra) {
     const Layer& L = net->layers[l];
     const TcLayerCfg& c = g_cfg_dg[l];
     if (L.kind != UPCONV2 || !c.ok || c.kind != KIND_UPDGRAD)
         return fail(NRV_ERR_UNSUPPORTED, "no tensor-core data gradient");
     const uint8_t* w = (const uint8_t*)net->wtbf16.p + c.w_off;
     return tc_launch(net, c, w, nullptr, 0, mask, L.cin, g, L.cout, nullptr, 0, out, n, H, W, s, 0,
-                     1.0f, nullptr, nullptr, g_ld, g_off);
+                     1.0f, nullptr, nullptr, g_ld, g_off, nullptr, extra);
 }
 
 nrv_status tc_upconv(const Net* net, int l, const void* x, void* y, const Geo& g, int level_in,
-                     nrv_prec prec, cudaStream_t s, float inv_out) {
+                     nrv_prec prec, cudaStream_t s, float inv_out, const TcExtra* extra) {
     if (prec != NRV_PREC_BF16 && prec != NRV_PREC_FP8_E4M3)
         return fail(NRV_ERR_UNSUPPORTED, "tensor-core path is BF16 or FP8");
     const Layer& L = net->layers[l];
@@ -2267,7 +2279,8 @@ nrv_status tc_upconv(const Net* net, int l, const void* x, void* y, const Geo& g
     const TcLayerCfg& c = g_cfg[fp8][l];
     const uint8_t* w = (const uint8_t*)(fp8 ? net->wfp8.p : net->wbf16.p) + c.w_off;
     return tc_launch(net, c, w, (const float*)net->params.p + L.boff, 0, nullptr, L.cout, x, L.cin,
-                     nullptr, 0, y, g.n, g.h[level_in], g.w[level_in], s, fp8, inv_out);
+                     nullptr, 0, y, g.n, g.h[level_in], g.w[level_in], s, fp8, inv_out, nullptr, nullptr, 0,
+                     0, nullptr, extra);
 }
 
 }  // namespace nrv

@@ -935,8 +935,8 @@ nrv_status net_layer_wgrad(Net* net, int l, const void* dy, const void* x1, cons
         NRV_TRY(net->layer_ws.ensure(bg + bx));
         char* ws = (char*)net->layer_ws.p;
         T *pg = (T*)ws, *px = (T*)(ws + bg);
-        NRV_TRY(relayout(dy, pg, 2 * rows, 2 * w, L.cout, 2, true, s));
-        NRV_TRY(relayout(x1, px, rows, w, L.cin, 2, true, s));
+        const RelayoutJob jobs[2] = {{dy, pg, 2 * rows, 2 * w, L.cout}, {x1, px, rows, w, L.cin}};
+        NRV_TRY(relayout_in(jobs, 2, 2, s));
         Bwd<T> b(net, s, g, dgrad);
         return b.alone(l, [&] {
             return b.wgrad_up(l, TView<const T>{px, L.cin, 1}, TView<const T>{pg, L.cout, 1}, 0);
@@ -969,9 +969,8 @@ nrv_status net_layer_wgrad(Net* net, int l, const void* dy, const void* x1, cons
     NRV_TRY(net->layer_ws.ensure(bg + b1 + b2));
     char* ws = (char*)net->layer_ws.p;
     T *pg = (T*)ws, *p1 = (T*)(ws + bg), *p2 = c2 ? (T*)(ws + bg + b1) : nullptr;
-    NRV_TRY(relayout(dy, pg, rows, w, L.cout, 2, true, s));
-    NRV_TRY(relayout(x1, p1, rows, w, c1, 2, true, s));
-    if (c2) NRV_TRY(relayout(x2, p2, rows, w, c2, 2, true, s));
+    const RelayoutJob jobs[3] = {{dy, pg, rows, w, L.cout}, {x1, p1, rows, w, c1}, {x2, p2, rows, w, c2}};
+    NRV_TRY(relayout_in(jobs, 3, 2, s));
     Bwd<T> b(net, s, g, dgrad);
     return b.alone(l, [&] {
         return b.wgrad_conv(l, TView<const T>{pg, L.cout, 1}, TView<const T>{p1, c1, 1}, c1,
@@ -1006,6 +1005,14 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
         char* ws = (char*)net->layer_ws.p;
         T *pg = (T*)ws, *pm = (T*)(ws + bg), *po = (T*)(ws + bg + bm);
         NRV_TRY(relayout(dy, pg, 2 * rows, 2 * w, L.cout, 2, true, s));
+        {
+            // the caller's NHWC mask and gradient read and written in place
+            TcExtra direct;
+            direct.nhwc = true;
+            const nrv_status st = tc_updgrad(net, l, pg, L.cout, 0, mask, dx, n, h, w, s, &direct);
+            if (st != NRV_ERR_UNSUPPORTED) return st;
+            clear_error();
+        }
         NRV_TRY(relayout(mask, pm, rows, w, L.cin, 2, true, s));
         Bwd<T> b(net, s, g, nullptr);
         NRV_TRY(b.dgrad_up(l, TView<const T>{pg, L.cout, 1}, TView<const T>{pm, L.cin, 1},
@@ -1035,6 +1042,14 @@ nrv_status net_layer_dgrad(Net* net, int l, const void* dy, const void* mask, in
     char* ws = (char*)net->layer_ws.p;
     T *pg = (T*)ws, *pm = mask ? (T*)(ws + bg) : nullptr, *po = (T*)(ws + bg + bm);
     NRV_TRY(relayout(dy, pg, rows, w, L.cout, 2, true, s));
+    {
+        // the caller's NHWC mask and gradient read and written in place
+        TcExtra direct;
+        direct.nhwc = true;
+        const nrv_status st = tc_dgrad(net, l, pg, dx, mask, n, h, w, s, &direct);
+        if (st != NRV_ERR_UNSUPPORTED) return st;
+        clear_error();
+    }
     if (mask) NRV_TRY(relayout(mask, pm, rows, w, L.cin, 2, true, s));
     Bwd<T> b(net, s, g, nullptr);
     NRV_TRY(b.dgrad_conv(l, TView<const T>{pg, L.cout, 1}, TView<T>{po, L.cin, 1},
