@@ -136,24 +136,74 @@ struct ReduceSeg {
     float* dw;
 };
 
-// Every segment in one launch: block b belongs to the segment whose range of 32-sum blocks
-// holds it.  Each thread reads eight chunks before it adds them, so the pass is bound by the
-// partials' bytes and not by a chain of dependent loads (a segment per launch, one load at a
-// time, took 0.2 ms of a 1.6 ms training step).
+// Every segment in one launch: block b belongs to the segment whose range of blocks holds it.
+// Each thread reads eight chunks of four sums before it adds them, so the pass is bound by the
+// partials' bytes (123 MB in the 16 x 256^2 training step) and not by a chain of dependent loads.
 constexpr int MAX_SEGS = 2 * NUM_LAYERS;
 struct ReduceTable {
     int n;
     int first[MAX_SEGS + 1];   // first block of each segment
     ReduceSeg seg[MAX_SEGS];
 };
+// four consecutive sums per thread?
+__host__ __device__ inline bool reduce_vec(const ReduceSeg& R) {
+    return R.mode != 3 && R.count % 4 == 0 && R.stride % 4 == 0;
+}
+__host__ __device__ inline int reduce_blocks(const ReduceSeg& R) {
+    const int per = reduce_vec(R) ? 128 : 32;
+    return (R.count + per - 1) / per;
+}
+
+__device__ __forceinline__ void reduce_put(const ReduceSeg& R, int i, float t) {
+    if (R.mode == 0) {
+        const int K = 9 * R.cin, o = i / K, q = i % K, tap = q / R.cin, c = q % R.cin;
+        if (c < R.cin_real) R.dw[((size_t)o * R.cin_real + c) * 9 + tap] = t;
+    } else if (R.mode == 1) {
+        const int K = 4 * R.cout, c = i / K, q = i % K, ab = q / R.cout, o = q % R.cout;
+        R.dw[((size_t)c * R.cout + o) * 4 + ab] = t;
+    } else {
+        R.dw[i] = t;
+    }
+}
 
 __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ ReduceTable T) {
-    __shared__ float red[8][33];
+    __shared__ float red[8][132];
     int k = 0;
     while ((int)blockIdx.x >= T.first[k + 1]) ++k;
     const ReduceSeg& R = T.seg[k];
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int i = ((int)blockIdx.x - T.first[k]) * 32 + tx;
+    const int tx = threadIdx.x, ty = threadIdx.y, blk = (int)blockIdx.x - T.first[k];
+    if (reduce_vec(R)) {
+        const int i = blk * 128 + 4 * tx;
+        float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (i < R.count)
+            for (int c0 = ty; c0 < R.nchunks; c0 += 64) {
+                float4 v[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const int ch = c0 + 8 * j;
+                    v[j] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                    if (ch < R.nchunks) v[j] = __ldcs(reinterpret_cast<const float4*>(R.part + (size_t)ch * R.stride + i));
+                }
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    s[0] += v[j].x;
+                    s[1] += v[j].y;
+                    s[2] += v[j].z;
+                    s[3] += v[j].w;
+                }
+            }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) red[ty][4 * tx + e] = s[e];
+        __syncthreads();
+        // 128 sums, the first 128 threads one each
+        const int t = ty * 32 + tx;
+        if (t >= 128 || blk * 128 + t >= R.count) return;
+        float a = red[0][t];
+        for (int j = 1; j < 8; ++j) a += red[j][t];
+        reduce_put(R, blk * 128 + t, a);
+        return;
+    }
+    const int i = blk * 32 + tx;
     float s = 0.0f;
     if (i < R.count)
         for (int c0 = ty; c0 < R.nchunks; c0 += 64) {
@@ -175,17 +225,9 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_const
     red[ty][tx] = s;
     __syncthreads();
     if (ty != 0 || i >= R.count) return;
-    float t = red[0][tx];
-    for (int j = 1; j < 8; ++j) t += red[j][tx];
-    if (R.mode == 0) {
-        const int K = 9 * R.cin, o = i / K, q = i % K, tap = q / R.cin, c = q % R.cin;
-        if (c < R.cin_real) R.dw[((size_t)o * R.cin_real + c) * 9 + tap] = t;
-    } else if (R.mode == 1) {
-        const int K = 4 * R.cout, c = i / K, q = i % K, ab = q / R.cout, o = q % R.cout;
-        R.dw[((size_t)c * R.cout + o) * 4 + ab] = t;
-    } else {
-        R.dw[i] = t;
-    }
+    float a = red[0][tx];
+    for (int j = 1; j < 8; ++j) a += red[j][tx];
+    reduce_put(R, i, a);
 }
 
 // The partial sums of a backward pass: one region per layer of the net's buffer, and the table
@@ -203,7 +245,7 @@ struct Partials {
     }
     void add(const ReduceSeg& R) {
         T.seg[T.n] = R;
-        T.first[T.n + 1] = T.first[T.n] + (R.count + 31) / 32;
+        T.first[T.n + 1] = T.first[T.n] + reduce_blocks(R);
         ++T.n;
     }
     nrv_status flush(cudaStream_t s) {
@@ -359,15 +401,32 @@ __global__ void pool_bwd_kernel(TView<const T> gp, TView<const T> gs, TView<cons
 }
 
 // ------------------------------------------------------------------ loss and optimizer
-__global__ void l1_partial_kernel(const float* y, const float* t, int64_t n, float* dy,
-                                  float inv_n, float* part) {
+// Four values per thread and step where the pointers allow (vec), else one.
+__global__ void __launch_bounds__(256) l1_partial_kernel(const float* y, const float* t, int64_t n, float* dy,
+                                                         float inv_n, float* part, int vec) {
     __shared__ float red[256];
     float s = 0.0f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float d = y[i] - t[i];
+    auto one = [&](float a, float b, float& g) {
+        const float d = a - b;
         s += fabsf(d);
-        if (dy) dy[i] = d > 0.0f ? inv_n : (d < 0.0f ? -inv_n : 0.0f);
+        g = d > 0.0f ? inv_n : (d < 0.0f ? -inv_n : 0.0f);
+    };
+    const int64_t n4 = vec ? n / 4 : 0, stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t i0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+#pragma unroll 2
+    for (int64_t i = i0; i < n4; i += stride) {
+        const float4 a = reinterpret_cast<const float4*>(y)[i], b = reinterpret_cast<const float4*>(t)[i];
+        float4 g;
+        one(a.x, b.x, g.x);
+        one(a.y, b.y, g.y);
+        one(a.z, b.z, g.z);
+        one(a.w, b.w, g.w);
+        if (dy) reinterpret_cast<float4*>(dy)[i] = g;
+    }
+    for (int64_t i = 4 * n4 + i0; i < n; i += stride) {
+        float g;
+        one(y[i], t[i], g);
+        if (dy) dy[i] = g;
     }
     red[threadIdx.x] = s;
     __syncthreads();
@@ -397,7 +456,8 @@ nrv_status launch_l1(const float* y, const float* t, int64_t n, float* loss, flo
                      cudaStream_t s) {
     const int nb = 512;
     NRV_TRY(g_l1_part.ensure(nb * sizeof(float)));
-    l1_partial_kernel<<<nb, 256, 0, s>>>(y, t, n, dy, (float)(1.0 / (double)n), (float*)g_l1_part.p);
+    const int vec = (((uintptr_t)y | (uintptr_t)t | (uintptr_t)dy) & 15) == 0;
+    l1_partial_kernel<<<nb, 256, 0, s>>>(y, t, n, dy, (float)(1.0 / (double)n), (float*)g_l1_part.p, vec);
     NRV_CHECK_LAUNCH();
     l1_final_kernel<<<1, 256, 0, s>>>((const float*)g_l1_part.p, nb, 1.0 / (double)n, loss);
     NRV_CHECK_LAUNCH();
