@@ -250,11 +250,10 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
     __shared__ __align__(16) float colscale_s[256];
     __shared__ __align__(16) float head_ws[52];
     __shared__ __align__(16) float2 head_w2[EPI == EPI_HEAD ? 48 : 1];   // {w, w}
-    __shared__ uint32_t alo_s[MAX_KS + 1];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_number(), lane = threadIdx.x % 32;
     const uint32_t s_w = smem_u32(smem);
     const uint32_t s_ring = s_w + P.w_region;
     const uint32_t b_w = smem_u32(&bars[0]);
@@ -306,7 +305,6 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
         }
         colscale_s[i] = FP8 ? P.colscale[slice * P.n_slice + i] : 1.0f;
     }
-    for (int i = threadIdx.x; i <= MAX_KS; i += NT) alo_s[i] = i < P.nks ? P.a_lo[i] : 0u;
     if (P.head_w && threadIdx.x < 51)
         head_ws[threadIdx.x] = threadIdx.x < 48 ? P.head_w[threadIdx.x] : P.head_b[threadIdx.x - 48];
     if (EPI == EPI_HEAD && threadIdx.x < 48) {
@@ -323,7 +321,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = uniform(tmem_slot);
     if (STREAM) {
         // row streaming accumulates into every block: start from zeros
         if (warp >= 2 && warp <= 5) {
@@ -344,7 +342,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             // each input row once per run of tiles (the weights are already on their way)
             TileWalk w;
             w.init(P, t_begin);
@@ -365,36 +363,38 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         // until that row's group has committed
                         if (nloads >= P.nslot) {
                             const int g = (nloads - P.nslot) / P.grp;
-                            if (!mbar_wait(smem_u32(&bars_g[g & 15]), (uint32_t)(g >> 4) & 1u,
+                            if (!warp_wait(smem_u32(&bars_g[g & 15]), (uint32_t)(g >> 4) & 1u,
                                            &abort_flag, P.status)) {
                                 ok = false;
                                 break;
                             }
                         }
-                    } else if (!mbar_wait(b_hempty(slot), phase ^ 1u, &abort_flag, P.status)) {
+                    } else if (!warp_wait(b_hempty(slot), phase ^ 1u, &abort_flag, P.status)) {
                         ok = false;
                         break;
                     }
                     const uint32_t dst = s_ring + (uint32_t)slot * P.slot_bytes;
-                    mbar_expect_tx(b_hfull(slot), P.tx_bytes);
-                    if (P.mode == 2) {
-                        // output rows 2y + a, pixels 2x + b of the gradient: four blocks
-                        for (int k = 0; k < 4; ++k)
-                            tma_load_5d(dst + (uint32_t)k * P.ab_bytes, &tm1, 0, k & 1, xe >> 1,
-                                        P.parity_plane0, (w.img * P.h + next_row) * 2 + (k >> 1),
-                                        b_hfull(slot));
-                    } else {
-                        tma_load_4d(dst, &tm1, xe, 0, next_row, w.img, b_hfull(slot));
-                        if (P.has_src2)
-                            tma_load_4d(dst + P.src2_off, &tm2, xe, 0, next_row, w.img,
-                                        b_hfull(slot));
+                    if (elect_one()) {
+                        mbar_expect_tx(b_hfull(slot), P.tx_bytes);
+                        if (P.mode == 2) {
+                            // output rows 2y + a, pixels 2x + b of the gradient: four blocks
+                            for (int k = 0; k < 4; ++k)
+                                tma_load_5d(dst + (uint32_t)k * P.ab_bytes, &tm1, 0, k & 1, xe >> 1,
+                                            P.parity_plane0, (w.img * P.h + next_row) * 2 + (k >> 1),
+                                            b_hfull(slot));
+                        } else {
+                            tma_load_4d(dst, &tm1, xe, 0, next_row, w.img, b_hfull(slot));
+                            if (P.has_src2)
+                                tma_load_4d(dst + P.src2_off, &tm2, xe, 0, next_row, w.img,
+                                            b_hfull(slot));
+                        }
                     }
                     ++nloads;
                     ring_next(slot, phase, P.nslot);
                 }
             }
             // this CTA's inputs are all requested: the next layer may start launching
-            asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+            if (elect_one()) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
             // every load issued must have landed before the CTA may exit: the last
             // min(nloads, nslot) loads, walking the ring backwards
             for (int q = nloads < P.nslot ? nloads : P.nslot; q > 0; --q) {
@@ -404,14 +404,14 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 } else {
                     --slot;
                 }
-                mbar_wait(b_hfull(slot), phase, &abort_flag, P.status, false);
+                warp_wait(b_hfull(slot), phase, &abort_flag, P.status, false);
             }
-            mbar_wait(b_w, 0, &abort_flag, P.status, false);
+            warp_wait(b_w, 0, &abort_flag, P.status, false);
         }
     } else if (warp == 1 || (!STREAM && warp == 6)) {
         const int iss = warp == 1 ? 0 : 1;   // this warp's issuer number
-        if (lane == 0 && iss < P.nissue) {
-            bool ok = mbar_wait(b_w, 0, &abort_flag, P.status);
+        if (iss < P.nissue) {
+            bool ok = warp_wait(b_w, 0, &abort_flag, P.status);
             // descriptor high words: SBO = 128 bytes, version 1; B: K halves n_slice * 16 bytes apart
             const uint64_t hi = (uint64_t)((128u >> 4) | (1u << 14)) << 32;
             const uint32_t b_lbo = (uint32_t)P.n_slice * 16;
@@ -429,9 +429,6 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 const uint32_t ns = (uint32_t)P.n_slice;
                 int slot = 0, blk = 0, gin = 0, k = 0;
                 uint32_t ph = 0;
-                uint32_t alo_r[6];
-#pragma unroll
-                for (int j = 0; j < 6; ++j) alo_r[j] = j < ks_row ? alo_s[j] : 0u;
                 // segments: runs of tiles in one tile column; a segment of R output rows
                 // streams its R + 2 input rows, whose slots hold output rows y0 - 2 .. y0 + R - 1
                 for (int t = t_begin; ok && t < t_end;) {
@@ -443,12 +440,12 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         if (gin == 0 && k >= P.gm) {
                             // the blocks this group writes were last drained in group k - gm
                             const int kk = k - P.gm;
-                            if (!mbar_wait(b_aempty(kk & 3), (kk >> 2) & 1, &abort_flag, P.status)) {
+                            if (!warp_wait(b_aempty(kk & 3), (kk >> 2) & 1, &abort_flag, P.status)) {
                                 ok = false;
                                 break;
                             }
                         }
-                        if (!mbar_wait(b_hfull(slot), ph, &abort_flag, P.status)) {
+                        if (!warp_wait(b_hfull(slot), ph, &abort_flag, P.status)) {
                             ok = false;
                             break;
                         }
@@ -456,49 +453,42 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         const uint32_t base = ring16 + (uint32_t)slot * slot16;
                         const uint32_t d = tmem + (uint32_t)blk * ns;
                         uint32_t b_lo = b_lo0s;
-                        if (blk <= P.nb - 3 && ks_row <= 6) {
-                            // short rows (the narrow layers): descriptor words from registers
-#pragma unroll
-                            for (int j = 0; j < 6; ++j)
-                                if (j < ks_row) {
-                                    const uint64_t a = hi | (uint64_t)(base + alo_r[j]);
-                                    const uint64_t b = hi | (uint64_t)(b_lo0s + (uint32_t)j * b_jstep);
-                                    if (FP8) mma_fp8(d, a, b, P.idesc, 1u);
-                                    else mma_bf16(d, a, b, P.idesc, 1u);
+                        if (elect_one()) {
+                            if (blk <= P.nb - 3) {
+                                for (int j = 0; j < ks_row; ++j, b_lo += b_jstep) {
+                                    const uint64_t a = hi | (uint64_t)(base + P.a_lo[j]);
+                                    if (FP8) mma_fp8(d, a, hi | (uint64_t)b_lo, P.idesc, 1u);
+                                    else mma_bf16(d, a, hi | (uint64_t)b_lo, P.idesc, 1u);
                                 }
-                        } else if (blk <= P.nb - 3) {
-                            for (int j = 0; j < ks_row; ++j, b_lo += b_jstep) {
-                                const uint64_t a = hi | (uint64_t)(base + alo_s[j]);
-                                if (FP8) mma_fp8(d, a, hi | (uint64_t)b_lo, P.idesc, 1u);
-                                else mma_bf16(d, a, hi | (uint64_t)b_lo, P.idesc, 1u);
-                            }
-                        } else {
-                            // the three blocks wrap around the ring: two MMAs per K-step
-                            const uint32_t id_a = blk == P.nb - 2 ? P.idesc2 : P.idesc1;
-                            const uint32_t id_b = blk == P.nb - 2 ? P.idesc1 : P.idesc2;
-                            const uint32_t b_off = blk == P.nb - 2 ? 2 * b_n1 : b_n1;
-                            for (int j = 0; j < ks_row; ++j, b_lo += b_jstep) {
-                                const uint64_t a = hi | (uint64_t)(base + alo_s[j]);
-                                if (FP8) {
-                                    mma_fp8(d, a, hi | (uint64_t)b_lo, id_a, 1u);
-                                    mma_fp8(tmem, a, hi | (uint64_t)(b_lo + b_off), id_b, 1u);
-                                } else {
-                                    mma_bf16(d, a, hi | (uint64_t)b_lo, id_a, 1u);
-                                    mma_bf16(tmem, a, hi | (uint64_t)(b_lo + b_off), id_b, 1u);
+                            } else {
+                                // the three blocks wrap around the ring: two MMAs per K-step
+                                const uint32_t id_a = blk == P.nb - 2 ? P.idesc2 : P.idesc1;
+                                const uint32_t id_b = blk == P.nb - 2 ? P.idesc1 : P.idesc2;
+                                const uint32_t b_off = blk == P.nb - 2 ? 2 * b_n1 : b_n1;
+                                for (int j = 0; j < ks_row; ++j, b_lo += b_jstep) {
+                                    const uint64_t a = hi | (uint64_t)(base + P.a_lo[j]);
+                                    if (FP8) {
+                                        mma_fp8(d, a, hi | (uint64_t)b_lo, id_a, 1u);
+                                        mma_fp8(tmem, a, hi | (uint64_t)(b_lo + b_off), id_b, 1u);
+                                    } else {
+                                        mma_bf16(d, a, hi | (uint64_t)b_lo, id_a, 1u);
+                                        mma_bf16(tmem, a, hi | (uint64_t)(b_lo + b_off), id_b, 1u);
+                                    }
                                 }
                             }
+                            // the group's rows are consumed and its output rows final
+                            if (gin + 1 == P.grp) mma_commit(smem_u32(&bars_g[k & 15]));
                         }
                         ring_next(slot, ph, P.nslot);
                         if (++blk == P.nb) blk = 0;
                         if (++gin == P.grp) {
-                            // the group's rows are consumed and its output rows final
-                            mma_commit(smem_u32(&bars_g[k & 15]));
                             gin = 0;
                             ++k;
                         }
                     }
                 }
-                if (ok && gin > 0) mma_commit(smem_u32(&bars_g[k & 15]));   // the last, partial group
+                if (ok && gin > 0 && elect_one())
+                    mma_commit(smem_u32(&bars_g[k & 15]));   // the last, partial group
             } else {
             TileWalk w;
             w.init(P, t_begin);
@@ -519,7 +509,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                     if (++end_slot == P.nslot) end_slot = 0;
                 }
                 for (; waited < loaded; ++waited) {
-                    if (!mbar_wait(b_hfull(wslot), wphase, &abort_flag, P.status)) {
+                    if (!warp_wait(b_hfull(wslot), wphase, &abort_flag, P.status)) {
                         ok = false;
                         break;
                     }
@@ -527,7 +517,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 }
                 if (!ok) break;
                 const int ab = i & (P.nacc - 1);
-                if (!mbar_wait(b_aempty(ab), ((i >> P.acc_shift) & 1) ^ 1, &abort_flag, P.status))
+                if (!warp_wait(b_aempty(ab), ((i >> P.acc_shift) & 1) ^ 1, &abort_flag, P.status))
                     break;
                 tc_fence_after();
                 // the tile's rows y+row0 .. y+row0+rows+rpt-2 are the last rows+rpt-1 loads;
@@ -535,6 +525,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 int s0 = end_slot - (P.rows + P.rpt - 1);
                 if (s0 < 0) s0 += P.nslot;
                 const uint32_t b_adv = (uint32_t)nis * b_step;
+                if (elect_one())
                 for (int r = 0; r < P.rpt; ++r) {
                     const uint32_t d =
                         tmem + (uint32_t)(((ab * P.rpt + r) * nis + iss) * P.n_slice);
@@ -544,12 +535,12 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                     uint32_t b_lo = b_lo0 + (uint32_t)iss * b_step;
                     uint32_t base = ring16 + (uint32_t)sr * slot16;
                     int j = iss;
-                    uint32_t e = alo_s[j];
+                    uint32_t e = P.a_lo[j];
                     for (int ks = iss; ks < P.nks; ks += nis) {
                         int jn = j + nis;                              // next position, read ahead
                         const bool wrap = jn >= ks_row;
                         if (wrap) jn -= ks_row;
-                        const uint32_t e_next = alo_s[jn];
+                        const uint32_t e_next = P.a_lo[jn];
                         const uint64_t a = hi | (uint64_t)(base + e);
                         const uint64_t b = hi | (uint64_t)b_lo;
                         if (FP8) mma_fp8(d, a, b, P.idesc, ks >= nis ? 1u : 0u);
@@ -573,16 +564,16 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                            (P.rows + P.rpt - 1);
                 }
                 for (; released < keep; ++released) {
-                    mma_commit(b_hempty(rslot));
+                    if (elect_one()) mma_commit(b_hempty(rslot));
                     if (++rslot == P.nslot) rslot = 0;
                 }
-                mma_commit(b_afull(ab));
+                if (elect_one()) mma_commit(b_afull(ab));
                 w = w2;
             }
             }
             // wait until every MMA issued above (by both issuers) has completed
-            mma_commit(b_done);
-            mbar_wait(b_done, 0, &abort_flag, P.status, false);
+            if (elect_one()) mma_commit(b_done);
+            warp_wait(b_done, 0, &abort_flag, P.status, false);
         }
     } else if ((warp >= 2 && warp <= 5) || (STREAM && warp >= 6 && warp <= 9)) {
         // epilogue: warps 2..5 own TMEM lanes 32*(warp%4) ..; one lane per warp polls

@@ -64,6 +64,34 @@ __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_fla
     }
 }
 
+// True in one lane of a converged warp.  Roles that issue MMAs and TMA loads run as whole warps
+// with uniform control flow (waits and counters in every lane, warp_wait) and put only the
+// issuing instructions under elect_one(): the compiler then keeps descriptors and addresses in
+// uniform registers.  Issued from a lane == 0 branch instead, every operand of every MMA went
+// through a loop that makes it uniform, and one 128-pixel row cost the issuing thread 800 cycles.
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "elect.sync _|p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(p));
+    return p != 0;
+}
+
+// mbar_wait by a whole converged warp; the result is warp-uniform.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                          unsigned* status, bool heed_abort = true) {
+    if (__all_sync(0xffffffffu, mbar_try(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status, heed_abort));
+}
+
+// This thread's warp number and a value of a converged warp, known to the compiler as uniform.
+__device__ __forceinline__ int warp_number() {
+    return __shfl_sync(0xffffffffu, (int)(threadIdx.x / 32), 0);
+}
+__device__ __forceinline__ uint32_t uniform(uint32_t v) { return __shfl_sync(0xffffffffu, v, 0); }
+
 __device__ __forceinline__ void tma_load_5d(uint32_t dst, const CUtensorMap* map, int c0, int c1,
                                             int c2, int c3, int c4, uint32_t bar) {
     asm volatile(

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(WG_NT, 1)
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
 
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+    const int warp = warp_number(), lane = threadIdx.x % 32;
     const uint32_t s0 = smem_u32(smem);
     auto b_full = [&](int i) { return smem_u32(&bars[i]); };
     auto b_empty = [&](int i) { return smem_u32(&bars[2 + i]); };
@@ -135,64 +135,68 @@ __global__ void __launch_bounds__(WG_NT, 1)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
+    const uint32_t tmem = uniform(tmem_slot);
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             int nloads = 0;
             for (int t = t_begin, i = 0; t < t_end; ++t, ++i) {
                 const int st = i & 1;
-                if (!mbar_wait(b_empty(st), ((i >> 1) & 1) ^ 1u, &abort_flag, P.status)) break;
+                if (!warp_wait(b_empty(st), ((i >> 1) & 1) ^ 1u, &abort_flag, P.status)) break;
                 const int xt = t % P.tiles_x;
                 const int row = t / P.tiles_x;
                 const int y = row % P.h, img = row / P.h;
                 const int x0 = xt * 128;
                 const uint32_t sa = s0 + (uint32_t)st * P.stage_bytes;
                 const uint32_t sb = sa + P.a_bytes;
-                mbar_expect_tx(b_full(st), P.a_bytes + P.b_bytes);
-                if (P.mode == 0) {
-                    tma_load_4d(sa, &tg, 2 * x0, 0, y, img, b_full(st));
-                    for (int dy = 0; dy < 3; ++dy)
-                        for (int dx = 0; dx < 3; ++dx)
-                            tma_load_4d(sb + (uint32_t)(3 * dy + dx) * 2 * WG_PLANE, tx,
-                                        2 * (x0 - 1 + dx), plane0, y + dy - 1, img, b_full(st));
-                } else {
-                    // kernel position (a, b): output row 2y + a, output pixels 2j + b
-                    const uint32_t ab_bytes = P.a_bytes / (uint32_t)P.n_ab;
-                    for (int k = 0; k < P.n_ab; ++k) {
-                        const int ab = ab0 + k;
-                        tma_load_5d(sa + (uint32_t)k * ab_bytes, &tg, 0, ab & 1, x0, P.g_plane0,
-                                    (img * P.h + y) * 2 + (ab >> 1), b_full(st));
+                if (elect_one()) {
+                    mbar_expect_tx(b_full(st), P.a_bytes + P.b_bytes);
+                    if (P.mode == 0) {
+                        tma_load_4d(sa, &tg, 2 * x0, 0, y, img, b_full(st));
+                        for (int dy = 0; dy < 3; ++dy)
+                            for (int dx = 0; dx < 3; ++dx)
+                                tma_load_4d(sb + (uint32_t)(3 * dy + dx) * 2 * WG_PLANE, tx,
+                                            2 * (x0 - 1 + dx), plane0, y + dy - 1, img, b_full(st));
+                    } else {
+                        // kernel position (a, b): output row 2y + a, output pixels 2j + b
+                        const uint32_t ab_bytes = P.a_bytes / (uint32_t)P.n_ab;
+                        for (int k = 0; k < P.n_ab; ++k) {
+                            const int ab = ab0 + k;
+                            tma_load_5d(sa + (uint32_t)k * ab_bytes, &tg, 0, ab & 1, x0, P.g_plane0,
+                                        (img * P.h + y) * 2 + (ab >> 1), b_full(st));
+                        }
+                        tma_load_4d(sb, &t1, 2 * x0, 0, y, img, b_full(st));
                     }
-                    tma_load_4d(sb, &t1, 2 * x0, 0, y, img, b_full(st));
                 }
                 ++nloads;
             }
             // the last loads issued must land before the CTA may exit
             const int last = nloads;
             for (int i = last - 2 < 0 ? 0 : last - 2; i < last; ++i)
-                mbar_wait(b_full(i & 1), (i >> 1) & 1, &abort_flag, P.status, false);
+                warp_wait(b_full(i & 1), (i >> 1) & 1, &abort_flag, P.status, false);
         }
     } else if (warp == 1) {
-        if (lane == 0 && t_end > t_begin) {
+        if (t_end > t_begin) {
             bool ok = true;
             for (int t = t_begin, i = 0; ok && t < t_end; ++t, ++i) {
                 const int st = i & 1;
-                if (!mbar_wait(b_full(st), (i >> 1) & 1, &abort_flag, P.status)) {
+                if (!warp_wait(b_full(st), (i >> 1) & 1, &abort_flag, P.status)) {
                     ok = false;
                     break;
                 }
                 tc_fence_after();
                 const uint32_t sa = s0 + (uint32_t)st * P.stage_bytes;
                 const uint32_t sb = sa + P.a_bytes;
+                if (elect_one()) {
 #pragma unroll
-                for (int ks = 0; ks < 8; ++ks)   // 16 pixels per K-step
-                    mma_bf16(tmem, wg_desc(sa + 256u * ks), wg_desc(sb + 256u * ks), P.idesc,
-                             (i > 0 || ks > 0) ? 1u : 0u);
-                mma_commit(b_empty(st));
+                    for (int ks = 0; ks < 8; ++ks)   // 16 pixels per K-step
+                        mma_bf16(tmem, wg_desc(sa + 256u * ks), wg_desc(sb + 256u * ks), P.idesc,
+                                 (i > 0 || ks > 0) ? 1u : 0u);
+                    mma_commit(b_empty(st));
+                }
             }
-            mma_commit(b_done);
-            mbar_wait(b_done, 0, &abort_flag, P.status, false);
+            if (elect_one()) mma_commit(b_done);
+            warp_wait(b_done, 0, &abort_flag, P.status, false);
         }
     } else {
         // epilogue: TMEM lane o (warp quadrant q = warp % 4) holds dW[o][tap][16 channels]
