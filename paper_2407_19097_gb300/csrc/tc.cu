@@ -67,6 +67,7 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "net.h"
 #include "project.cuh"
@@ -189,6 +190,19 @@ struct TileWalk {
         }
     }
 };
+
+// Row streaming: slots (input rows) of a run of tiles: it splits into segments, one per tile
+// column, and a segment of R output rows streams R + 2 input rows.
+__device__ __forceinline__ int stream_slots(const TcParams& P, int t_begin, int t_end) {
+    int s = 0;
+    for (int t = t_begin; t < t_end;) {
+        const int col = t / P.hr;
+        const int te = t_end < (col + 1) * P.hr ? t_end : (col + 1) * P.hr;
+        s += (te - t) * P.rpt + 2;
+        t = te;
+    }
+    return s;
+}
 
 // Two floats as a BF16 pair (lo in the low half), rounded to nearest; with relu, negative
 // values (and -0) become +0 in the same conversion.
@@ -422,73 +436,90 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
             const int nis = P.nissue;
             if (STREAM) {
                 // B of one row K-step: 3 n_slice rows, halves 3 n_slice * 16 bytes apart
-                const uint32_t b_lbo3 = (uint32_t)P.n_slice * 48;
-                const uint32_t b_lo0s = ((s_w >> 4) & 0x3FFFu) | ((b_lbo3 >> 4) << 16);
-                const uint32_t b_jstep = (2 * b_lbo3) >> 4;
-                const uint32_t b_n1 = (uint32_t)P.n_slice;   // n_slice rows of B, in 16 bytes
-                const uint32_t ns = (uint32_t)P.n_slice;
-                int slot = 0, blk = 0, gin = 0, k = 0;
-                uint32_t ph = 0;
-                // segments: runs of tiles in one tile column; a segment of R output rows
-                // streams its R + 2 input rows, whose slots hold output rows y0 - 2 .. y0 + R - 1
-                for (int t = t_begin; ok && t < t_end;) {
-                    const int col = t / P.hr;
-                    const int te = t_end < (col + 1) * P.hr ? t_end : (col + 1) * P.hr;
-                    const int nrows = (te - t) * P.rpt + 2;
-                    t = te;
-                    for (int r = 0; r < nrows; ++r) {
-                        if (gin == 0 && k >= P.gm) {
-                            // the blocks this group writes were last drained in group k - gm
+                const uint32_t ns = (uint32_t)P.n_slice;   // n_slice rows of B, in 16 bytes
+                const uint32_t b_lo0s = ((s_w >> 4) & 0x3FFFu) | ((3 * ns) << 16);
+                const uint32_t b_jstep = 6 * ns;
+                // the input rows of every segment (R + 2 for R output rows) in one sequence
+                const int S = stream_slots(P, t_begin, t_end);
+                // KS: K-steps of a row known at compile time (0: not), so that a row's MMAs are
+                // straight code with the descriptor words in uniform registers
+                auto issue = [&](auto ks_const) {
+                    constexpr int KS = decltype(ks_const)::value;
+                    const int ksr = KS ? KS : ks_row;
+                    uint32_t alo[KS ? KS : 1];
+#pragma unroll
+                    for (int j = 0; j < KS; ++j) alo[j] = P.a_lo[j];
+                    uint32_t base = ring16, d = tmem, ph = 0;
+                    int slot = 0, blk = 0, q = 0;
+                    for (int k = 0; q < S; ++k) {
+                        // the blocks this group writes were last drained in group k - gm
+                        if (k >= P.gm) {
                             const int kk = k - P.gm;
                             if (!warp_wait(b_aempty(kk & 3), (kk >> 2) & 1, &abort_flag, P.status)) {
                                 ok = false;
-                                break;
+                                return;
                             }
                         }
-                        if (!warp_wait(b_hfull(slot), ph, &abort_flag, P.status)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
-                        const uint32_t base = ring16 + (uint32_t)slot * slot16;
-                        const uint32_t d = tmem + (uint32_t)blk * ns;
-                        uint32_t b_lo = b_lo0s;
-                        if (elect_one()) {
-                            if (blk <= P.nb - 3) {
-                                for (int j = 0; j < ks_row; ++j, b_lo += b_jstep) {
-                                    const uint64_t a = hi | (uint64_t)(base + P.a_lo[j]);
-                                    if (FP8) mma_fp8(d, a, hi | (uint64_t)b_lo, P.idesc, 1u);
-                                    else mma_bf16(d, a, hi | (uint64_t)b_lo, P.idesc, 1u);
-                                }
-                            } else {
-                                // the three blocks wrap around the ring: two MMAs per K-step
-                                const uint32_t id_a = blk == P.nb - 2 ? P.idesc2 : P.idesc1;
-                                const uint32_t id_b = blk == P.nb - 2 ? P.idesc1 : P.idesc2;
-                                const uint32_t b_off = blk == P.nb - 2 ? 2 * b_n1 : b_n1;
-                                for (int j = 0; j < ks_row; ++j, b_lo += b_jstep) {
-                                    const uint64_t a = hi | (uint64_t)(base + P.a_lo[j]);
-                                    if (FP8) {
-                                        mma_fp8(d, a, hi | (uint64_t)b_lo, id_a, 1u);
-                                        mma_fp8(tmem, a, hi | (uint64_t)(b_lo + b_off), id_b, 1u);
-                                    } else {
-                                        mma_bf16(d, a, hi | (uint64_t)b_lo, id_a, 1u);
-                                        mma_bf16(tmem, a, hi | (uint64_t)(b_lo + b_off), id_b, 1u);
+                        const int qe = q + P.grp < S ? q + P.grp : S;
+                        for (; q < qe; ++q) {
+                            if (!warp_wait(b_hfull(slot), ph, &abort_flag, P.status)) {
+                                ok = false;
+                                return;
+                            }
+                            tc_fence_after();
+                            if (elect_one()) {
+                                if (blk <= P.nb - 3) {
+#pragma unroll
+                                    for (int j = 0; j < (KS ? KS : MAX_KS); ++j) {
+                                        if (!KS && j >= ksr) break;
+                                        const uint64_t a = hi | (uint64_t)(base + (KS ? alo[j] : P.a_lo[j]));
+                                        const uint64_t bd = hi | (uint64_t)(b_lo0s + (uint32_t)j * b_jstep);
+                                        if (FP8) mma_fp8(d, a, bd, P.idesc, 1u);
+                                        else mma_bf16(d, a, bd, P.idesc, 1u);
+                                    }
+                                } else {
+                                    // the three blocks wrap around the ring: two MMAs per K-step
+                                    const bool two = blk == P.nb - 2;
+                                    const uint32_t id_a = two ? P.idesc2 : P.idesc1;
+                                    const uint32_t id_b = two ? P.idesc1 : P.idesc2;
+                                    const uint32_t b_off = two ? 2 * ns : ns;
+                                    uint32_t b_lo = b_lo0s;
+                                    for (int j = 0; j < ksr; ++j, b_lo += b_jstep) {
+                                        const uint64_t a = hi | (uint64_t)(base + P.a_lo[j]);
+                                        const uint64_t b0 = hi | (uint64_t)b_lo, b1 = hi | (uint64_t)(b_lo + b_off);
+                                        if (FP8) {
+                                            mma_fp8(d, a, b0, id_a, 1u);
+                                            mma_fp8(tmem, a, b1, id_b, 1u);
+                                        } else {
+                                            mma_bf16(d, a, b0, id_a, 1u);
+                                            mma_bf16(tmem, a, b1, id_b, 1u);
+                                        }
                                     }
                                 }
+                                // the group's rows are consumed and its output rows final
+                                if (q + 1 == qe) mma_commit(smem_u32(&bars_g[k & 15]));
                             }
-                            // the group's rows are consumed and its output rows final
-                            if (gin + 1 == P.grp) mma_commit(smem_u32(&bars_g[k & 15]));
-                        }
-                        ring_next(slot, ph, P.nslot);
-                        if (++blk == P.nb) blk = 0;
-                        if (++gin == P.grp) {
-                            gin = 0;
-                            ++k;
+                            base += slot16;
+                            d += ns;
+                            if (++slot == P.nslot) {
+                                slot = 0;
+                                ph ^= 1u;
+                                base = ring16;
+                            }
+                            if (++blk == P.nb) {
+                                blk = 0;
+                                d = tmem;
+                            }
                         }
                     }
+                };
+                if (ok) {
+                    if (ks_row == 2) issue(std::integral_constant<int, 2>{});
+                    else if (ks_row == 3) issue(std::integral_constant<int, 3>{});
+                    else if (ks_row == 6) issue(std::integral_constant<int, 6>{});
+                    else if (ks_row == 12) issue(std::integral_constant<int, 12>{});
+                    else issue(std::integral_constant<int, 0>{});
                 }
-                if (ok && gin > 0 && elect_one())
-                    mma_commit(smem_u32(&bars_g[k & 15]));   // the last, partial group
             } else {
             TileWalk w;
             w.init(P, t_begin);
@@ -803,13 +834,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
             // biases, sums and the head run on pairs of channels or rows (f32x2).
             const uint32_t lanes = (uint32_t)(32 * q) << 16;
             const uint32_t ns = (uint32_t)P.n_slice;
-            int S = 0;
-            for (int tt = t_begin; tt < t_end;) {
-                const int col = tt / P.hr;
-                const int te = t_end < (col + 1) * P.hr ? t_end : (col + 1) * P.hr;
-                S += (te - tt) * P.rpt + 2;
-                tt = te;
-            }
+            const int S = stream_slots(P, t_begin, t_end);
             const int oc0 = (slice * P.n_slice) >> (GATED ? 1 : 0);   // first output channel
             const bool dec = FP8 && P.dec_scale != 0.0f;                // BF16 output of an FP8 layer
             const int nch = dec ? 2 * P.out_nch : P.out_nch;            // planes of the stored output
