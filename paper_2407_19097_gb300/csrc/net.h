@@ -138,15 +138,15 @@ nrv_status tc_upconv(const Net* net, int layer, const void* x, void* y, const Ge
                      nrv_prec prec, cudaStream_t s, float inv_out = 1.0f,
                      const TcExtra* extra = nullptr);
 nrv_status tc_repack_fp8(Net* net, cudaStream_t s);
-// TMA map of a row-planar tensor [n][h][nch][w][16 bytes] (tc.cu): boxes of 128 pixels x
+// TMA map of a row-planar tensor [n][h][nch][w][16 bytes] (tc.cu): boxes of box_px pixels x
 // box_planes planes of one row
 nrv_status tc_planar_map(CUtensorMap* map, const void* base, int n, int h, int w, int nch,
-                         int box_planes);
+                         int box_planes, int box_px = 128);
 // TMA map of the pixels of one parity b of a row-planar tensor with `rows` rows (all images)
 // of w pixels (w even) and nch planes: 8-byte elements (half, parity, pixel pair, plane, row);
-// a box is 128 pixel pairs x box_planes planes of one row at one parity (tc.cu)
+// a box is box_px pixel pairs x box_planes planes of one row at one parity (tc.cu)
 nrv_status tc_parity_map(CUtensorMap* map, const void* base, int rows, int w, int nch,
-                         int box_planes);
+                         int box_planes, int box_px = 128);
 // Weight gradient of a 2x2 stride-2 transposed conv on the tensor cores (wgrad_tc.cu):
 // part[split][c][ab * C_out + o] over the input level (n, H, W); x at (H, W), g at (2H, 2W),
 // both BF16 row-planar; g holds g_ld channels of which C_out from channel g_off on (the

@@ -1286,7 +1286,7 @@ EncodeTiledFn encode_fn() {
 // plane is a contiguous 2 KB run in global memory.  Pixels outside [0, w) and
 // rows outside [0, h) read as zero.
 nrv_status make_planar_map(CUtensorMap* map, const void* base, int n, int h, int w, int nch,
-                           int box_planes = 0) {
+                           int box_planes = 0, int box_px = TILE_M) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(NRV_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled unavailable");
     if (((uintptr_t)base & 15) != 0) return fail(NRV_ERR_ARG, "tensor base not 16-byte aligned");
@@ -1296,7 +1296,7 @@ nrv_status make_planar_map(CUtensorMap* map, const void* base, int n, int h, int
     const cuuint64_t dims[4] = {(cuuint64_t)2 * w, (cuuint64_t)nch, (cuuint64_t)h, (cuuint64_t)n};
     const cuuint64_t row = (cuuint64_t)w * 16;
     const cuuint64_t strides[3] = {row, row * nch, row * nch * h};
-    const cuuint32_t box[4] = {2 * TILE_M, (cuuint32_t)box_planes, 1, 1};
+    const cuuint32_t box[4] = {(cuuint32_t)(2 * box_px), (cuuint32_t)box_planes, 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 4, const_cast<void*>(base), dims, strides,
                      box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -2250,12 +2250,12 @@ nrv_status tc_dgrad(const Net* net, int l, const void* gin, void* out, const voi
 }
 
 nrv_status tc_planar_map(CUtensorMap* map, const void* base, int n, int h, int w, int nch,
-                         int box_planes) {
-    return make_planar_map(map, base, n, h, w, nch, box_planes);
+                         int box_planes, int box_px) {
+    return make_planar_map(map, base, n, h, w, nch, box_planes, box_px);
 }
 
 nrv_status tc_parity_map(CUtensorMap* map, const void* base, int rows, int w, int nch,
-                         int box_planes) {
+                         int box_planes, int box_px) {
     EncodeTiledFn enc = encode_fn();
     if (!enc) return fail(NRV_ERR_UNSUPPORTED, "cuTensorMapEncodeTiled unavailable");
     if (((uintptr_t)base & 15) != 0) return fail(NRV_ERR_ARG, "tensor base not 16-byte aligned");
@@ -2265,7 +2265,7 @@ nrv_status tc_parity_map(CUtensorMap* map, const void* base, int rows, int w, in
     const cuuint64_t dims[5] = {2, 2, (cuuint64_t)w / 2, (cuuint64_t)nch, (cuuint64_t)rows};
     const cuuint64_t row = (cuuint64_t)w * 16;
     const cuuint64_t strides[4] = {16, 32, row, row * nch};
-    const cuuint32_t box[5] = {2, 1, TILE_M, (cuuint32_t)box_planes, 1};
+    const cuuint32_t box[5] = {2, 1, (cuuint32_t)box_px, (cuuint32_t)box_planes, 1};
     const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
     CUresult r = enc(map, CU_TENSOR_MAP_DATA_TYPE_UINT64, 5, const_cast<void*>(base), dims, strides,
                      box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,

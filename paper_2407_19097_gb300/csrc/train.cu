@@ -306,60 +306,60 @@ __global__ void __launch_bounds__(256) wgrad_up_kernel(TView<const T> x, int cin
 }
 
 // ------------------------------------------------------------------ head
-// gd[q][c] = (sum_o drgb[o] W[o][c]) * (x[q][c] > 0) over the canvas (zero outside the view)
+// One pass over the last conv's output x and the image gradient makes both head gradients (two
+// passes read them twice, 42 us in the 16 x 256^2 step):
+//   gd[q][c] = (sum_o drgb[o] W[o][c]) * (x[q][c] > 0) over the canvas (zero outside the view);
+//   part[blk][o*16 + c] = sum drgb[o] * x[c], part[blk][48 + o] = sum drgb[o] over the block's chunk
+// of cropped pixels: every thread keeps all 51 sums, then the block adds them (warp shuffles,
+// then the 8 warps in order).
 template <typename T>
-__global__ void head_dgrad_kernel(const float* drgb, const float* w, TView<const T> x, TView<T> gd,
-                                  int n, int hn, int wn, int h, int wd) {
-    const size_t total = (size_t)n * hn * wn;
-    for (size_t q = blockIdx.x * (size_t)blockDim.x + threadIdx.x; q < total;
-         q += (size_t)gridDim.x * blockDim.x) {
-        const int X = (int)(q % wn), Y = (int)((q / wn) % hn);
-        const size_t img = q / ((size_t)wn * hn);
-        float out[16];
-        if (X < wd && Y < h) {
-            const float* gr = drgb + 3 * ((img * h + Y) * wd + X);
-            float xv[16];
-            ld8<T>(x.at(img * hn + Y, X, 0, wn), xv);
-            ld8<T>(x.at(img * hn + Y, X, 8, wn), xv + 8);
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const float s = fmaf(gr[2], w[32 + c], fmaf(gr[1], w[16 + c], gr[0] * w[c]));
-                out[c] = xv[c] > 0.0f ? s : 0.0f;
-            }
-        } else {
-#pragma unroll
-            for (int c = 0; c < 16; ++c) out[c] = 0.0f;
-        }
-        st8<T>(gd.at(img * hn + Y, X, 0, wn), out);
-        st8<T>(gd.at(img * hn + Y, X, 8, wn), out + 8);
-    }
-}
-
-// part[blk][o*16 + c] = sum drgb[o] * x[c]; part[blk][48 + o] = sum drgb[o], over the block's
-// chunk of cropped pixels: every thread keeps all 51 sums, then the block adds them (warp
-// shuffles, then the 8 warps in order).
-template <typename T>
-__global__ void __launch_bounds__(256) head_wgrad_kernel(const float* drgb, TView<const T> x, int n,
-                                                         int hn, int wn, int h, int wd,
-                                                         size_t chunk, float* part) {
+__global__ void __launch_bounds__(256) head_bwd_kernel(const float* drgb, const float* __restrict__ w,
+                                                       TView<const T> x, TView<T> gd, int n, int hn, int wn,
+                                                       int h, int wd, size_t chunk, float* part) {
     __shared__ float red[8][51];
+    __shared__ float ws[48];
+    if (threadIdx.x < 48) ws[threadIdx.x] = w[threadIdx.x];
+    __syncthreads();
     float acc[51];
 #pragma unroll
     for (int k = 0; k < 51; ++k) acc[k] = 0.0f;
     const size_t total = (size_t)n * h * wd;
     const size_t i0 = blockIdx.x * chunk, i1 = i0 + chunk < total ? i0 + chunk : total;
     for (size_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        const int X = (int)(i % wd), Y = (int)((i / wd) % h);
-        const size_t img = i / ((size_t)wd * h);
+        const uint32_t row = (uint32_t)(i / (uint32_t)wd), X = (uint32_t)(i - (size_t)row * wd);
+        const uint32_t img = row / (uint32_t)h, Y = row - img * (uint32_t)h;
+        const size_t at = (size_t)img * hn + Y;
         float v[16];
-        ld8<T>(x.at(img * hn + Y, X, 0, wn), v);
-        ld8<T>(x.at(img * hn + Y, X, 8, wn), v + 8);
+        ld8<T>(x.at(at, X, 0, wn), v);
+        ld8<T>(x.at(at, X, 8, wn), v + 8);
         const float d[3] = {drgb[3 * i], drgb[3 * i + 1], drgb[3 * i + 2]};
+        float out[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+            const float s = fmaf(d[2], ws[32 + c], fmaf(d[1], ws[16 + c], d[0] * ws[c]));
+            out[c] = v[c] > 0.0f ? s : 0.0f;
+        }
+        st8<T>(gd.at(at, X, 0, wn), out);
+        st8<T>(gd.at(at, X, 8, wn), out + 8);
 #pragma unroll
         for (int o = 0; o < 3; ++o) {
 #pragma unroll
             for (int c = 0; c < 16; ++c) acc[o * 16 + c] = fmaf(d[o], v[c], acc[o * 16 + c]);
             acc[48 + o] += d[o];
+        }
+    }
+    // the canvas margin
+    if (hn != h || wn != wd) {
+        float zero[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c) zero[c] = 0.0f;
+        const uint32_t rows = (uint32_t)n * hn;
+        for (uint32_t r = blockIdx.x; r < rows; r += gridDim.x) {
+            const int x0 = (int)(r % (uint32_t)hn) < h ? wd : 0;
+            for (int X = x0 + (int)threadIdx.x; X < wn; X += blockDim.x) {
+                st8<T>(gd.at(r, X, 0, wn), zero);
+                st8<T>(gd.at(r, X, 8, wn), zero);
+            }
         }
     }
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -869,7 +869,6 @@ struct Bwd {
         NRV_TRY(net->partial.ensure(floats * sizeof(float)));
         NRV_TRY(net_side_stream(net));
         sw = net->side;
-        NRV_TRY(point());
         const nrv_status st = layers_bwd(drgb, netin, hch, hchunk);
         const nrv_status fs = st == NRV_OK ? parts.flush(sw) : st;
         const nrv_status js = join();   // also after a failure: nothing runs on past this call
@@ -884,17 +883,14 @@ struct Bwd {
         {
             float* part = parts.take(hch * 51);
             if (!part) return fail(NRV_ERR_STATE, "partial sums");
-            head_wgrad_kernel<T><<<(unsigned)hch, 256, 0, sw>>>(drgb, CA(A_D0B), g.n, g.h[0], g.w[0], H, Wd,
-                                                               hchunk, part);
+            head_bwd_kernel<T><<<(unsigned)hch, 256, 0, s>>>(
+                drgb, (const float*)net->params.p + Lh.woff, CA(A_D0B), V(G[G_D0B], 16), g.n, g.h[0], g.w[0],
+                H, Wd, hchunk, part);
             NRV_CHECK_LAUNCH();
             // weight (48) and bias (3) are consecutive in the parameter vector
             if (Lh.boff != Lh.woff + 48) return fail(NRV_ERR_STATE, "head parameter layout");
             parts.add(ReduceSeg{part, (int)hch, 51, 51, 2, 3, 16, 16, dparams + Lh.woff});
         }
-        head_dgrad_kernel<T><<<blocks_for(g.px(0)), 256, 0, s>>>(
-            drgb, (const float*)net->params.p + Lh.woff, CA(A_D0B), V(G[G_D0B], 16), g.n, g.h[0],
-            g.w[0], H, Wd);
-        NRV_CHECK_LAUNCH();
         NRV_TRY(point());
         // level 0 decoder
         NRV_TRY(wgrad_conv(L_D0B, C(G[G_D0B], 16), CA(A_D0A), 16, none, 0, 0));

@@ -8,8 +8,10 @@
 // pixels serves all nine taps.  Both operands come straight from the row-planar BF16
 // layout ([row][plane][pixel][8 channels]), which is the MN-major no-swizzle operand
 // layout: a core matrix is 8 consecutive pixels (K) x 16 bytes (8 channels of M or N),
-// K-adjacent core matrices 128 bytes apart (LBO), MN-adjacent ones one 2 KB plane apart
-// (SBO).  A tile is 128 pixels x0..x0+127 of one row: its A block is the output gradient
+// K-adjacent core matrices 128 bytes apart (LBO), MN-adjacent ones one plane apart
+// (SBO).  A tile is 128 pixels x0..x0+127 of one row (64 or 32 where the image is narrow: at
+// level 3 of 256-pixel crops three quarters of a 128-pixel tile were padding, loaded and
+// multiplied): its A block is the output gradient
 // (all C_out planes), its B block nine shifted copies of the group's two input planes --
 // rows y-1, y, y+1 at pixel offsets -1, 0, +1 -- loaded by TMA, so the nine taps are
 // nine consecutive N blocks and zero padding is TMA's out-of-bounds fill.
@@ -29,10 +31,12 @@
 //
 // Each CTA takes a channel group and a contiguous range of tiles (a split of K), sums
 // its MMAs in one TMEM accumulator and writes its partial dW; partials are added in a
-// fixed order afterwards (deterministic).  Warp 0 issues TMA into two stages, warp 1
+// fixed order afterwards (deterministic).  Warp 0 issues TMA into two to eight stages, warp 1
 // owns TMEM and issues the MMAs, warps 2-5 read the accumulator at the end.  Waits are
 // bounded: on timeout the kernel sets STATUS_TIMEOUT, drains its copies, frees TMEM and
 // returns.
+#include <algorithm>
+
 #include "net.h"
 #include "tcgen05.cuh"
 
@@ -41,16 +45,17 @@ namespace nrv {
 namespace {
 
 constexpr int WG_NT = 192;           // producer, MMA issuer, 4 epilogue warps
-constexpr int WG_PLANE = 2048;       // one plane of a 128-pixel tile
+constexpr int WG_STAGES = 8;         // at most
 constexpr int WG_N = 144;            // 9 taps x 16 channels
-constexpr uint32_t WG_B_BYTES = 9 * 2 * WG_PLANE;
-constexpr uint32_t WG_ONES = 2 * WG_PLANE;   // two planes of ones after each B block
 constexpr int WG_COLS = 256;         // TMEM columns allocated (>= WG_N)
 
 struct WgParams {
     int mode;              // 0: 3x3 conv; 1: 2x2 stride-2 transposed conv
     int n, h, w;           // input level geometry
-    int tiles_x, ntiles;   // tiles of 128 pixels: t = (img * h + y) * tiles_x + xt
+    int tpx;               // pixels of a tile: 128, 64 or 32
+    uint32_t plane;        // bytes of one plane of a tile (tpx x 16)
+    int nst;               // stages
+    int tiles_x, ntiles;   // t = (img * h + y) * tiles_x + xt
     int nsplit;            // CTAs per channel group (blockIdx.x)
     int cout, cin;         // channels of the output gradient and of the whole input
     int groups1;           // channel groups that read source 1 (the rest read source 2)
@@ -70,10 +75,10 @@ struct WgParams {
     unsigned* status;
 };
 
-__device__ __forceinline__ uint64_t wg_desc(uint32_t saddr) {
+__device__ __forceinline__ uint64_t wg_desc(uint32_t saddr, uint32_t plane) {
     // start address, LBO = 128 bytes (K), SBO = one plane (M / N), version 1, no swizzle
     const uint64_t lo = ((saddr >> 4) & 0x3FFFu) | ((uint64_t)(128u >> 4) << 16);
-    const uint64_t hi = (uint64_t)((WG_PLANE >> 4) | (1u << 14));
+    const uint64_t hi = (uint64_t)((plane >> 4) | (1u << 14));
     return lo | (hi << 32);
 }
 
@@ -81,15 +86,15 @@ __global__ void __launch_bounds__(WG_NT, 1)
     wgrad_tc_kernel(const __grid_constant__ CUtensorMap tg, const __grid_constant__ CUtensorMap t1,
                     const __grid_constant__ CUtensorMap t2, const __grid_constant__ WgParams P) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ __align__(8) uint64_t bars[5];
+    __shared__ __align__(8) uint64_t bars[2 * WG_STAGES + 1];
     __shared__ uint32_t tmem_slot;
     __shared__ volatile int abort_flag;
 
     const int warp = warp_number(), lane = threadIdx.x % 32;
     const uint32_t s0 = smem_u32(smem);
     auto b_full = [&](int i) { return smem_u32(&bars[i]); };
-    auto b_empty = [&](int i) { return smem_u32(&bars[2 + i]); };
-    const uint32_t b_done = smem_u32(&bars[4]);
+    auto b_empty = [&](int i) { return smem_u32(&bars[WG_STAGES + i]); };
+    const uint32_t b_done = smem_u32(&bars[2 * WG_STAGES]);
 
     const int split = blockIdx.x, grp = blockIdx.y;
     const int t_begin = (int)(((long long)split * P.ntiles) / P.nsplit);
@@ -100,7 +105,7 @@ __global__ void __launch_bounds__(WG_NT, 1)
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < P.nst; ++i) {
             mbar_init(b_full(i), 1);
             mbar_init(b_empty(i), 1);
         }
@@ -112,14 +117,14 @@ __global__ void __launch_bounds__(WG_NT, 1)
         // constant parts of both stages: the ones planes (BF16 1.0), and for a one-plane
         // input the unused second plane of every tap (zero)
         const uint4 one = make_uint4(0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u);
-        for (int st = 0; st < 2; ++st) {
+        for (int st = 0; st < P.nst; ++st) {
             uint8_t* b = smem + (size_t)st * P.stage_bytes + P.a_bytes;
             uint4* ones = reinterpret_cast<uint4*>(b + P.b_bytes_span);
-            for (int i = threadIdx.x; i < (int)(WG_ONES / 16); i += WG_NT) ones[i] = one;
+            for (int i = threadIdx.x; i < 2 * P.tpx; i += WG_NT) ones[i] = one;
             if (P.mode == 0 && P.b_planes == 1)
-                for (int i = threadIdx.x; i < 9 * WG_PLANE / 16; i += WG_NT) {
-                    const int tap = i / (WG_PLANE / 16), r = i % (WG_PLANE / 16);
-                    reinterpret_cast<uint4*>(b + (size_t)tap * 2 * WG_PLANE + WG_PLANE)[r] =
+                for (int i = threadIdx.x; i < 9 * P.tpx; i += WG_NT) {
+                    const int tap = i / P.tpx, r = i % P.tpx;
+                    reinterpret_cast<uint4*>(b + (size_t)(2 * tap + 1) * P.plane)[r] =
                         make_uint4(0u, 0u, 0u, 0u);
                 }
         }
@@ -139,14 +144,14 @@ __global__ void __launch_bounds__(WG_NT, 1)
 
     if (warp == 0) {
         {
-            int nloads = 0;
-            for (int t = t_begin, i = 0; t < t_end; ++t, ++i) {
-                const int st = i & 1;
-                if (!warp_wait(b_empty(st), ((i >> 1) & 1) ^ 1u, &abort_flag, P.status)) break;
+            int nloads = 0, st = 0;
+            uint32_t ph = 1;
+            for (int t = t_begin; t < t_end; ++t) {
+                if (!warp_wait(b_empty(st), ph, &abort_flag, P.status)) break;
                 const int xt = t % P.tiles_x;
                 const int row = t / P.tiles_x;
                 const int y = row % P.h, img = row / P.h;
-                const int x0 = xt * 128;
+                const int x0 = xt * P.tpx;
                 const uint32_t sa = s0 + (uint32_t)st * P.stage_bytes;
                 const uint32_t sb = sa + P.a_bytes;
                 if (elect_one()) {
@@ -155,7 +160,7 @@ __global__ void __launch_bounds__(WG_NT, 1)
                         tma_load_4d(sa, &tg, 2 * x0, 0, y, img, b_full(st));
                         for (int dy = 0; dy < 3; ++dy)
                             for (int dx = 0; dx < 3; ++dx)
-                                tma_load_4d(sb + (uint32_t)(3 * dy + dx) * 2 * WG_PLANE, tx,
+                                tma_load_4d(sb + (uint32_t)(3 * dy + dx) * 2 * P.plane, tx,
                                             2 * (x0 - 1 + dx), plane0, y + dy - 1, img, b_full(st));
                     } else {
                         // kernel position (a, b): output row 2y + a, output pixels 2j + b
@@ -169,30 +174,42 @@ __global__ void __launch_bounds__(WG_NT, 1)
                     }
                 }
                 ++nloads;
+                if (++st == P.nst) {
+                    st = 0;
+                    ph ^= 1u;
+                }
             }
             // the last loads issued must land before the CTA may exit
-            const int last = nloads;
-            for (int i = last - 2 < 0 ? 0 : last - 2; i < last; ++i)
-                warp_wait(b_full(i & 1), (i >> 1) & 1, &abort_flag, P.status, false);
+            for (int i = nloads - P.nst < 0 ? 0 : nloads - P.nst; i < nloads; ++i)
+                warp_wait(b_full(i % P.nst), (i / P.nst) & 1, &abort_flag, P.status, false);
         }
     } else if (warp == 1) {
         if (t_end > t_begin) {
-            bool ok = true;
-            for (int t = t_begin, i = 0; ok && t < t_end; ++t, ++i) {
-                const int st = i & 1;
-                if (!warp_wait(b_full(st), (i >> 1) & 1, &abort_flag, P.status)) {
-                    ok = false;
-                    break;
-                }
+            int st = 0;
+            uint32_t ph = 0;
+            for (int t = t_begin; t < t_end; ++t) {
+                if (!warp_wait(b_full(st), ph, &abort_flag, P.status)) break;
                 tc_fence_after();
                 const uint32_t sa = s0 + (uint32_t)st * P.stage_bytes;
                 const uint32_t sb = sa + P.a_bytes;
                 if (elect_one()) {
+                    // 16 pixels per K-step
+                    const uint64_t da = wg_desc(sa, P.plane), db = wg_desc(sb, P.plane);
+                    if (P.tpx == 128) {
 #pragma unroll
-                    for (int ks = 0; ks < 8; ++ks)   // 16 pixels per K-step
-                        mma_bf16(tmem, wg_desc(sa + 256u * ks), wg_desc(sb + 256u * ks), P.idesc,
-                                 (i > 0 || ks > 0) ? 1u : 0u);
+                        for (int ks = 0; ks < 8; ++ks)
+                            mma_bf16(tmem, da + 16u * ks, db + 16u * ks, P.idesc,
+                                     (t > t_begin || ks > 0) ? 1u : 0u);
+                    } else {
+                        for (int ks = 0; ks < P.tpx / 16; ++ks)
+                            mma_bf16(tmem, da + 16u * ks, db + 16u * ks, P.idesc,
+                                     (t > t_begin || ks > 0) ? 1u : 0u);
+                    }
                     mma_commit(b_empty(st));
+                }
+                if (++st == P.nst) {
+                    st = 0;
+                    ph ^= 1u;
                 }
             }
             if (elect_one()) mma_commit(b_done);
@@ -288,10 +305,20 @@ static nrv_status wg_launch(WgParams& P, int groups, const CUtensorMap& mg, cons
     P.status = status_word();
     if (!P.status) return fail(NRV_ERR_CUDA, "status word unavailable");
     // the A descriptor spans 16 planes (M = 128) from its block: keep that inside the stage
-    P.stage_bytes = P.a_bytes + P.b_bytes_span + WG_ONES;
-    if (P.stage_bytes < 16u * WG_PLANE) P.stage_bytes = 16u * WG_PLANE;
-    const uint32_t smem = 2 * P.stage_bytes;
-    if (smem > 215 * 1024) return fail(NRV_ERR_UNSUPPORTED, "stages do not fit");
+    auto stage = [&](uint32_t plane) {
+        const uint32_t bytes = (P.a_bytes + P.b_bytes_span) / P.plane * plane + 2 * plane;
+        return bytes < 16u * plane ? 16u * plane : bytes;
+    };
+    P.stage_bytes = stage(P.plane);
+    // CTAs per SM (TMEM: 256 columns each): two where two stages of 128 pixels fit twice; the
+    // stages of narrower tiles then share that space
+    const int per_sm = 2 * stage(2048) <= 110 * 1024 ? 2 : 1;
+    const uint32_t room = per_sm == 2 ? 110 * 1024 : 215 * 1024;
+    P.nst = (int)(room / P.stage_bytes);
+    if (P.nst > WG_STAGES) P.nst = WG_STAGES;
+    if (P.nst < 2) return fail(NRV_ERR_UNSUPPORTED, "stages do not fit");
+    if (P.tpx == 128) P.nst = 2;
+    const uint32_t smem = P.nst * P.stage_bytes;
     static bool attr = false;
     if (!attr) {
         NRV_CHECK_CUDA(cudaFuncSetAttribute(wgrad_tc_kernel,
@@ -305,7 +332,6 @@ static nrv_status wg_launch(WgParams& P, int groups, const CUtensorMap& mg, cons
         NRV_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         if (sms <= 0) sms = 148;
     }
-    const int per_sm = smem <= 110 * 1024 ? 2 : 1;   // TMEM: 256 columns each
     long long ns = (long long)sms * per_sm / groups;
     if (ns < 1) ns = 1;
     if (ns > P.ntiles) ns = P.ntiles;
@@ -325,7 +351,12 @@ static nrv_status wg_geometry(WgParams& P, int n, int H, int W) {
     P.n = n;
     P.h = H;
     P.w = W;
-    P.tiles_x = (W + 127) / 128;
+    // the widest tile within a tenth of the fewest padded pixels
+    auto padded = [&](int t) { return (W + t - 1) / t * t; };
+    const int least = std::min(padded(128), std::min(padded(64), padded(32)));
+    P.tpx = 10 * padded(128) <= 11 * least ? 128 : 10 * padded(64) <= 11 * least ? 64 : 32;
+    P.plane = (uint32_t)P.tpx * 16;
+    P.tiles_x = (W + P.tpx - 1) / P.tpx;
     const long long ntiles = (long long)P.tiles_x * H * n;
     if (ntiles > 0x3FFFFFFFll) return fail(NRV_ERR_UNSUPPORTED, "too many tiles");
     P.ntiles = (int)ntiles;
@@ -358,14 +389,14 @@ nrv_status tc_wgrad(const Net* net, int l, const void* g, const void* x1, int c1
     P.m_real = L.cout;
     P.ncols = WG_N;
     P.b_planes = bp;
-    P.a_bytes = (uint32_t)(L.cout / 8) * WG_PLANE;
-    P.b_bytes = 9u * bp * WG_PLANE;
-    P.b_bytes_span = WG_B_BYTES;
+    P.a_bytes = (uint32_t)(L.cout / 8) * P.plane;
+    P.b_bytes = 9u * bp * P.plane;
+    P.b_bytes_span = 9u * 2 * P.plane;
     P.idesc = wg_idesc(WG_N + 16);
     CUtensorMap mg, m1, m2;
-    NRV_TRY(tc_planar_map(&mg, g, n, H, W, L.cout / 8, L.cout / 8));
-    NRV_TRY(tc_planar_map(&m1, x1, n, H, W, c1 / 8, bp));
-    if (c2) NRV_TRY(tc_planar_map(&m2, x2, n, H, W, c2 / 8, bp));
+    NRV_TRY(tc_planar_map(&mg, g, n, H, W, L.cout / 8, L.cout / 8, P.tpx));
+    NRV_TRY(tc_planar_map(&m1, x1, n, H, W, c1 / 8, bp, P.tpx));
+    if (c2) NRV_TRY(tc_planar_map(&m2, x2, n, H, W, c2 / 8, bp, P.tpx));
     else m2 = m1;
     return wg_launch(P, cin / (8 * bp), mg, m1, m2, (size_t)L.cout * 9 * cin, part, part_floats,
                      partb, nsplit, s);
@@ -391,14 +422,14 @@ nrv_status tc_wgrad_up(const Net* net, int l, const void* g, int g_ld, int g_off
     P.m_real = P.n_ab * L.cout;
     P.ncols = L.cin;
     P.b_planes = 2;
-    P.a_bytes = (uint32_t)P.n_ab * (L.cout / 8) * WG_PLANE;
-    P.b_bytes = (uint32_t)(L.cin / 8) * WG_PLANE;
+    P.a_bytes = (uint32_t)P.n_ab * (L.cout / 8) * P.plane;
+    P.b_bytes = (uint32_t)(L.cin / 8) * P.plane;
     P.b_bytes_span = P.b_bytes;
     P.idesc = wg_idesc(L.cin + 16);
     CUtensorMap mg, m1;
     P.g_plane0 = g_off / 8;
-    NRV_TRY(tc_parity_map(&mg, g, n * 2 * H, 2 * W, g_ld / 8, L.cout / 8));
-    NRV_TRY(tc_planar_map(&m1, x, n, H, W, L.cin / 8, L.cin / 8));
+    NRV_TRY(tc_parity_map(&mg, g, n * 2 * H, 2 * W, g_ld / 8, L.cout / 8, P.tpx));
+    NRV_TRY(tc_planar_map(&m1, x, n, H, W, L.cin / 8, L.cin / 8, P.tpx));
     return wg_launch(P, groups, mg, m1, m1, (size_t)L.cin * 4 * L.cout, part, part_floats, partb,
                      nsplit, s);
 }
