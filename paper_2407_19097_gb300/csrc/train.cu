@@ -139,6 +139,8 @@ struct ReduceSeg {
 // Every segment in one launch: block b belongs to the segment whose range of blocks holds it.
 // Each thread reads eight chunks of four sums before it adds them, so the pass is bound by the
 // partials' bytes (123 MB in the 16 x 256^2 training step) and not by a chain of dependent loads.
+// Before the search by halves and the batched loads of the odd segments, single blocks with
+// chains of dependent loads ran 78k cycles against a mean of 27k (45 us; now 27).
 constexpr int MAX_SEGS = 2 * NUM_LAYERS;
 struct ReduceTable {
     int n;
@@ -168,8 +170,12 @@ __device__ __forceinline__ void reduce_put(const ReduceSeg& R, int i, float t) {
 
 __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_constant__ ReduceTable T) {
     __shared__ float red[8][132];
-    int k = 0;
-    while ((int)blockIdx.x >= T.first[k + 1]) ++k;
+    int k = 0, end = T.n;      // first[k] <= block < first[end]
+    while (end - k > 1) {
+        const int mid = (k + end) >> 1;
+        if ((int)blockIdx.x >= T.first[mid]) k = mid;
+        else end = mid;
+    }
     const ReduceSeg& R = T.seg[k];
     const int tx = threadIdx.x, ty = threadIdx.y, blk = (int)blockIdx.x - T.first[k];
     if (reduce_vec(R)) {
@@ -203,25 +209,36 @@ __global__ void __launch_bounds__(256) reduce_partials_kernel(const __grid_const
         reduce_put(R, blk * 128 + t, a);
         return;
     }
+    // The few odd segments (the head's 51 sums, biases of transposed convs) have the longest
+    // chains of chunks, and their blocks end last.
     const int i = blk * 32 + tx;
     float s = 0.0f;
-    if (i < R.count)
-        for (int c0 = ty; c0 < R.nchunks; c0 += 64) {
-            float v[8];
+    auto eight = [&](int c0, int off, float (&v)[8]) {
+        const float* pc = R.part + (size_t)c0 * R.stride + off + i;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const int ch = c0 + 8 * j;
-                v[j] = 0.0f;
-                if (ch < R.nchunks) {
-                    const float* pc = R.part + (size_t)ch * R.stride;
-                    if (R.mode == 3)
-                        v[j] = ((pc[i] + pc[R.cout + i]) + pc[2 * R.cout + i]) + pc[3 * R.cout + i];
-                    else v[j] = pc[i];
-                }
-            }
-#pragma unroll
-            for (int j = 0; j < 8; ++j) s += v[j];
+        for (int j = 0; j < 8; ++j) {
+            v[j] = 0.0f;
+            if (c0 + 8 * j < R.nchunks) v[j] = __ldcs(pc + (size_t)(8 * j) * R.stride);
         }
+    };
+    if (i < R.count) {
+        if (R.mode == 3) {
+            for (int c0 = ty; c0 < R.nchunks; c0 += 64) {
+                float v[4][8];
+#pragma unroll
+                for (int ab = 0; ab < 4; ++ab) eight(c0, ab * R.cout, v[ab]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s += ((v[0][j] + v[1][j]) + v[2][j]) + v[3][j];
+            }
+        } else {
+            for (int c0 = ty; c0 < R.nchunks; c0 += 64) {
+                float v[8];
+                eight(c0, 0, v);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) s += v[j];
+            }
+        }
+    }
     red[ty][tx] = s;
     __syncthreads();
     if (ty != 0 || i >= R.count) return;
