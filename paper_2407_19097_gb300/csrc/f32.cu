@@ -22,6 +22,8 @@
 //  * Where the tiles of a layer are fewer than the SMs can hold (the deep levels), the input
 //    channels are split over a cluster of KS blocks, whose sums are added through distributed
 //    shared memory in rank order (deterministic).
+#include <atomic>
+
 #include <cooperative_groups.h>
 #include <string.h>
 
@@ -57,7 +59,7 @@ __device__ __forceinline__ void cp16(uint32_t dst, const void* src, bool ok) {
                  : "memory");
 }
 
-template <int MODE, int OCB, int TW>
+template <int MODE, int OCB, int TW, int NB>   // NB threads
 struct F32Tile {
     static constexpr int HALO = MODE == 0 ? 1 : 0;
     static constexpr int TAPS = MODE == 0 ? 9 : 1;
@@ -65,7 +67,7 @@ struct F32Tile {
     static constexpr int GX = TW / 8;                  // pixel groups per row
     static constexpr int RQ = 8 / GX;                  // rows of a quarter-warp
     static constexpr int RW = RQ * (4 / OG);           // rows of a warp
-    static constexpr int TH = RW * (NT / 32);
+    static constexpr int TH = RW * (NB / 32);
     static constexpr int COLS = TW + 2 * HALO, ROWS = TH + 2 * HALO;
     static constexpr int RAW = (COLS - 1) * 32 + ((COLS - 1) / 8) * 16 + 32;
     // two rows per quarter-warp: the second one 64 bytes off in the banks
@@ -73,15 +75,15 @@ struct F32Tile {
     static constexpr int IN_BYTES = ROWS * RS;
     static constexpr int W_BYTES = TAPS * CK * OCB * 4;
     static constexpr int STAGE = IN_BYTES + W_BYTES;
-    static constexpr int RED = NT * 64 * 4;            // a block's sums, for the cluster
+    static constexpr int RED = NB * 64 * 4;            // a block's sums, for the cluster
     static constexpr int SMEM1 = 2 * STAGE;
     static constexpr int SMEMK = SMEM1 > RED ? SMEM1 : RED;
     static_assert(RS >= RAW && RS % 16 == 0 && (RQ == 1 || RS % 128 == 64), "row stride");
 };
 
-template <int MODE, int OCB, int TW>
-__global__ void __launch_bounds__(NT, 2) conv_f32_kernel(const __grid_constant__ F32Args a) {
-    using T = F32Tile<MODE, OCB, TW>;
+template <int MODE, int OCB, int TW, int NB>
+__global__ void __launch_bounds__(NB, 512 / NB) conv_f32_kernel(const __grid_constant__ F32Args a) {
+    using T = F32Tile<MODE, OCB, TW, NB>;
     namespace cg = cooperative_groups;
     extern __shared__ __align__(128) uint8_t smem[];
     const uint32_t s0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
@@ -114,7 +116,7 @@ __global__ void __launch_bounds__(NT, 2) conv_f32_kernel(const __grid_constant__
             src = a.x2 + (ch - a.c1);
             ld = a.ld2;
         }
-        for (int i = tid; i < T::ROWS * T::COLS * 2; i += NT) {
+        for (int i = tid; i < T::ROWS * T::COLS * 2; i += NB) {
             const int q = i & 1, pp = i >> 1, r = pp / T::COLS, p = pp - r * T::COLS;
             const int y = y0 + r - T::HALO, x = x0 + p - T::HALO;
             const bool ok = (unsigned)y < (unsigned)hh && (unsigned)x < (unsigned)ww;
@@ -123,7 +125,7 @@ __global__ void __launch_bounds__(NT, 2) conv_f32_kernel(const __grid_constant__
             cp16(base + r * T::RS + p * 32 + (p >> 3) * 16 + q * 16, s, ok);
         }
         const uint32_t wb = base + T::IN_BYTES;
-        for (int i = tid; i < T::TAPS * CK * (OCB / 4); i += NT) {
+        for (int i = tid; i < T::TAPS * CK * (OCB / 4); i += NB) {
             const int n4 = i % (OCB / 4), kc = i / (OCB / 4);   // kc = tap * CK + c
             const float* s;
             if (MODE == 1) {
@@ -223,8 +225,8 @@ __global__ void __launch_bounds__(NT, 2) conv_f32_kernel(const __grid_constant__
     ulonglong2* red = reinterpret_cast<ulonglong2*>(smem);
 #pragma unroll
     for (int p = 0; p < 8; ++p) {
-        red[(2 * p) * NT + tid] = make_ulonglong2(acc[p][0], acc[p][1]);
-        red[(2 * p + 1) * NT + tid] = make_ulonglong2(acc[p][2], acc[p][3]);
+        red[(2 * p) * NB + tid] = make_ulonglong2(acc[p][0], acc[p][1]);
+        red[(2 * p + 1) * NB + tid] = make_ulonglong2(acc[p][2], acc[p][3]);
     }
     cg::cluster_group cl = cg::this_cluster();
     cl.sync();
@@ -233,7 +235,7 @@ __global__ void __launch_bounds__(NT, 2) conv_f32_kernel(const __grid_constant__
         float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         for (int r = 0; r < ks; ++r) {
             const float4* q = reinterpret_cast<const float4*>(cl.map_shared_rank(smem, r));
-            const float4 u0 = q[(2 * p) * NT + tid], u1 = q[(2 * p + 1) * NT + tid];
+            const float4 u0 = q[(2 * p) * NB + tid], u1 = q[(2 * p + 1) * NB + tid];
             v[0] += u0.x; v[1] += u0.y; v[2] += u0.z; v[3] += u0.w;
             v[4] += u1.x; v[5] += u1.y; v[6] += u1.z; v[7] += u1.w;
         }
@@ -242,9 +244,25 @@ __global__ void __launch_bounds__(NT, 2) conv_f32_kernel(const __grid_constant__
     cl.sync();   // no block leaves while a peer reads its sums
 }
 
-template <int MODE, int OCB, int TW>
+// Allows `kern` `bytes` of dynamic shared memory on the current device, once per device.
+template <typename K>
+nrv_status allow_smem(K kern, int bytes, std::atomic<uint64_t>& done) {
+    int dev = 0;
+    NRV_CHECK_CUDA(cudaGetDevice(&dev));
+    const uint64_t bit = dev < 64 ? 1ull << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return NRV_OK;
+    NRV_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+    done.fetch_or(bit, std::memory_order_release);
+    return NRV_OK;
+}
+
+// Two blocks of 128 threads or one of 256 to an SM: a grid that needs no more asks for the shared
+// memory that keeps others out, because clusters are otherwise packed two (four) blocks to an
+// SM while SMs stay empty.
+template <int MODE, int OCB, int TW, int NB>
 nrv_status launch_tile(F32Args& a, cudaStream_t s) {
-    using T = F32Tile<MODE, OCB, TW>;
+    using T = F32Tile<MODE, OCB, TW, NB>;
+    constexpr int SPREAD = NB == 128 ? 80 * 1024 : 120 * 1024;
     a.tiles_x = (a.w + TW - 1) / TW;
     a.tiles_y = (a.h + T::TH - 1) / T::TH;
     const long long tiles = (long long)a.tiles_x * a.tiles_y * a.n;
@@ -253,17 +271,16 @@ nrv_status launch_tile(F32Args& a, cudaStream_t s) {
     // split the input channels while the blocks do not fill the SMs (two blocks each)
     int ks = 1;
     while (ks < 8 && tiles * ob * ks < 256 && 2 * ks <= nst) ks *= 2;
-    static bool attr = false;
-    auto kern = conv_f32_kernel<MODE, OCB, TW>;
-    if (!attr) {
-        NRV_CHECK_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEMK));
-        attr = true;
-    }
+    static std::atomic<uint64_t> attr{0};
+    auto kern = conv_f32_kernel<MODE, OCB, TW, NB>;
+    const nrv_status st = allow_smem(kern, T::SMEMK > SPREAD ? T::SMEMK : SPREAD, attr);
+    if (st != NRV_OK) return st;
     cudaLaunchConfig_t cfg;
     memset(&cfg, 0, sizeof(cfg));
     cfg.gridDim = dim3((unsigned)tiles, ob, ks);
-    cfg.blockDim = dim3(NT);
+    cfg.blockDim = dim3(NB);
     cfg.dynamicSmemBytes = ks > 1 ? T::SMEMK : (nst > 1 ? T::SMEM1 : T::STAGE);
+    if (NB == 128 && cfg.dynamicSmemBytes < SPREAD) cfg.dynamicSmemBytes = SPREAD;
     cfg.stream = s;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -277,15 +294,28 @@ nrv_status launch_tile(F32Args& a, cudaStream_t s) {
     return NRV_OK;
 }
 
+// Blocks of 128 threads (half the tile) where 256-thread blocks split eight ways would not give
+// every SM one. 128 channels at 2 x 32^2 pixels, 256 blocks of 128 against 128 of 256 threads:
+// 21.4 us against 34.7 (64 channels in: 15.0 against 22.6).
+template <int MODE, int OCB, int TW>
+nrv_status launch_block(F32Args& a, cudaStream_t s) {
+    constexpr int TH = F32Tile<MODE, OCB, TW, NT>::TH;
+    const long long tiles = (long long)((a.w + TW - 1) / TW) * ((a.h + TH - 1) / TH) * a.n;
+    int ks = 1;
+    while (ks < 8 && 2 * ks <= a.cin / CK) ks *= 2;
+    if (OCB == 32 && tiles * (a.ncols / OCB) * ks <= 152) return launch_tile<MODE, OCB, TW, OCB == 32 ? 128 : NT>(a, s);
+    return launch_tile<MODE, OCB, TW, NT>(a, s);
+}
+
 // The tile width that covers the image with the fewest pixels (64 where equal).
 template <int MODE, int OCB>
 nrv_status launch_width(F32Args& a, cudaStream_t s) {
     auto area = [&](int tw, int th) {
         return (long long)((a.w + tw - 1) / tw * tw) * ((a.h + th - 1) / th * th);
     };
-    if (area(32, F32Tile<MODE, OCB, 32>::TH) < area(64, F32Tile<MODE, OCB, 64>::TH))
-        return launch_tile<MODE, OCB, 32>(a, s);
-    return launch_tile<MODE, OCB, 64>(a, s);
+    if (area(32, F32Tile<MODE, OCB, 32, NT>::TH) < area(64, F32Tile<MODE, OCB, 64, NT>::TH))
+        return launch_block<MODE, OCB, 32>(a, s);
+    return launch_block<MODE, OCB, 64>(a, s);
 }
 
 template <int MODE>
@@ -300,13 +330,17 @@ nrv_status launch_mode(F32Args& a, cudaStream_t s) {
 // x 16 output channels x 9 taps over a contiguous run of 32 x 8 pixel tiles.  Thread (slice,
 // dy, channel pair) walks one row of the tile with 3 dx x 2 c x 16 o sums: a window of three
 // pixels slides along the row, so each step reads one new channel pair and 16 gradients for 48
-// paired FMAs (the first form read 2 quads for 16).  The eight slices are added in order.
+// paired FMAs; the row is unrolled, so the window is register names and not moves.  The eight
+// slices are added in order, through shared memory laid out [sum][thread]: with a thread's sums
+// side by side the writes met in one bank (70% of all shared wavefronts).  16 x 16 channels over
+// 2 x 256^2 pixels: 36 us before, 22 now (0.60 GFLOP: 8 us of the FP32 pipe).
 constexpr int WT = 192;              // 8 slices x 3 kernel rows x 8 channel pairs
 constexpr int WTW = 32, WTH = 8;     // tile
 constexpr int WXRS = (WTW + 2) * 64 + 64;   // 64 bytes off per row in the banks
 constexpr int WX_BYTES = (WTH + 2) * WXRS, WG_BYTES = WTH * WTW * 64;
 constexpr int WSTAGE = WX_BYTES + WG_BYTES;
-constexpr int WRED = WT * 96 * 4;
+constexpr int WRLD = WT + 1;         // the odd pair count sets the two channels of a pair 16 banks apart
+constexpr int WRED = 48 * WRLD * 8;
 constexpr int WSMEM = 2 * WSTAGE > WRED ? 2 * WSTAGE : WRED;
 
 struct F32Wgrad {
@@ -377,9 +411,9 @@ __global__ void __launch_bounds__(WT, 2) wgrad_f32_kernel(const __grid_constant_
         };
         take(0, win[0]);
         take(1, win[1]);
-#pragma unroll 2
+#pragma unroll
         for (int p = 0; p < WTW; ++p) {
-            take(p + 2, win[2]);
+            take(p + 2, win[(p + 2) % 3]);
             const ulonglong2* gp = reinterpret_cast<const ulonglong2*>(gr + p * 64);
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
@@ -388,38 +422,34 @@ __global__ void __launch_bounds__(WT, 2) wgrad_f32_kernel(const __grid_constant_
                 for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
                     for (int c = 0; c < 2; ++c) {
-                        acc[dx][c][2 * k] = f2_fma(win[dx][c], gv.x, acc[dx][c][2 * k]);
-                        acc[dx][c][2 * k + 1] = f2_fma(win[dx][c], gv.y, acc[dx][c][2 * k + 1]);
+                        const f2 xv = win[(p + dx) % 3][c];
+                        acc[dx][c][2 * k] = f2_fma(xv, gv.x, acc[dx][c][2 * k]);
+                        acc[dx][c][2 * k + 1] = f2_fma(xv, gv.y, acc[dx][c][2 * k + 1]);
                     }
-            }
-#pragma unroll
-            for (int c = 0; c < 2; ++c) {
-                win[0][c] = win[1][c];
-                win[1][c] = win[2][c];
-            }
-        }
+            }        }
         if (blockIdx.z == 0)
             for (int p = t >> 4; p < WTH * WTW; p += WT / 16)
                 bsum += *reinterpret_cast<const float*>(gs + p * 64 + (t & 15) * 4);
     }
     __syncthreads();
-    float* red = reinterpret_cast<float*>(smem);   // [slice][u][96]
+    f2* red = reinterpret_cast<f2*>(smem);   // [sum][thread]: neighbouring threads in neighbouring banks
 #pragma unroll
     for (int dx = 0; dx < 3; ++dx)
 #pragma unroll
         for (int c = 0; c < 2; ++c)
 #pragma unroll
             for (int k = 0; k < 8; ++k)
-                reinterpret_cast<f2*>(red)[(size_t)t * 48 + (dx * 2 + c) * 8 + k] = acc[dx][c][k];
+                red[((dx * 2 + c) * 8 + k) * WRLD + t] = acc[dx][c][k];
     bred[t >> 4][t & 15] = bsum;
     __syncthreads();
     for (int i = t; i < 16 * 144; i += WT) {
         const int c = i & 15, tap = (i >> 4) % 9, o = i / 144;
         if (c >= nc) continue;
-        const int at = ((tap / 3) * 8 + c / 2) * 96 + ((tap % 3) * 2 + (c & 1)) * 16 + o;
-        float v = red[at];
+        const float* at = reinterpret_cast<const float*>(
+            red + (((tap % 3) * 2 + (c & 1)) * 8 + o / 2) * WRLD + (tap / 3) * 8 + c / 2) + (o & 1);
+        float v = at[0];
 #pragma unroll
-        for (int sl = 1; sl < 8; ++sl) v += red[sl * 24 * 96 + at];
+        for (int sl = 1; sl < 8; ++sl) v += at[sl * 48];
         a.part[((size_t)blockIdx.x * a.cout + og + o) * 9 * cin + tap * cin + cg + c] = v;
     }
     if (blockIdx.z == 0 && t < 16) {
@@ -434,7 +464,8 @@ __global__ void __launch_bounds__(WT, 2) wgrad_f32_kernel(const __grid_constant_
 // the eight warps every eighth pixel each, added in order at the end.
 constexpr int UPX = 64;
 constexpr int USTAGE = UPX * (32 + 64) * 4;
-constexpr int URED = NT * 64 * 4;
+constexpr int URLD = NT + 1;
+constexpr int URED = 64 * URLD * 4;
 constexpr int USMEM = 2 * USTAGE > URED ? 2 * USTAGE : URED;
 
 struct F32WgradUp {
@@ -508,24 +539,24 @@ __global__ void __launch_bounds__(NT, 2) wgrad_up_f32_kernel(const __grid_consta
             for (int p = t >> 6; p < UPX; p += 4) bsum += *reinterpret_cast<const float*>(gs + p * 256 + (t & 63) * 4);
     }
     __syncthreads();
-    float* red = reinterpret_cast<float*>(smem);   // [warp][lane][channel 8][column 8]
+    float* red = reinterpret_cast<float*>(smem);   // [channel 8][column 8][thread]
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             float lo, hi;
             f2_unpack(acc[i][j], lo, hi);
-            red[t * 64 + (2 * i) * 8 + j] = lo;
-            red[t * 64 + (2 * i + 1) * 8 + j] = hi;
+            red[((2 * i) * 8 + j) * URLD + t] = lo;
+            red[((2 * i + 1) * 8 + j) * URLD + t] = hi;
         }
     bred[t >> 6][t & 63] = bsum;
     __syncthreads();
     for (int i = t; i < 32 * 64; i += NT) {
         const int col = i & 63, c = i >> 6;
-        const int at = ((col >> 3) * 4 + (c >> 3)) * 64 + (c & 7) * 8 + (col & 7);
+        const int at = ((c & 7) * 8 + (col & 7)) * URLD + (col >> 3) * 4 + (c >> 3);
         float v = red[at];
 #pragma unroll
-        for (int wv = 1; wv < 8; ++wv) v += red[wv * 32 * 64 + at];
+        for (int wv = 1; wv < 8; ++wv) v += red[wv * 32 + at];
         a.part[((size_t)blockIdx.x * a.cin + cg + c) * K + ng + col] = v;
     }
     if (blockIdx.y == 0 && t < 64) {
@@ -577,11 +608,9 @@ nrv_status f32_wgrad(const float* g, int cout, const float* x1, int c1, const fl
     a.tiles_per_block = (a.ntiles + nb - 1) / nb;
     a.part = part;
     a.partb = partb;
-    static bool attr = false;
-    if (!attr) {
-        NRV_CHECK_CUDA(cudaFuncSetAttribute(wgrad_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, WSMEM));
-        attr = true;
-    }
+    static std::atomic<uint64_t> attr{0};
+    const nrv_status st = allow_smem(wgrad_f32_kernel, WSMEM, attr);
+    if (st != NRV_OK) return st;
     wgrad_f32_kernel<<<dim3(nb, cout / 16, (cin + 15) / 16), WT, WSMEM, s>>>(a);
     NRV_CHECK_LAUNCH();
     return NRV_OK;
@@ -606,11 +635,9 @@ nrv_status f32_wgrad_up(const float* x, int cin, const float* g, int ldg, int co
     a.px_per_block = (units + nb - 1) / nb * UPX;
     a.part = part;
     a.partb = partb;
-    static bool attr = false;
-    if (!attr) {
-        NRV_CHECK_CUDA(cudaFuncSetAttribute(wgrad_up_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, USMEM));
-        attr = true;
-    }
+    static std::atomic<uint64_t> attr{0};
+    const nrv_status st = allow_smem(wgrad_up_f32_kernel, USMEM, attr);
+    if (st != NRV_OK) return st;
     wgrad_up_f32_kernel<<<dim3(nb, cin / 32, cout / 16), NT, USMEM, s>>>(a);
     NRV_CHECK_LAUNCH();
     return NRV_OK;
