@@ -76,16 +76,19 @@ __global__ void repack_f32_kernel(const float* __restrict__ P, const __grid_cons
     const size_t all = J.start[J.n];
     for (size_t g = blockIdx.x * (size_t)blockDim.x + threadIdx.x; g < all;
          g += (size_t)gridDim.x * blockDim.x) {
-        int j = 0;
-        while (g >= J.start[j + 1]) ++j;
+        int j = 0, end = J.n;      // start[j] <= g < start[end]
+        while (end - j > 1) {
+            const int mid = (j + end) >> 1;
+            if (g >= J.start[mid]) j = mid;
+            else end = mid;
+        }
         const Layer& L = J.L[j];
         const int cinp = J.cinp[j];
         float* wf = wf_all + J.off[j];
         float* wt = wt_all + J.off[j];
-        const size_t i = g - J.start[j];
-        const int o = (int)(i % L.cout);
-        const int c = (int)((i / L.cout) % cinp);
-        const int tap = (int)(i / ((size_t)L.cout * cinp));
+        const uint32_t i = (uint32_t)(g - J.start[j]), r = i / (uint32_t)L.cout;
+        const int o = (int)(i - r * L.cout);
+        const int tap = (int)(r / (uint32_t)cinp), c = (int)(r - (uint32_t)tap * cinp);
         if (L.kind == CONV3) {
             wf[i] = c < L.cin ? P[L.woff + ((size_t)o * L.cin + c) * 9 + tap] : 0.0f;
             // wt index: [tap][o][c] holds W[o][c][8 - tap]

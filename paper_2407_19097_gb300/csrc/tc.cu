@@ -1354,25 +1354,26 @@ struct PackJob {
 
 // Element i of job J (i < nslices * nks * 2 * n_slice * ce).
 __device__ __forceinline__ void pack_element(const float* __restrict__ P, const PackJob& J,
-                                             size_t i) {
-    const int ce = J.fp8 ? 16 : 8;
+                                             uint32_t i) {
+    const uint32_t ce = J.fp8 ? 16 : 8, at = i;
     const int e = (int)(i % ce);
+    i /= ce;
     int nl, hf, ks, sl;
     if (J.stream) {
         // the weights of kernel rows 2, 1, 0 side by side: column n3 = (2 - dy) * n_slice + nl
         // of row K-step j, which is K-step dy * (nks / 3) + j of the tile layout
-        const int n3w = 3 * J.n_slice, ksr = J.nks / 3;
-        const int n3 = (int)((i / ce) % n3w);
-        hf = (int)((i / (ce * (size_t)n3w)) % 2);
-        const int j = (int)((i / (2 * ce * (size_t)n3w)) % ksr);
-        sl = (int)(i / (2 * ce * (size_t)n3w * ksr));
+        const uint32_t n3w = 3 * J.n_slice, ksr = J.nks / 3;
+        const uint32_t r = i / n3w, n3 = i - r * n3w, r2 = r / 2, j = r2 % ksr;
+        hf = (int)(r & 1);
+        sl = (int)(r2 / ksr);
         nl = n3 % J.n_slice;
         ks = (2 - n3 / J.n_slice) * ksr + j;
     } else {
-        nl = (int)((i / ce) % J.n_slice);
-        hf = (int)((i / (ce * (size_t)J.n_slice)) % 2);
-        ks = (int)((i / (2 * ce * (size_t)J.n_slice)) % J.nks);
-        sl = (int)(i / (2 * ce * (size_t)J.n_slice * J.nks));
+        const uint32_t r = i / (uint32_t)J.n_slice, r2 = r / 2;
+        nl = (int)(i - r * J.n_slice);
+        hf = (int)(r & 1);
+        sl = (int)(r2 / (uint32_t)J.nks);
+        ks = (int)(r2 - (uint32_t)sl * J.nks);
     }
     const int4 h = J.halves[2 * ks + hf];
     const int n = sl * J.n_slice + nl;
@@ -1399,10 +1400,10 @@ __device__ __forceinline__ void pack_element(const float* __restrict__ P, const 
         }
     }
     if (J.fp8) {
-        J.out[i] = __nv_cvt_float_to_fp8(v / J.s_w[n], __NV_SATFINITE, __NV_E4M3);
+        J.out[at] = __nv_cvt_float_to_fp8(v / J.s_w[n], __NV_SATFINITE, __NV_E4M3);
     } else {
         __nv_bfloat16 b = __float2bfloat16_rn(v);
-        reinterpret_cast<uint16_t*>(J.out)[i] = *reinterpret_cast<uint16_t*>(&b);
+        reinterpret_cast<uint16_t*>(J.out)[at] = *reinterpret_cast<uint16_t*>(&b);
     }
 }
 
@@ -1414,7 +1415,7 @@ __global__ void pack_tc_weights_kernel(const float* __restrict__ P, const __grid
     const size_t total = pack_count(J);
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
          i += (size_t)gridDim.x * blockDim.x)
-        pack_element(P, J, i);
+        pack_element(P, J, (uint32_t)i);
 }
 
 // Every layer of one layout in one launch: element i belongs to the job whose range holds it.
@@ -1429,9 +1430,13 @@ __global__ void pack_tc_weights_all_kernel(const float* __restrict__ P,
     const size_t total = J.start[J.n];
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
          i += (size_t)gridDim.x * blockDim.x) {
-        int j = 0;
-        while (i >= J.start[j + 1]) ++j;
-        pack_element(P, J.job[j], i - J.start[j]);
+        int j = 0, end = J.n;      // start[j] <= i < start[end]
+        while (end - j > 1) {
+            const int mid = (j + end) >> 1;
+            if (i >= J.start[mid]) j = mid;
+            else end = mid;
+        }
+        pack_element(P, J.job[j], (uint32_t)(i - J.start[j]));
     }
 }
 

@@ -395,25 +395,32 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const float* drgb, const 
 }
 
 // ------------------------------------------------------------------ pooling backward
-// ge[q][c] = (0.25 * gp[q/2][c] + gs[q][c]) * (e[q][c] > 0)
+// ge[q][c] = (0.25 * gp[q/2][c] + gs[q][c]) * (e[q][c] > 0): a thread makes 8 channels of 2 x 2
+// pixels, so each pooled gradient is read once and nine loads are in flight.  Bound by memory
+// (16 channels of 16 x 256^2 pixels: 107 MB in 22 us; one pixel per thread 26; 32 and 64
+// channels at levels 1 and 2: 16 -> 13.6 and 12 -> 8).
 template <typename T>
-__global__ void pool_bwd_kernel(TView<const T> gp, TView<const T> gs, TView<const T> e, TView<T> ge,
-                                int c, int n, int h, int w) {
-    const size_t total = (size_t)n * h * w * (c / 8);
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        const int cg = (int)(i % (c / 8)) * 8;
-        const size_t q = i / (c / 8);
-        const int X = (int)(q % w), Y = (int)((q / w) % h);
-        const size_t img = q / ((size_t)w * h);
-        const size_t row = img * h + Y;
-        float a[8], b[8], m[8], r[8];
-        ld8<T>(gp.at(img * (h / 2) + Y / 2, X / 2, cg, w / 2), a);
-        ld8<T>(gs.at(row, X, cg, w), b);
-        ld8<T>(e.at(row, X, cg, w), m);
+__global__ void __launch_bounds__(256) pool_bwd_kernel(TView<const T> gp, TView<const T> gs, TView<const T> e,
+                                                       TView<T> ge, int c, int rows2, int w) {
+    const uint32_t w2 = w / 2, ng = c / 8, u = blockIdx.x * 256u + threadIdx.x;
+    if (u >= w2 * ng) return;
+    // neighbouring threads take neighbouring memory: pixels of a plane, or channels of a pixel
+    const uint32_t grp = ge.planar ? u / w2 : u % ng, X = ge.planar ? u - grp * w2 : u / ng;
+    const int cg = 8 * (int)grp;
+    for (int r2 = blockIdx.y; r2 < rows2; r2 += gridDim.y) {
+        float a[8], b[4][8], m[4][8];
+        ld8<T>(gp.at(r2, X, cg, w2), a);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) r[k] = m[k] > 0.0f ? fmaf(0.25f, a[k], b[k]) : 0.0f;
-        st8<T>(ge.at(row, X, cg, w), r);
+        for (int k = 0; k < 4; ++k) {
+            ld8<T>(gs.at(2 * (size_t)r2 + (k >> 1), 2 * X + (k & 1), cg, w), b[k]);
+            ld8<T>(e.at(2 * (size_t)r2 + (k >> 1), 2 * X + (k & 1), cg, w), m[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) b[k][j] = m[k][j] > 0.0f ? fmaf(0.25f, a[j], b[k][j]) : 0.0f;
+            st8<T>(ge.at(2 * (size_t)r2 + (k >> 1), 2 * X + (k & 1), cg, w), b[k]);
+        }
     }
 }
 
@@ -840,8 +847,11 @@ struct Bwd {
 
     nrv_status pool_bwd(TView<const T> gp, TView<const T> gs, int e, TView<T> ge, int level) {
         const int c = net->act_c[e];
-        pool_bwd_kernel<T><<<blocks_for(g.px(level) * c / 8), 256, 0, s>>>(
-            gp, gs, CA(e), ge, c, g.n, g.h[level], g.w[level]);
+        // the levels a pool reads are of even size: the canvas is a multiple of 8
+        const long long rows2 = (long long)g.n * (g.h[level] / 2);
+        const unsigned bx = (unsigned)((g.w[level] / 2 * (c / 8) + 255) / 256);
+        pool_bwd_kernel<T><<<dim3(bx, (unsigned)(rows2 < 65535 ? rows2 : 65535)), 256, 0, s>>>(
+            gp, gs, CA(e), ge, c, (int)rows2, g.w[level]);
         NRV_CHECK_LAUNCH();
         return NRV_OK;
     }
