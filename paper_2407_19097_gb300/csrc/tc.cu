@@ -1216,6 +1216,59 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 }
             }
         };
+        // data gradients: no bias, activation or fused consumer, zeroed by the mask (the sign of
+        // the forward activation).  The first mask words are read before the accumulators are
+        // waited for, the next ones while TMEM is read, so the epilogue does not stand still for
+        // a global load per 16 columns.
+        const bool grad_fast = !FP8 && !GATED && !STREAM && P.mode != 1 && !P.bias && !P.relu && !P.nhwc &&
+                               P.store_y && !P.head_w && !P.pool_y;
+        const size_t gplane = (size_t)P.w * 16;
+        uint4 mk0, mk1;
+        auto mask_words = [&](size_t at, bool valid) {
+            const uint8_t* mp = (const uint8_t*)P.mask + at;
+            if (P.mask && valid) {
+                mk0 = *reinterpret_cast<const uint4*>(mp);
+                mk1 = *reinterpret_cast<const uint4*>(mp + gplane);
+            }
+        };
+        // `at`: byte of this pixel's first plane; mk0 and mk1 hold its first mask words
+        auto emit_grad = [&](uint32_t tbase, size_t at, bool valid) {
+#pragma unroll 1
+            for (int c0 = 0; c0 < P.n_slice; c0 += 16) {
+                uint32_t a[16], b[16];
+                tmem_ld16_nowait(tbase + (uint32_t)c0, a);
+                if (P.nissue == 2) tmem_ld16_nowait(tbase + (uint32_t)(P.n_slice + c0), b);
+                const uint4 m0 = mk0, m1 = mk1;
+                if (c0 + 16 < P.n_slice) mask_words(at + 2 * gplane, valid);
+                tmem_ld_wait();
+                tmem_tie8(a);
+                tmem_tie8(a + 8);
+                tmem_tie8(b);
+                tmem_tie8(b + 8);
+                const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+                uint32_t o[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    float v[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        v[e] = __uint_as_float(a[2 * j + e]);
+                        if (P.nissue == 2) v[e] += __uint_as_float(b[2 * j + e]);
+                    }
+                    o[j] = bf16x2(v[0], v[1]);
+                    if (P.mask) {
+                        // BF16 bits of a positive number: sign clear, not +0, not NaN
+                        if ((mw[j] & 0xFFFFu) - 1u >= 0x7F80u) o[j] &= 0xFFFF0000u;
+                        if ((mw[j] >> 16) - 1u >= 0x7F80u) o[j] &= 0x0000FFFFu;
+                    }
+                }
+                if (valid) {
+                    *reinterpret_cast<uint4*>((uint8_t*)P.y + at) = make_uint4(o[0], o[1], o[2], o[3]);
+                    *reinterpret_cast<uint4*>((uint8_t*)P.y + at + gplane) = make_uint4(o[4], o[5], o[6], o[7]);
+                }
+                at += 2 * gplane;
+            }
+        };
         const bool up_fast = !FP8 && !GATED && P.mode == 1 && P.nslices == 1 && P.nissue == 1 &&
                              !P.mask &&
                              P.store_y && !P.head_w && !P.pool_y && (P.cout % 8) == 0;
@@ -1223,14 +1276,19 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
         w.init(P, t_begin);
         for (int t = t_begin, i = 0; t < t_end; ++t, ++i, w.next(P)) {
             const int ab = i & (P.nacc - 1);
+            const int x = w.xt * P.tile_w + m;
+            const bool valid_x = m < P.tile_w && x < P.w;
+            size_t gat = 0;
+            if (grad_fast) {
+                gat = ((((size_t)w.img * P.h + w.y) * P.out_nch + slice * (P.n_slice / 8)) * P.w + x) * 16;
+                mask_words(gat, valid_x && w.y < P.h);
+            }
             int ok = 1;
             if (lane == 0)
                 ok = mbar_wait(b_afull(ab), (i >> P.acc_shift) & 1, &abort_flag, P.status) ? 1 : 0;
             ok = __shfl_sync(0xffffffffu, ok, 0);
             if (!ok) break;
             tc_fence_after();
-            const int x = w.xt * P.tile_w + m;
-            const bool valid_x = m < P.tile_w && x < P.w;
 #pragma unroll 1
             for (int r = 0; r < P.rpt; ++r) {
                 const int yy = w.y + r;
@@ -1238,7 +1296,11 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) +
                                        (uint32_t)((ab * P.rpt + r) * P.nissue * P.n_slice);
                 if (up_fast) emit_up(tbase, w.img, x, valid, yy);
-                else emit_row(tbase, w.img, x, valid, yy);
+                else if (grad_fast) {
+                    if (r > 0) mask_words(gat, valid);
+                    emit_grad(tbase, gat, valid);
+                    gat += P.out_nch * gplane;
+                } else emit_row(tbase, w.img, x, valid, yy);
             }
             tc_fence_before();
             __syncwarp();
