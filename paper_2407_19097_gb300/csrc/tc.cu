@@ -1269,6 +1269,50 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 at += 2 * gplane;
             }
         };
+        // the same in E4M3: 16 channels (one plane) of both parities of a row at a time
+        auto emit_up8 = [&](uint32_t tbase, int img, int x, bool valid, int yy) {
+            const size_t wo = 2 * (size_t)P.w;
+#pragma unroll 1
+            for (int a = 0; a < 2; ++a) {
+                uint8_t* dst = (uint8_t*)P.y +
+                               ((((size_t)img * 2 * P.h + 2 * yy + a) * P.out_nch) * wo + 2 * x) * 16;
+#pragma unroll 1
+                for (int o = 0; o < P.cout; o += 16, dst += wo * 16) {
+                    const int c0 = 2 * a * P.cout + o;
+                    uint32_t f[2][16];
+                    tmem_ld16_nowait(tbase + (uint32_t)c0, f[0]);
+                    tmem_ld16_nowait(tbase + (uint32_t)(c0 + P.cout), f[1]);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int b = 0; b < 2; ++b) {
+                        tmem_tie8(f[b]);
+                        tmem_tie8(f[b] + 8);
+                        const float4* b4 = reinterpret_cast<const float4*>(bias_s + c0 + b * P.cout);
+                        const float4* s4 = reinterpret_cast<const float4*>(colscale_s + c0 + b * P.cout);
+                        uint32_t wd[4];
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const float4 bb = b4[q], ss = s4[q];
+                            float v[4] = {fmaf(__uint_as_float(f[b][4 * q]), ss.x, bb.x),
+                                          fmaf(__uint_as_float(f[b][4 * q + 1]), ss.y, bb.y),
+                                          fmaf(__uint_as_float(f[b][4 * q + 2]), ss.z, bb.z),
+                                          fmaf(__uint_as_float(f[b][4 * q + 3]), ss.w, bb.w)};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                if (P.relu) v[e] = fmaxf(v[e], 0.0f);
+                                v[e] *= P.inv_out;
+                            }
+                            const uint32_t lo = __nv_cvt_float2_to_fp8x2(make_float2(v[0], v[1]), __NV_SATFINITE, __NV_E4M3);
+                            const uint32_t hi = __nv_cvt_float2_to_fp8x2(make_float2(v[2], v[3]), __NV_SATFINITE, __NV_E4M3);
+                            wd[q] = lo | (hi << 16);
+                        }
+                        if (valid) reinterpret_cast<uint4*>(dst)[b] = make_uint4(wd[0], wd[1], wd[2], wd[3]);
+                    }
+                }
+            }
+        };
+        const bool up8_fast = FP8 && P.mode == 1 && P.nslices == 1 && P.nissue == 1 && !P.mask && !P.nhwc &&
+                              P.store_y && !P.head_w && !P.pool_y && (P.cout % 16) == 0;
         const bool up_fast = !FP8 && !GATED && P.mode == 1 && P.nslices == 1 && P.nissue == 1 &&
                              !P.mask &&
                              P.store_y && !P.head_w && !P.pool_y && (P.cout % 8) == 0;
@@ -1296,6 +1340,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 const uint32_t tbase = tmem + ((uint32_t)(32 * q) << 16) +
                                        (uint32_t)((ab * P.rpt + r) * P.nissue * P.n_slice);
                 if (up_fast) emit_up(tbase, w.img, x, valid, yy);
+                else if (up8_fast) emit_up8(tbase, w.img, x, valid, yy);
                 else if (grad_fast) {
                     if (r > 0) mask_words(gat, valid);
                     emit_grad(tbase, gat, valid);
