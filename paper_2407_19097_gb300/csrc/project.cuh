@@ -37,6 +37,11 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
 }
 // (.ftz: the depths it is used for, 2^-60 .. 2^125, and their reciprocals are normal; without
 // it every call carries a scaling for subnormal arguments, a tenth of the pass's instructions)
+__device__ __forceinline__ float ex2_approx(float x) {
+    float r;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
 __device__ __forceinline__ float rcp_approx(float v) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));

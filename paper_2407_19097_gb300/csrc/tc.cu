@@ -956,27 +956,35 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         tmem_tie8(fb);
                         tmem_tie8(ga);
                         tmem_tie8(gb);
-                        const float4* b4 = reinterpret_cast<const float4*>(bias_s + cf);
-                        const float4 f0 = b4[0], f1 = b4[1], g0 = b4[4], g1 = b4[5];
-                        const float bq[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-                        const float gq[8] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
-                        // ELU(f) * sigmoid(g), as in the per-row epilogue
-                        auto gate = [](float f, float g) {
-                            const float e = __expf(fminf(f, 0.0f));
-                            return __fdividef(f > 0.0f ? f : e - 1.0f, 1.0f + __expf(-g));
+                        const f2* b2 = reinterpret_cast<const f2*>(bias_s + cf);   // gates: b2 + 8
+                        // ELU(f) * sigmoid(g) of two channels, as in the per-row epilogue.  Three
+                        // special-function results per value are the floor (24 issue cycles of
+                        // that unit a warp); the rest is packed, and the flushing forms need no
+                        // scaling around them: a subnormal e^x is lost beside the 1 either way,
+                        // and 1 + e^-g is at least 1.
+                        auto gate2 = [](f2 f, f2 g) -> f2 {
+                            constexpr float L2E = 1.4426950408889634f;
+                            float f0, f1, x0, x1, y0, y1;
+                            f2_unpack(f, f0, f1);
+                            f2_unpack(f2_mul(f2_pack(fminf(f0, 0.0f), fminf(f1, 0.0f)), f2_pack(L2E, L2E)), x0, x1);
+                            f2_unpack(f2_add(f2_pack(ex2_approx(x0), ex2_approx(x1)), f2_pack(-1.0f, -1.0f)), x0, x1);
+                            f2_unpack(f2_mul(g, f2_pack(-L2E, -L2E)), y0, y1);
+                            f2_unpack(f2_add(f2_pack(ex2_approx(y0), ex2_approx(y1)), f2_pack(1.0f, 1.0f)), y0, y1);
+                            return f2_mul(f2_pack(f0 > 0.0f ? f0 : x0, f1 > 0.0f ? f1 : x1),
+                                          f2_pack(rcp_approx(y0), rcp_approx(y1)));
                         };
                         uint32_t pa[4], pb[4];
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
-                            float u[2], w[2];
-#pragma unroll
-                            for (int e = 0; e < 2; ++e) {
-                                const int i = 2 * j + e;
-                                u[e] = gate(__uint_as_float(fa[i]) + bq[i], __uint_as_float(ga[i]) + gq[i]);
-                                w[e] = gate(__uint_as_float(fb[i]) + bq[i], __uint_as_float(gb[i]) + gq[i]);
-                            }
-                            pa[j] = bf16x2(u[0], u[1]);
-                            pb[j] = bf16x2(w[0], w[1]);
+                            auto at = [&](const uint32_t* v, f2 b) {
+                                return f2_add(f2_pack(__uint_as_float(v[2 * j]), __uint_as_float(v[2 * j + 1])), b);
+                            };
+                            const f2 bf = b2[j], bg = b2[8 + j];
+                            float u0, u1;
+                            f2_unpack(gate2(at(fa, bf), at(ga, bg)), u0, u1);
+                            pa[j] = bf16x2(u0, u1);
+                            f2_unpack(gate2(at(fb, bf), at(gb, bg)), u0, u1);
+                            pb[j] = bf16x2(u0, u1);
                         }
                         float mean[8];
                         finish8(ra, rb, sa, sb, k, pa, pb, mean);
