@@ -344,13 +344,15 @@ __global__ void tile_bound_kernel(RViews vs_arg, const RViews* __restrict__ view
     if (v >= vs.n) return;    // whole warps leave together
     const RView& vw = vs.v[v];
     const int tx = (vw.width + TILE - 1) / TILE;
-    constexpr int LPR = 32 / TILE, PPL = TILE / LPR;   // lanes per tile row, pixels per lane
-    const int x0 = (t % tx) * TILE + (lane % LPR) * PPL, y = (t / tx) * TILE + lane / LPR;
+    // a load of the warp covers 32 / TILE whole rows of the tile: each 32-byte sector once
+    constexpr int RPL = 32 / TILE;
+    const int x = (t % tx) * TILE + lane % TILE, y0 = (t / tx) * TILE + lane / TILE;
+    const uint32_t* depth = reinterpret_cast<const uint32_t*>(vw.key) + 1;
     unsigned m = 0;
-    if (y < vw.height)
-        for (int k = 0; k < PPL; ++k)
-            if (x0 + k < vw.width)
-                m = max(m, (unsigned)(__ldcg(vw.key + (size_t)y * vw.width + x0 + k) >> 32));
+#pragma unroll
+    for (int k = 0; k < TILE; k += RPL)
+        if (x < vw.width && y0 + k < vw.height)
+            m = max(m, __ldcg(depth + 2 * ((size_t)(y0 + k) * vw.width + x)));
     m = __reduce_max_sync(0xffffffffu, m);
     if (lane == 0) out[t] = m;
 }
