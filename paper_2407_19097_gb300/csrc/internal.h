@@ -94,9 +94,9 @@ struct ResolveArgs {
 };
 
 nrv_status launch_clear_keys(const RViews& views, cudaStream_t s);
-// Render pass.  `tiles` is scratch for the per-tile depth bounds of the culling
+// Render pass.  `tiles` is scratch for the per-tile depth bounds of the chunk-culling
 // variants: visibility_scratch_bytes(views) bytes of device memory (may be null,
-// which disables culling).  `chunks` holds the bounding boxes of the scene's
+// which disables them).  `chunks` holds the bounding boxes of the scene's
 // 32-point chunks (6 floats each, chunk_count(n) of them) followed by those of
 // their 8-point sub-chunks (RENDER_SUBS per chunk, 6 floats each), from
 // launch_chunk_bounds (chunk_box_bytes(n) bytes); may be null, which disables

@@ -33,19 +33,20 @@
 // asked, the 2x2 average pool of that output or the 1x1 head on it.
 // Accumulators are double-buffered.  The loader reads activations only after
 // griddepcontrol.wait (programmatic dependent launch: the setup and the weight
-// load overlap the previous kernel).  The MMA issue loop is kept free of
-// branches and of dependent parameter loads (the operand kind is a template
-// parameter, the per-K-step descriptor words sit in shared memory and are read
-// one step ahead): with narrow N the issuing thread, not the tensor pipe, sets
-// the pace.  Every wait is bounded: on timeout the
-// kernel records STATUS_TIMEOUT in the status word, waits (bounded) for its
+// load overlap the previous kernel).  With narrow N the issuing warp, not the
+// tensor pipe, sets the pace, so its loop is kept short: the warp stays uniform
+// and elects the lane that issues (a branch on the lane makes every following
+// instruction a divergent one), the operand kind is a template parameter, and
+// the K-step pattern of a row comes from the kernel's parameters with the loop
+// over it unrolled for the row lengths in use.  Every wait is bounded: on
+// timeout the kernel records STATUS_TIMEOUT in the status word, waits (bounded) for its
 // own copies in flight, frees TMEM and returns.
 //
 // The data gradient of the 2x2 stride-2 transposed conv (mode 2) is a GEMM of one input
 // row's pixels (M) against K = (a, b, C_out): each "row load" is four 5-D TMA boxes of the
 // output gradient at output row 2y + a and pixel parity b (dense [plane][pixel][16 bytes]
 // tiles, K-major like any input row), the weights W[c][o][a][b] resident as B, and the
-// epilogue of mode 0 (mask, no bias, no ReLU).
+// epilogue of mode 0 (mask, no bias, no ReLU), which reads the mask ahead of the accumulators.
 //
 // The 2x2 stride-2 transposed conv runs through the same kernel as a GEMM of
 // one input row (K = C_in, tiles of 128 pixels, no halo) against all four
@@ -61,8 +62,8 @@
 // epilogue zeroes each block after draining it, and input rows are committed in groups (one
 // commit per group releases the group's slots to the loader and hands its final output rows
 // to the epilogue).  One MMA issuer; two groups of four epilogue warps (warps 2-5 and 6-9)
-// take alternate groups and drain two output rows at a time, 8 channels per step, with the
-// fused 2x2 pool computed from the even/odd pair in registers.
+// take alternate groups and drain two output rows at a time, 16 columns per step (8 channels of
+// gated layers), with the fused 2x2 pool computed from the even/odd pair in registers.
 #include <cuda.h>
 #include <string.h>
 
