@@ -1534,12 +1534,14 @@ __global__ void pack_tc_weights_kernel(const float* __restrict__ P, const __grid
         pack_element(P, J, (uint32_t)i);
 }
 
-// Every layer of one layout in one launch: element i belongs to the job whose range holds it.
+// Every layer, of the forward and of the data-gradient layout, in one launch: element i belongs
+// to the job whose range holds it.
 struct PackJobs {
     int n;
-    size_t start[NUM_LAYERS + 1];
-    PackJob job[NUM_LAYERS];
+    size_t start[2 * NUM_LAYERS + 1];
+    PackJob job[2 * NUM_LAYERS];
 };
+static_assert(sizeof(PackJobs) <= 4000, "kernel parameters");
 
 __global__ void pack_tc_weights_all_kernel(const float* __restrict__ P,
                                            const __grid_constant__ PackJobs J) {
@@ -1769,7 +1771,8 @@ static nrv_status build_cfg_dgrad(Net* net, std::vector<int4>& all_halves, std::
     return NRV_OK;
 }
 
-static nrv_status tc_repack_dgrad(Net* net, cudaStream_t s) {
+// Adds the jobs of the data-gradient weights to J.
+static nrv_status tc_repack_dgrad(Net* net, PackJobs& J, cudaStream_t s) {
     std::vector<int4> all_halves;
     std::vector<size_t> hoff(NUM_LAYERS, 0);
     size_t off = 0;
@@ -1777,8 +1780,6 @@ static nrv_status tc_repack_dgrad(Net* net, cudaStream_t s) {
     if (off == 0) return NRV_OK;
     NRV_TRY(net->wtbf16.ensure(off));
     NRV_TRY(upload_halves(2, all_halves, s));
-    PackJobs J;
-    memset(&J, 0, sizeof(J));
     for (int l = 0; l < NUM_LAYERS; ++l) {
         const TcLayerCfg& c = g_cfg_dg[l];
         if (!c.ok) continue;
@@ -1788,7 +1789,7 @@ static nrv_status tc_repack_dgrad(Net* net, cudaStream_t s) {
                                1.0f, nullptr, (const int4*)g_halves[2].p + hoff[l],
                                (uint8_t*)net->wtbf16.p + c.w_off};
     }
-    return pack_all((const float*)net->params.p, J, s);
+    return NRV_OK;
 }
 
 nrv_status tc_repack(Net* net, cudaStream_t s) {
@@ -1809,8 +1810,8 @@ nrv_status tc_repack(Net* net, cudaStream_t s) {
                                1.0f, nullptr, (const int4*)g_halves[0].p + hoff[l],
                                (uint8_t*)net->wbf16.p + c.w_off, c.stream};
     }
+    NRV_TRY(tc_repack_dgrad(net, J, s));
     NRV_TRY(pack_all((const float*)net->params.p, J, s));
-    NRV_TRY(tc_repack_dgrad(net, s));
     if (net->fp8_ready) return tc_repack_fp8(net, s);
     return NRV_OK;
 }

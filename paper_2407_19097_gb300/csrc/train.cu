@@ -7,6 +7,7 @@
 #include "f32.h"
 #include "net.h"
 #include "net_simt.cuh"
+#include "project.cuh"
 
 namespace nrv {
 
@@ -329,40 +330,74 @@ __global__ void __launch_bounds__(256) wgrad_up_kernel(TView<const T> x, int cin
 //   part[blk][o*16 + c] = sum drgb[o] * x[c], part[blk][48 + o] = sum drgb[o] over the block's chunk
 // of cropped pixels: every thread keeps all 51 sums, then the block adds them (warp shuffles,
 // then the 8 warps in order).
+// Latency- and issue-bound (78 MB would take 12 us there): channels in pairs, and the position
+// advanced by the block's width instead of divided out per pixel, 38 -> 26 us; two threads per
+// pixel at twice the warps measured 48.
 template <typename T>
-__global__ void __launch_bounds__(256) head_bwd_kernel(const float* drgb, const float* __restrict__ w,
+__global__ void __launch_bounds__(256, 2) head_bwd_kernel(const float* drgb, const float* __restrict__ w,
                                                        TView<const T> x, TView<T> gd, int n, int hn, int wn,
                                                        int h, int wd, size_t chunk, float* part) {
     __shared__ float red[8][51];
-    __shared__ float ws[48];
+    __shared__ __align__(16) float ws[48];
     if (threadIdx.x < 48) ws[threadIdx.x] = w[threadIdx.x];
     __syncthreads();
-    float acc[51];
+    f2 acc[3][8];        // channel pairs
+    float accb[3];
 #pragma unroll
-    for (int k = 0; k < 51; ++k) acc[k] = 0.0f;
+    for (int o = 0; o < 3; ++o) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[o][j] = 0ull;
+        accb[o] = 0.0f;
+    }
     const size_t total = (size_t)n * h * wd;
     const size_t i0 = blockIdx.x * chunk, i1 = i0 + chunk < total ? i0 + chunk : total;
-    for (size_t i = i0 + threadIdx.x; i < i1; i += blockDim.x) {
-        const uint32_t row = (uint32_t)(i / (uint32_t)wd), X = (uint32_t)(i - (size_t)row * wd);
-        const uint32_t img = row / (uint32_t)h, Y = row - img * (uint32_t)h;
-        const size_t at = (size_t)img * hn + Y;
+    // row and column from the block's first pixel on, in 32 bits
+    const uint64_t row0 = i0 / (uint32_t)wd;
+    const uint32_t X0 = (uint32_t)(i0 - row0 * (uint32_t)wd), cnt = i1 > i0 ? (uint32_t)(i1 - i0) : 0;
+    const uint32_t img0 = (uint32_t)(row0 / (uint32_t)h), Y0 = (uint32_t)(row0 - (uint64_t)img0 * (uint32_t)h);
+    const uint32_t q0 = X0 + threadIdx.x, r0 = Y0 + q0 / (uint32_t)wd;
+    uint32_t X = q0 % (uint32_t)wd, Y = r0 % (uint32_t)h, img = img0 + r0 / (uint32_t)h;
+    const uint32_t stepY = 256u / (uint32_t)wd, stepX = 256u - stepY * (uint32_t)wd;
+    // both tensors hold 16 channels: the elements of a row, and from one half of a pixel to the other
+    const T* const xb = x.at(0, 0, 0, wn);
+    T* const gb = gd.at(0, 0, 0, wn);
+    const bool planar = gd.planar;
+    const uint32_t row_e = 16u * (uint32_t)wn, half = planar ? 8u * (uint32_t)wn : 8u;
+    const float* dp = drgb + 3 * (i0 + threadIdx.x);
+    for (uint32_t p = threadIdx.x; p < cnt; p += 256, dp += 768) {
+        const size_t at = ((size_t)img * (uint32_t)hn + Y) * row_e + X * (planar ? 8u : 16u);
+        X += stepX;
+        Y += stepY;
+        if (X >= (uint32_t)wd) {
+            X -= (uint32_t)wd;
+            ++Y;
+        }
+        while (Y >= (uint32_t)h) {
+            Y -= (uint32_t)h;
+            ++img;
+        }
         float v[16];
-        ld8<T>(x.at(at, X, 0, wn), v);
-        ld8<T>(x.at(at, X, 8, wn), v + 8);
-        const float d[3] = {drgb[3 * i], drgb[3 * i + 1], drgb[3 * i + 2]};
+        ld8<T>(xb + at, v);
+        ld8<T>(xb + at + half, v + 8);
+        const float d[3] = {dp[0], dp[1], dp[2]};
+        const f2 dd[3] = {f2_pack(d[0], d[0]), f2_pack(d[1], d[1]), f2_pack(d[2], d[2])};
+        const f2* w2 = reinterpret_cast<const f2*>(ws);
         float out[16];
 #pragma unroll
-        for (int c = 0; c < 16; ++c) {
-            const float s = fmaf(d[2], ws[32 + c], fmaf(d[1], ws[16 + c], d[0] * ws[c]));
-            out[c] = v[c] > 0.0f ? s : 0.0f;
+        for (int j = 0; j < 8; ++j) {
+            const f2 s = f2_fma(dd[2], w2[16 + j], f2_fma(dd[1], w2[8 + j], f2_mul(dd[0], w2[j])));
+            float s0, s1;
+            f2_unpack(s, s0, s1);
+            out[2 * j] = v[2 * j] > 0.0f ? s0 : 0.0f;
+            out[2 * j + 1] = v[2 * j + 1] > 0.0f ? s1 : 0.0f;
         }
-        st8<T>(gd.at(at, X, 0, wn), out);
-        st8<T>(gd.at(at, X, 8, wn), out + 8);
+        st8<T>(gb + at, out);
+        st8<T>(gb + at + half, out + 8);
 #pragma unroll
         for (int o = 0; o < 3; ++o) {
 #pragma unroll
-            for (int c = 0; c < 16; ++c) acc[o * 16 + c] = fmaf(d[o], v[c], acc[o * 16 + c]);
-            acc[48 + o] += d[o];
+            for (int j = 0; j < 8; ++j) acc[o][j] = f2_fma(dd[o], f2_pack(v[2 * j], v[2 * j + 1]), acc[o][j]);
+            accb[o] += d[o];
         }
     }
     // the canvas margin
@@ -380,11 +415,20 @@ __global__ void __launch_bounds__(256) head_bwd_kernel(const float* drgb, const 
         }
     }
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-#pragma unroll
-    for (int k = 0; k < 51; ++k) {
-        float a = acc[k];
+    auto put = [&](float a, int k) {
         for (int off = 16; off > 0; off >>= 1) a += __shfl_xor_sync(0xffffffffu, a, off);
         if (lane == 0) red[wp][k] = a;
+    };
+#pragma unroll
+    for (int o = 0; o < 3; ++o) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            float a0, a1;
+            f2_unpack(acc[o][j], a0, a1);
+            put(a0, o * 16 + 2 * j);
+            put(a1, o * 16 + 2 * j + 1);
+        }
+        put(accb[o], 48 + o);
     }
     __syncthreads();
     if (threadIdx.x < 51) {
