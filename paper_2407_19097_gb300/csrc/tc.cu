@@ -962,7 +962,7 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                         // special-function results per value are the floor (24 issue cycles of
                         // that unit a warp); the rest is packed, and the flushing forms need no
                         // scaling around them: a subnormal e^x is lost beside the 1 either way,
-                        // and 1 + e^-g is at least 1.
+                        // and 1 + e^-g is at least 1.  1080p gated network 289 -> 268 us.
                         auto gate2 = [](f2 f, f2 g) -> f2 {
                             constexpr float L2E = 1.4426950408889634f;
                             float f0, f1, x0, x1, y0, y1;
@@ -1228,7 +1228,8 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
         // data gradients: no bias, activation or fused consumer, zeroed by the mask (the sign of
         // the forward activation).  The first mask words are read before the accumulators are
         // waited for, the next ones while TMEM is read, so the epilogue does not stand still for
-        // a global load per 16 columns.
+        // a global load per 16 columns (the sixteen data gradients of a 16 x 256^2 step: 465 ->
+        // 436 us, the deep levels' most: 26 -> 20).
         const bool grad_fast = !FP8 && !GATED && !STREAM && P.mode != 1 && !P.bias && !P.relu && !P.nhwc &&
                                P.store_y && !P.head_w && !P.pool_y;
         const size_t gplane = (size_t)P.w * 16;
@@ -1278,7 +1279,8 @@ __global__ void __launch_bounds__(STREAM ? NTHREADS_S : NTHREADS, STREAM ? 2 : 4
                 at += 2 * gplane;
             }
         };
-        // the same in E4M3: 16 channels (one plane) of both parities of a row at a time
+        // the same in E4M3: 16 channels (one plane) of both parities of a row at a time (1080p
+        // FP8 network 268 -> 256 us; the general epilogue took 16 and 20 us for the two layers)
         auto emit_up8 = [&](uint32_t tbase, int img, int x, bool valid, int yy) {
             const size_t wo = 2 * (size_t)P.w;
 #pragma unroll 1
