@@ -126,12 +126,17 @@ nrv_status net_repack(Net* net, cudaStream_t s) {
         J.start[J.n + 1] = J.start[J.n] + (size_t)kk * J.cinp[J.n] * L.cout;
         ++J.n;
     }
+    // The tensor-core copies first, then this plain launch.  The first conv of the next forward
+    // loads its weights before it waits for its predecessor (a programmatic dependent launch), so
+    // the kernel that wrote them must not be that predecessor: the launch below starts only once
+    // the packing is complete, and the conv not before this one ends.
+    NRV_TRY(tc_repack(net, s));
     size_t blocks = (J.start[J.n] + 255) / 256;
     if (blocks > 152 * 8) blocks = 152 * 8;
     repack_f32_kernel<<<(unsigned)(blocks ? blocks : 1), 256, 0, s>>>(P, J, (float*)net->wf32.p,
                                                                     (float*)net->wtf32.p);
     NRV_CHECK_LAUNCH();
-    return tc_repack(net, s);
+    return NRV_OK;
 }
 
 // ------------------------------------------------------------------ workspace

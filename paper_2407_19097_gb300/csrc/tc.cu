@@ -1599,7 +1599,11 @@ nrv_status upload_halves(int k, const std::vector<int4>& h, cudaStream_t s) {
     return NRV_OK;
 }
 
-// One launch for a table of packing jobs.
+// One launch for a table of packing jobs.  conv3_tc_kernel reads packed weights before its
+// griddepcontrol.wait, so a caller has a plain launch follow this one ahead of any conv that reads
+// them: net_repack ends with the FP32 copies, tc_repack_fp8 packs layer by layer (the first
+// layer's conv is the only one not behind another conv's wait), and the gated network's calls
+// start with the injection or the conversion of their operands.
 nrv_status pack_all(const float* P, PackJobs& J, cudaStream_t s) {
     J.start[0] = 0;
     for (int j = 0; j < J.n; ++j)
