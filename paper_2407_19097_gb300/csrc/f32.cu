@@ -19,9 +19,10 @@
 //    with 16-byte cp.async into one of two buffers while it works on the other.  In a row the
 //    pixels of a group of 8 sit 32 bytes apart and groups 16 bytes further, so that the eight
 //    groups a quarter-warp reads lie in eight different bank quads.
-//  * Where the tiles of a layer are fewer than the SMs can hold (the deep levels), the input
+//  * Where the tiles of one image are fewer than the SMs (the deep levels), the input
 //    channels are split over a cluster of KS blocks, whose sums are added through distributed
-//    shared memory in rank order (deterministic).
+//    shared memory in rank order (deterministic).  The split decides the order of the sums, so
+//    it follows from the image's size alone: images computed together come out as they do alone.
 #include <atomic>
 
 #include <cooperative_groups.h>
@@ -260,7 +261,7 @@ nrv_status allow_smem(K kern, int bytes, std::atomic<uint64_t>& done) {
 // memory that keeps others out, because clusters are otherwise packed two (four) blocks to an
 // SM while SMs stay empty.
 template <int MODE, int OCB, int TW, int NB>
-nrv_status launch_tile(F32Args& a, cudaStream_t s) {
+nrv_status launch_tile(F32Args& a, int ks, cudaStream_t s) {
     using T = F32Tile<MODE, OCB, TW, NB>;
     constexpr int SPREAD = NB == 128 ? 80 * 1024 : 120 * 1024;
     a.tiles_x = (a.w + TW - 1) / TW;
@@ -268,9 +269,6 @@ nrv_status launch_tile(F32Args& a, cudaStream_t s) {
     const long long tiles = (long long)a.tiles_x * a.tiles_y * a.n;
     if (tiles > 0x7FFFFFFFll) return fail(NRV_ERR_UNSUPPORTED, "too many tiles");
     const int ob = a.ncols / OCB, nst = a.cin / CK;
-    // split the input channels while the blocks do not fill the SMs (two blocks each)
-    int ks = 1;
-    while (ks < 8 && tiles * ob * ks < 256 && 2 * ks <= nst) ks *= 2;
     static std::atomic<uint64_t> attr{0};
     auto kern = conv_f32_kernel<MODE, OCB, TW, NB>;
     const nrv_status st = allow_smem(kern, T::SMEMK > SPREAD ? T::SMEMK : SPREAD, attr);
@@ -300,11 +298,17 @@ nrv_status launch_tile(F32Args& a, cudaStream_t s) {
 template <int MODE, int OCB, int TW>
 nrv_status launch_block(F32Args& a, cudaStream_t s) {
     constexpr int TH = F32Tile<MODE, OCB, TW, NT>::TH;
-    const long long tiles = (long long)((a.w + TW - 1) / TW) * ((a.h + TH - 1) / TH) * a.n;
-    int ks = 1;
-    while (ks < 8 && 2 * ks <= a.cin / CK) ks *= 2;
-    if (OCB == 32 && tiles * (a.ncols / OCB) * ks <= 152) return launch_tile<MODE, OCB, TW, OCB == 32 ? 128 : NT>(a, s);
-    return launch_tile<MODE, OCB, TW, NT>(a, s);
+    const long long blocks = (long long)((a.w + TW - 1) / TW) * ((a.h + TH - 1) / TH) * (a.ncols / OCB);
+    const int nst = a.cin / CK;
+    // Split the input channels until one image has 128 blocks.  (256, two to an SM: 588 us against
+    // 580 for a 512 x 512 frame, 1071 against 1027 for the 2 x 256^2 training step.  A split that
+    // also counted the images took 1858 us for 16 x 256^2 against 2051 here, but then an image's
+    // result depended on how many shared its call.)
+    int ks = 1, most = 1;
+    while (ks < 8 && blocks * ks < 128 && 2 * ks <= nst) ks *= 2;
+    while (most < 8 && 2 * most <= nst) most *= 2;
+    if (OCB == 32 && blocks * a.n * most <= 152) return launch_tile<MODE, OCB, TW, OCB == 32 ? 128 : NT>(a, ks, s);
+    return launch_tile<MODE, OCB, TW, NT>(a, ks, s);
 }
 
 // The tile width that covers the image with the fewest pixels (64 where equal).
