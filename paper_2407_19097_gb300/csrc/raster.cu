@@ -141,11 +141,24 @@ __device__ __noinline__ void render_point_wide(const RView& v, float x, float y,
     render_point(v, x, y, z, idx);
 }
 
-// The points of a group that project4 leaves to the wide path.
-__device__ __forceinline__ void render_wide4(const RView& v, const f2* X, const f2* Y, const f2* Z,
-                                             const uint32_t* idx, uint32_t in) {
+// The points of a group that project4 leaves to the wide path.  Few scenes have one, however wide
+// the view's range (an unbounded far plane is common), so the four depths come first, two by two
+// and by project4's sequence; f: the same view in shared memory.  Kept out of render_view: a mask
+// returned from there cost the bounded views 1 to 4%.  Terrain, 9M points, eight views of 960 x
+// 540: 291 us with the plain division of every point, 233 here, 221 with a bounded range.
+__device__ __forceinline__ void render_wide4(const FView& f, const RView& v, const f2* X, const f2* Y,
+                                             const f2* Z, const uint32_t* idx, uint32_t in) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
+        const f2 xy = f2_fma(f2_mul(f.m[9], Y[h]), f.one, f2_mul(f.m[8], X[h]));
+        float w[2];
+        f2_unpack(f2_add(f2_fma(f2_mul(f.m[10], Z[h]), f.one, xy), f.m[11]), w[0], w[1]);
+        // bits order like the values of non-negative floats; negative ones and NaN are above infinity
+        auto fast = [](float d) {
+            const uint32_t b = __float_as_uint(d);
+            return b - FAST_W_LO <= FAST_W_HI - FAST_W_LO || b > 0x7F800000u;
+        };
+        if (fast(w[0]) && fast(w[1])) continue;
         float x[2], y[2], z[2];
         f2_unpack(X[h], x[0], x[1]);
         f2_unpack(Y[h], y[0], y[1]);
@@ -276,7 +289,7 @@ __global__ void __launch_bounds__(256, MINB) visibility_kernel(const float4* __r
             FView fv;
             if (!SINGLE) fv = fs[v];
             render_view<true>(SINGLE ? f0 : fv, X, Y, Z, idx, 15u);
-            if (fs[v].wide) render_wide4(vs.v[v], X, Y, Z, idx, 15u);
+            if (fs[v].wide) render_wide4(fs[v], vs.v[v], X, Y, Z, idx, 15u);
         }
         if (PREFETCH) {
             a = na;
@@ -645,7 +658,7 @@ __global__ void __launch_bounds__(256, 4) chunk_render_kernel(const float* __res
             FView fv;
             if (!SINGLE) fv = fs[v];
             render_view<false>(SINGLE ? freg : fv, X, Y, Z, idx, inv);
-            if (fs[v].wide) render_wide4(vs.v[v], X, Y, Z, idx, inv);
+            if (fs[v].wide) render_wide4(fs[v], vs.v[v], X, Y, Z, idx, inv);
         }
     };
     // up to four chunks: one point of each per lane
