@@ -163,6 +163,9 @@ nrv_status tc_wgrad_up(const Net* net, int l, const void* g, int g_ld, int g_off
 nrv_status tc_wgrad(const Net* net, int l, const void* g, const void* x1, int c1, const void* x2,
                     int c2, int n, int H, int W, float* part, size_t part_floats, float* partb,
                     int* nsplit, cudaStream_t s);
+// The splits that tc_wgrad or tc_wgrad_up (by the layer's kind) makes of layer l at (n, H, W) when
+// the buffer of partial sums has room for them (0: too many tiles, both are unsupported).
+nrv_status tc_wgrad_splits(const Net* net, int l, int n, int H, int W, int* splits);
 // data gradient of 3x3 conv layer l on the tensor cores (BF16, row-planar): out = conv3x3 of
 // the output gradient gin with the flipped, transposed kernel, zeroed where mask <= 0 (mask
 // may be null); NRV_ERR_UNSUPPORTED when the layer has no such path

@@ -671,11 +671,12 @@ struct Bwd {
                               !x1.coff && x1.ld == c1 &&
                               (!c2 || (x2.planar && !x2.coff && x2.ld == c2));
             if (fits) {
-                const size_t per_split = (size_t)L.cout * 9 * cin, max_split = tc_splits(cin);
+                int max_split = 0, nsplit = 0;
+                NRV_TRY(tc_wgrad_splits(net, l, g.n, g.h[level], g.w[level], &max_split));
+                const size_t per_split = (size_t)L.cout * 9 * cin, mark = parts.used;
                 float* part = parts.take(max_split * per_split);
-                float* partb = parts.take(max_split * L.cout);
+                float* partb = parts.take((size_t)max_split * L.cout);
                 if (!part || !partb) return fail(NRV_ERR_STATE, "partial sums");
-                int nsplit = 0;
                 const nrv_status st = tc_wgrad(net, l, gpre.p, x1.p, c1, c2 ? x2.p : nullptr, c2, g.n,
                                                g.h[level], g.w[level], part, max_split * per_split,
                                                partb, &nsplit, sw);
@@ -688,6 +689,7 @@ struct Bwd {
                 }
                 if (st != NRV_ERR_UNSUPPORTED) return st;
                 clear_error();
+                parts.used = mark;
             }
         }
         const int h = g.h[level], w = g.w[level];
@@ -713,12 +715,8 @@ struct Bwd {
         return NRV_OK;
     }
 
-    // Splits of a layer's weight gradient: at most this many on the tensor cores; on the CUDA
-    // cores in BF16 about four blocks per SM in all, each a contiguous run of tpb tiles.
-    static size_t tc_splits(int cin) {
-        const int groups = cin / 16 > 0 ? cin / 16 : 1;
-        return (size_t)(304 + groups - 1) / groups;
-    }
+    // Splits of a layer's weight gradient on the CUDA cores in BF16: about four blocks per SM in
+    // all, each a contiguous run of tpb tiles.
     int simt_splits(int cout, int cin, int h, int w, int* tpb) const {
         const int CG = cin < 16 ? cin : 16, TW = wgrad_tile_width(w), R = WG_TILE / TW;
         const long long ntiles = (long long)g.n * ((h + R - 1) / R) * ((w + TW - 1) / TW);
@@ -738,35 +736,26 @@ struct Bwd {
         *chunk = (npx + nch - 1) / nch;
         return (int)((npx + *chunk - 1) / *chunk);
     }
-    // Floats of partial sums layer l may take (either path), its pixels at `level` of g.
-    size_t need(int l, int level) const {
+    // Floats of partial sums that layer l takes, its pixels at `level` of g: one path's, the larger
+    // of the two in BF16 (the CUDA cores are for layers that the tensor cores refuse).
+    nrv_status need(int l, int level, size_t* floats) const {
         const Layer& L = net->layers[l];
         const int h = g.h[level], w = g.w[level];
-        auto pad = [](size_t f) { return (f + 31) / 32 * 32; };
-        size_t per, bias, ns;
-        if (L.kind == CONV3) {
-            const int cin = l == L_E0A ? net->c0p : L.cin;
-            int tpb;
-            per = (size_t)L.cout * 9 * cin;
-            bias = L.cout;
-            if (sizeof(T) == 4) return pad(f32_wgrad_splits(cin, L.cout, g.n, h, w) * per) + pad((size_t)f32_wgrad_splits(cin, L.cout, g.n, h, w) * bias);
-            ns = simt_splits(L.cout, cin, h, w, &tpb);
-            return pad(tc_splits(cin) * per) + pad(tc_splits(cin) * bias) + pad(ns * per) + pad(ns * bias);
-        }
-        per = (size_t)L.cin * 4 * L.cout;
-        bias = 4 * L.cout;
+        const bool conv = L.kind == CONV3;
+        const int cin = l == L_E0A ? net->c0p : L.cin;
+        const size_t per = (conv ? 9 : 4) * (size_t)L.cout * cin, bias = conv ? L.cout : 4 * L.cout;
+        auto room = [&](size_t ns) { return (ns * per + 31) / 32 * 32 + (ns * bias + 31) / 32 * 32; };
         if (sizeof(T) == 4) {
-            ns = f32_wgrad_up_splits(L.cin, L.cout, g.n, h, w);
-            return pad(ns * per) + pad(ns * bias);
+            *floats = room(conv ? f32_wgrad_splits(cin, L.cout, g.n, h, w)
+                                : f32_wgrad_up_splits(cin, L.cout, g.n, h, w));
+            return NRV_OK;
         }
+        int tpb, tc = 0;
         size_t chunk;
-        ns = simt_up_splits(L.cin, g.px(level), &chunk);
-        const size_t tc = up_splits(L.cout);
-        return pad(tc * per) + pad(tc * bias) + pad(ns * per) + pad(ns * bias);
-    }
-    static size_t up_splits(int cout) {
-        const int groups = 4 * cout <= 128 ? 1 : 2;
-        return (size_t)(304 + groups - 1) / groups;
+        NRV_TRY(tc_wgrad_splits(net, l, g.n, h, w, &tc));
+        const size_t simt = conv ? simt_splits(L.cout, cin, h, w, &tpb) : simt_up_splits(cin, g.px(level), &chunk);
+        *floats = room(simt > (size_t)tc ? simt : (size_t)tc);
+        return NRV_OK;
     }
 
     nrv_status dgrad_conv(int l, TView<const T> gpre, TView<T> out, TView<const T> mask,
@@ -822,11 +811,12 @@ struct Bwd {
         if (sizeof(T) == 2 && x.planar && !x.coff && x.ld == L.cin && gout.planar &&
             gout.ld % 8 == 0 && gout.coff % 8 == 0 && gout.coff + L.cout <= gout.ld) {
             // BF16: on the tensor cores, the bias gradient beside it
-            const size_t per_split = (size_t)L.cin * 4 * L.cout, max_split = up_splits(L.cout);
+            int max_split = 0, nsplit = 0;
+            NRV_TRY(tc_wgrad_splits(net, l, g.n, g.h[level_in], g.w[level_in], &max_split));
+            const size_t per_split = (size_t)L.cin * 4 * L.cout, mark = parts.used;
             float* part = parts.take(max_split * per_split);
-            float* partb = parts.take(max_split * 4 * L.cout);
+            float* partb = parts.take((size_t)max_split * 4 * L.cout);
             if (!part || !partb) return fail(NRV_ERR_STATE, "partial sums");
-            int nsplit = 0;
             const nrv_status st = tc_wgrad_up(net, l, gout.p, gout.ld, gout.coff, x.p, g.n,
                                               g.h[level_in], g.w[level_in], part,
                                               max_split * per_split, partb, &nsplit, sw);
@@ -840,6 +830,7 @@ struct Bwd {
             }
             if (st != NRV_ERR_UNSUPPORTED) return st;
             clear_error();
+            parts.used = mark;
         }
         const size_t npx = g.px(level_in);
         const int K = 4 * L.cout;
@@ -936,7 +927,11 @@ struct Bwd {
         if (hchunk < 64) hchunk = 64;
         hch = (tot + hchunk - 1) / hchunk;
         size_t floats = (hch * 51 + 31) / 32 * 32;
-        for (int l = 0; l < L_HEAD; ++l) floats += need(l, lvl[l]);
+        for (int l = 0; l < L_HEAD; ++l) {
+            size_t f = 0;
+            NRV_TRY(need(l, lvl[l], &f));
+            floats += f;
+        }
         NRV_TRY(net->partial.ensure(floats * sizeof(float)));
         NRV_TRY(net_side_stream(net));
         sw = net->side;
@@ -1027,7 +1022,9 @@ struct Bwd {
     // one layer's weight gradient alone, on s
     template <typename Fn>
     nrv_status alone(int l, Fn fn) {
-        NRV_TRY(net->partial.ensure(need(l, 0) * sizeof(float)));
+        size_t floats = 0;
+        NRV_TRY(need(l, 0, &floats));
+        NRV_TRY(net->partial.ensure(floats * sizeof(float)));
         NRV_TRY(fn());
         return parts.flush(s);
     }

@@ -298,21 +298,36 @@ __global__ void __launch_bounds__(WG_NT, 1)
 
 }  // namespace
 
-// Launch: grid (splits, groups), two stages of (A block, B block), partials in `part`.
+// Planes of a stage whose A and B blocks hold `planes`: the ones planes after them, and at least the
+// 16 planes (M = 128) that the A descriptor spans from its block.
+static uint32_t stage_planes(uint32_t planes) { return planes + 2 < 16 ? 16 : planes + 2; }
+// CTAs per SM (TMEM: 256 columns each): two where two stages of 128 pixels fit twice; the stages
+// of narrower tiles then share that space.
+static int wg_per_sm(uint32_t planes) { return 2 * stage_planes(planes) * 2048 <= 110 * 1024 ? 2 : 1; }
+// Splits of K over the CTAs of one channel group, at most one per tile.
+static nrv_status wg_splits(int per_sm, int groups, int ntiles, long long* ns) {
+    static int sms = 0;
+    if (!sms) {
+        int dev = 0;
+        NRV_CHECK_CUDA(cudaGetDevice(&dev));
+        NRV_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+        if (sms <= 0) sms = 148;
+    }
+    *ns = (long long)sms * per_sm / groups;
+    if (*ns < 1) *ns = 1;
+    if (*ns > ntiles) *ns = ntiles;
+    return NRV_OK;
+}
+
+// Launch: grid (splits, groups), stages of (A block, B block), partials in `part`.
 static nrv_status wg_launch(WgParams& P, int groups, const CUtensorMap& mg, const CUtensorMap& m1,
                             const CUtensorMap& m2, size_t per_split, float* part,
                             size_t part_floats, float* partb, int* nsplit, cudaStream_t s) {
     P.status = status_word();
     if (!P.status) return fail(NRV_ERR_CUDA, "status word unavailable");
-    // the A descriptor spans 16 planes (M = 128) from its block: keep that inside the stage
-    auto stage = [&](uint32_t plane) {
-        const uint32_t bytes = (P.a_bytes + P.b_bytes_span) / P.plane * plane + 2 * plane;
-        return bytes < 16u * plane ? 16u * plane : bytes;
-    };
-    P.stage_bytes = stage(P.plane);
-    // CTAs per SM (TMEM: 256 columns each): two where two stages of 128 pixels fit twice; the
-    // stages of narrower tiles then share that space
-    const int per_sm = 2 * stage(2048) <= 110 * 1024 ? 2 : 1;
+    const uint32_t planes = (P.a_bytes + P.b_bytes_span) / P.plane;
+    P.stage_bytes = stage_planes(planes) * P.plane;
+    const int per_sm = wg_per_sm(planes);
     const uint32_t room = per_sm == 2 ? 110 * 1024 : 215 * 1024;
     P.nst = (int)(room / P.stage_bytes);
     if (P.nst > WG_STAGES) P.nst = WG_STAGES;
@@ -325,16 +340,8 @@ static nrv_status wg_launch(WgParams& P, int groups, const CUtensorMap& mg, cons
                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 215 * 1024));
         attr = true;
     }
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        NRV_CHECK_CUDA(cudaGetDevice(&dev));
-        NRV_CHECK_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-        if (sms <= 0) sms = 148;
-    }
-    long long ns = (long long)sms * per_sm / groups;
-    if (ns < 1) ns = 1;
-    if (ns > P.ntiles) ns = P.ntiles;
+    long long ns = 0;
+    NRV_TRY(wg_splits(per_sm, groups, P.ntiles, &ns));
     if ((size_t)ns * per_split > part_floats) ns = (long long)(part_floats / per_split);
     if (ns < 1) return fail(NRV_ERR_ARG, "partial buffer too small");
     P.nsplit = (int)ns;
@@ -366,10 +373,37 @@ static nrv_status wg_geometry(WgParams& P, int n, int H, int W) {
     return NRV_OK;
 }
 
+// Channel groups of a transposed conv: all four kernel positions in one CTA while 4 C_out rows fit
+// in M = 128, else two groups (by a).
+static int up_groups(int cout) { return 4 * cout <= 128 ? 1 : 2; }
+
 // instruction descriptor: FP32 accumulator, A and B BF16 MN-major, M = 128
 static uint32_t wg_idesc(int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
            ((uint32_t)(N >> 3) << 17) | ((uint32_t)(128 >> 4) << 24);
+}
+
+nrv_status tc_wgrad_splits(const Net* net, int l, int n, int H, int W, int* splits) {
+    const Layer& L = net->layers[l];
+    WgParams P;
+    memset(&P, 0, sizeof(P));
+    *splits = 0;
+    const nrv_status st = wg_geometry(P, n, H, W);
+    if (st == NRV_ERR_UNSUPPORTED) {
+        clear_error();
+        return NRV_OK;
+    }
+    NRV_TRY(st);
+    long long ns = 0;
+    if (L.kind == CONV3) {
+        const int cin = l == L_E0A ? net->c0p : L.cin;
+        NRV_TRY(wg_splits(wg_per_sm(L.cout / 8 + 18), cin == 8 ? 1 : cin / 16, P.ntiles, &ns));
+    } else {
+        const int groups = up_groups(L.cout);
+        NRV_TRY(wg_splits(wg_per_sm(4 / groups * (L.cout / 8) + L.cin / 8), groups, P.ntiles, &ns));
+    }
+    *splits = (int)ns;
+    return NRV_OK;
 }
 
 nrv_status tc_wgrad(const Net* net, int l, const void* g, const void* x1, int c1, const void* x2,
@@ -419,8 +453,7 @@ nrv_status tc_wgrad_up(const Net* net, int l, const void* g, int g_ld, int g_off
     P.cout = L.cout;
     P.cin = L.cin;
     P.groups1 = 0;
-    // kernel positions per CTA: all four while 4 C_out rows fit in M = 128, else split by a
-    const int groups = 4 * L.cout <= 128 ? 1 : 2;
+    const int groups = up_groups(L.cout);
     P.n_ab = 4 / groups;
     P.m_real = P.n_ab * L.cout;
     P.ncols = L.cin;
