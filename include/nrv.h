@@ -571,7 +571,8 @@ int nrv_get_timings(float* ms, int cap);
  * file, nrv_tune_load reads one back (a later process then skips the timing); when the
  * environment variable NRV_TUNE_CACHE names an existing file, the library loads it at
  * its first lookup.  Format: '#' comment lines and one choice per line,
- * "<key> = <value>", the key free text ("render multi=1 log2n=27", "conv ...") and
+ * "<key> = <value>", the key free text ("render multi=1 log2n=27 table=9f0c1a52", "conv ...":
+ * the table is a hash of the variants, so a file of another build's selects nothing) and
  * the value a non-negative integer.  nrv_tune_count gives the number of choices held,
  * nrv_tune_timings the number of tuning runs this process made.  No counterpart in
  * the paper.  Errors: NRV_ERR_ARG (null path, I/O, a malformed line). */

@@ -969,6 +969,18 @@ int visibility_variant_count(int multi) {
 }
 const char* visibility_variant_name(int multi, int i) { return (multi ? kMulti : kSingle)[i].name; }
 
+// FNV-1a over the names of a variant table, in order.  A stored choice is an index into the table:
+// with the table's hash in its key, a file saved with other variants selects none of these.
+static uint32_t variant_table_hash(int multi) {
+    uint32_t h = 2166136261u;
+    for (int i = 0; i < visibility_variant_count(multi); ++i)
+        for (const char* c = visibility_variant_name(multi, i);; ++c) {
+            h = (h ^ (uint8_t)*c) * 16777619u;
+            if (!*c) break;
+        }
+    return h;
+}
+
 static bool verbose() {
     static int v = -1;
     if (v < 0) {
@@ -993,8 +1005,9 @@ nrv_status launch_visibility(const float* xyz, uint64_t n, const RViews& views, 
     int cls = 0;
     while (cls < 47 && (1ull << (cls + 1)) <= n) ++cls;
     int& choice = g_vis_choice[multi][cls];
+    static const uint32_t table[2] = {variant_table_hash(0), variant_table_hash(1)};
     char tkey[64];
-    snprintf(tkey, sizeof(tkey), "render multi=%d log2n=%d", multi, cls);
+    snprintf(tkey, sizeof(tkey), "render multi=%d log2n=%d table=%08x", multi, cls, table[multi]);
     if (choice == 0) {
         int v = 0;
         if (tune_get(tkey, &v) && v >= 0 && v < count) choice = v + 1;
