@@ -474,7 +474,9 @@ nrv_status nrv_net_backward(nrv_net* net, const float* d_drgb, float* d_grad, nr
 
 /* L1 loss of Sec. 3.3's reconstruction term, in the L1 form:
  * loss = mean |y - t| over n floats, written to d_loss[0]; if d_dy is not NULL,
- * d_dy = sign(y - t) / n with sign(0) = 0.  Deterministic. */
+ * d_dy = sign(y - t) / n with sign(0) = 0.  Deterministic.  Like nrv_recon_loss it
+ * takes 2 KB of partial sums in the order of its stream, so calls may overlap on
+ * different streams; the pool behind them keeps 32 MB of the device once used. */
 nrv_status nrv_l1_loss(const float* d_y, const float* d_t, int64_t n, float* d_loss, float* d_dy,
                        nrv_stream stream);
 

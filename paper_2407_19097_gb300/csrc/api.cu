@@ -597,17 +597,18 @@ extern "C" nrv_status nrv_train_step(nrv_net* net, float* params, float* grad, f
     if (prec >= NRV_PREC_FP8_E4M3) return fail(NRV_ERR_UNSUPPORTED, "training runs in F32 or BF16");
     cudaStream_t st = (cudaStream_t)stream;
     const size_t nout = (size_t)n * h * w * 3;
-    NRV_TRY(net->batch_ws.ensure(2 * nout * sizeof(float)));
+    NRV_TRY(net->batch_ws.ensure((2 * nout + LOSS_PARTS) * sizeof(float)));
     float* y = (float*)net->batch_ws.p;
     float* dy = y + nout;
+    float* part = dy + nout;
     NRV_TRY(net_forward(net, netin, n, h, w, prec, y, st));
     net->saved_in = netin;
     net->saved = true;
     const nrv_loss_weights& lw = net->loss_w;
     if (lw.l1 == 1.0f && lw.l2 == 0.0f && lw.tv == 0.0f)
-        NRV_TRY(launch_l1(y, target, (int64_t)nout, loss, dy, st));
+        NRV_TRY(launch_l1(y, target, (int64_t)nout, loss, dy, st, part));
     else
-        NRV_TRY(launch_recon(y, target, n, h, w, lw, loss, dy, st));
+        NRV_TRY(launch_recon(y, target, n, h, w, lw, loss, dy, st, part));
     NRV_TRY(net_backward(net, dy, grad, st));
     NRV_TRY(launch_adam(params, grad, m, v, net->n_params, step, lr, 0.9f, 0.999f, 1e-8f, st));
     NRV_CHECK_CUDA(cudaMemcpyAsync(net->params.p, params, net->n_params * sizeof(float),

@@ -202,11 +202,14 @@ nrv_status forward_fp8_mixed(Net* net, const void* netin, float* rgb, cudaStream
 void layer_scale_index(int l, int* in1, int* in2, int* out);
 nrv_status net_calibrate(Net* net, const void* netin, int n, int H, int W, cudaStream_t s);
 
-// training kernels (train.cu)
+// training kernels (train.cu); part: LOSS_PARTS floats for a loss's partial sums, null to have them
+// allocated in the order of the stream
+constexpr int LOSS_PARTS = 512;
 nrv_status launch_l1(const float* y, const float* t, int64_t n, float* loss, float* dy,
-                     cudaStream_t s);
+                     cudaStream_t s, float* part = nullptr);
 nrv_status launch_recon(const float* y, const float* t, int n_img, int h, int w,
-                        const nrv_loss_weights& wt, float* loss, float* dy, cudaStream_t s);
+                        const nrv_loss_weights& wt, float* loss, float* dy, cudaStream_t s,
+                        float* part = nullptr);
 nrv_status launch_adam(float* p, const float* g, float* m, float* v, int64_t n, int step,
                        float lr, float b1, float b2, float eps, cudaStream_t s);
 

@@ -4,6 +4,8 @@
 // Gradients of the weights are reductions over all pixels.  They are computed
 // in fixed pixel chunks whose partial sums are added in a fixed order by a
 // second kernel, so a step is bit-for-bit reproducible.
+#include <mutex>
+
 #include "f32.h"
 #include "net.h"
 #include "net_simt.cuh"
@@ -518,16 +520,71 @@ __global__ void l1_final_kernel(const float* part, int nb, double inv_n, float* 
     if (threadIdx.x == 0) loss[0] = (float)(red[0] * inv_n);
 }
 
-static DevBuf g_l1_part;
+// Where a loss puts its LOSS_PARTS partial sums: the caller's memory (a net's, one call at a time
+// anyway) or, for the free-standing losses, 2 KB of its own that the stream's order gives and
+// takes back -- calls on other streams, threads and devices have theirs, and a captured call's
+// belong to its graph.  They come from a pool per device that keeps its memory between calls (one
+// reservation of the driver's, 32 MB, holds those of 16K calls in flight); emptied at every
+// synchronisation it cost 170 us a call, kept 3 us over one buffer shared by all calls (a small
+// loss waited for: 23 -> 26 us), which raced.
+struct LossParts {
+    static constexpr size_t BYTES = LOSS_PARTS * sizeof(float);
+    float* p;
+    cudaStream_t s;
+    bool own = false;
+    LossParts(float* given, cudaStream_t stream) : p(given), s(stream) {}
+    LossParts(const LossParts&) = delete;
+    LossParts& operator=(const LossParts&) = delete;
+    ~LossParts() {
+        if (own) cudaFreeAsync(p, s);
+    }
+    nrv_status take() {
+        if (p) return NRV_OK;
+        const cudaMemPool_t pool = device_pool();
+        if (!pool || cudaMallocFromPoolAsync((void**)&p, BYTES, pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            if (cudaMallocAsync((void**)&p, BYTES, s) != cudaSuccess) {
+                p = nullptr;
+                cudaGetLastError();
+                return fail(NRV_ERR_OOM, "no device memory for a loss's partial sums");
+            }
+        }
+        own = true;
+        return NRV_OK;
+    }
+    // the current device's pool, made on first use; null where there is none
+    static cudaMemPool_t device_pool() {
+        static std::mutex mu;
+        static cudaMemPool_t pools[64] = {};
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+        std::lock_guard<std::mutex> lock(mu);
+        if (!pools[dev]) {
+            cudaMemPoolProps props;
+            memset(&props, 0, sizeof(props));
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            cudaMemPool_t pool = nullptr;
+            if (cudaMemPoolCreate(&pool, &props) != cudaSuccess) return nullptr;
+            uint64_t keep = ~0ull;
+            int no = 0;   // one stream's call never waits for another's memory
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            cudaMemPoolSetAttribute(pool, cudaMemPoolReuseAllowInternalDependencies, &no);
+            pools[dev] = pool;
+        }
+        return pools[dev];
+    }
+};
 
 nrv_status launch_l1(const float* y, const float* t, int64_t n, float* loss, float* dy,
-                     cudaStream_t s) {
-    const int nb = 512;
-    NRV_TRY(g_l1_part.ensure(nb * sizeof(float)));
+                     cudaStream_t s, float* part) {
+    LossParts parts(part, s);
+    NRV_TRY(parts.take());
     const int vec = (((uintptr_t)y | (uintptr_t)t | (uintptr_t)dy) & 15) == 0;
-    l1_partial_kernel<<<nb, 256, 0, s>>>(y, t, n, dy, (float)(1.0 / (double)n), (float*)g_l1_part.p, vec);
+    l1_partial_kernel<<<LOSS_PARTS, 256, 0, s>>>(y, t, n, dy, (float)(1.0 / (double)n), parts.p, vec);
     NRV_CHECK_LAUNCH();
-    l1_final_kernel<<<1, 256, 0, s>>>((const float*)g_l1_part.p, nb, 1.0 / (double)n, loss);
+    l1_final_kernel<<<1, 256, 0, s>>>(parts.p, LOSS_PARTS, 1.0 / (double)n, loss);
     NRV_CHECK_LAUNCH();
     return NRV_OK;
 }
@@ -578,16 +635,16 @@ __global__ void recon_partial_kernel(const float* __restrict__ y, const float* _
 }
 
 nrv_status launch_recon(const float* y, const float* t, int n_img, int h, int w,
-                        const nrv_loss_weights& wt, float* loss, float* dy, cudaStream_t s) {
-    const int nb = 512;
-    NRV_TRY(g_l1_part.ensure(nb * sizeof(float)));
+                        const nrv_loss_weights& wt, float* loss, float* dy, cudaStream_t s, float* part) {
+    LossParts parts(part, s);
+    NRV_TRY(parts.take());
     const int64_t n = (int64_t)n_img * h * w * 3;
     const double nh = (double)n_img * h * (w - 1) * 3, nv = (double)n_img * (h - 1) * w * 3;
-    recon_partial_kernel<<<nb, 256, 0, s>>>(y, t, n, h, w, dy, wt.l1, wt.l2, wt.tv,
+    recon_partial_kernel<<<LOSS_PARTS, 256, 0, s>>>(y, t, n, h, w, dy, wt.l1, wt.l2, wt.tv,
                                             (float)(1.0 / (double)n), nh > 0 ? (float)(1.0 / nh) : 0.0f,
-                                            nv > 0 ? (float)(1.0 / nv) : 0.0f, (float*)g_l1_part.p);
+                                            nv > 0 ? (float)(1.0 / nv) : 0.0f, parts.p);
     NRV_CHECK_LAUNCH();
-    l1_final_kernel<<<1, 256, 0, s>>>((const float*)g_l1_part.p, nb, 1.0, loss);
+    l1_final_kernel<<<1, 256, 0, s>>>(parts.p, LOSS_PARTS, 1.0, loss);
     NRV_CHECK_LAUNCH();
     return NRV_OK;
 }

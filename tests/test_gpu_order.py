@@ -68,3 +68,49 @@ def test_train_steps_back_to_back():
 
     (la, pa), (lb, pb) = run(True), run(False)
     assert torch.equal(la, lb) and torch.equal(pa, pb)
+
+
+@pytest.mark.parametrize("kind", ["l1", "recon"])
+def test_losses_on_two_streams(kind):
+    """Losses in flight on two streams at once, and a captured one replayed beside them, have
+    partial sums of their own: each value is that of the call alone."""
+    import torch
+    from paper_2407_19097_gb300 import nrv
+    dev = torch_dev()
+    shapes = [(2, 512, 512, 3), (1, 64, 96, 3), (4, 512, 512, 3)]
+    pairs = [[torch.rand(s, device=dev, generator=torch.Generator(device=dev).manual_seed(10 * i + j))
+              for j in range(2)] for i, s in enumerate(shapes)]
+
+    def call(i, out, d):
+        y, t = pairs[i]
+        if kind == "l1":
+            nrv.l1_loss(y, t, out, d)
+        else:
+            nrv.recon_loss(y, t, (0.5, 1.0, 0.25), out, d)
+
+    refs = []
+    for i, (y, _) in enumerate(pairs):
+        out, d = torch.zeros(1, device=dev), torch.empty_like(y)
+        call(i, out, d)
+        torch.cuda.synchronize()
+        refs.append((out, d))
+    streams = [torch.cuda.Stream() for _ in range(3)]
+    rounds = 60
+    outs = [torch.zeros((rounds, 1), device=dev) for _ in pairs]
+    grads = [torch.empty_like(y) for y, _ in pairs]
+    graph_out = torch.zeros(1, device=dev)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=streams[2]):
+        call(2, graph_out, grads[2])
+    torch.cuda.synchronize()
+    for r in range(rounds):
+        for i in range(2):
+            with torch.cuda.stream(streams[i]):
+                call(i, outs[i][r], grads[i])
+        with torch.cuda.stream(streams[2]):
+            graph.replay()
+            outs[2][r].copy_(graph_out)
+    torch.cuda.synchronize()
+    for i, (ref, d) in enumerate(refs):
+        assert torch.equal(outs[i], ref.expand(rounds, 1)), i
+        assert torch.equal(grads[i], d), i
