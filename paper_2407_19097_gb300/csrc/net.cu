@@ -184,40 +184,44 @@ static nrv_status simt_conv3(const Net* net, int l, TView<const T> x1, int c1, T
     const Layer& L = net->layers[l];
     const float* wf = (const float*)net->wf32.p + net->wf_off[l];
     const float* bias = (const float*)net->params.p + L.boff;
-    if constexpr (sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4) {
         return f32_conv3(x1.p, c1, x2.p, c2, wf, bias, relu ? 1 : 0, nullptr, y.p, L.cout, g.n, g.h[level],
                          g.w[level], s);
-    Conv3Args<T> a;
-    a.x1 = x1; a.x2 = x2; a.c1 = c1; a.c2 = c2;
-    a.w = wf;
-    a.bias = bias;
-    a.y = y;
-    a.cout = L.cout;
-    a.n = g.n; a.h = g.h[level]; a.w_ = g.w[level];
-    a.relu = relu ? 1 : 0;
-    a.mask = TView<const T>{nullptr, 0};
-    const size_t npx = g.px(level);
-    dim3 grid((unsigned)((npx + 127) / 128), L.cout / 16);
-    const size_t smem = (size_t)9 * (c1 + c2) * 16 * 4;
-    conv3_simt_kernel<T><<<grid, 128, smem, s>>>(a);
-    NRV_CHECK_LAUNCH();
-    return NRV_OK;
+    } else {
+        Conv3Args<T> a;
+        a.x1 = x1; a.x2 = x2; a.c1 = c1; a.c2 = c2;
+        a.w = wf;
+        a.bias = bias;
+        a.y = y;
+        a.cout = L.cout;
+        a.n = g.n; a.h = g.h[level]; a.w_ = g.w[level];
+        a.relu = relu ? 1 : 0;
+        a.mask = TView<const T>{nullptr, 0};
+        const size_t npx = g.px(level);
+        dim3 grid((unsigned)((npx + 127) / 128), L.cout / 16);
+        const size_t smem = (size_t)9 * (c1 + c2) * 16 * 4;
+        conv3_simt_kernel<T><<<grid, 128, smem, s>>>(a);
+        NRV_CHECK_LAUNCH();
+        return NRV_OK;
+    }
 }
 
 template <typename T>
 static nrv_status simt_upconv(const Net* net, int l, TView<const T> x, TView<T> y, int n, int hi,
                               int wi, cudaStream_t s) {
     const Layer& L = net->layers[l];
-    if constexpr (sizeof(T) == 4)
+    if constexpr (sizeof(T) == 4) {
         return f32_upconv(x.p, L.cin, (const float*)net->wf32.p + net->wf_off[l],
                           (const float*)net->params.p + L.boff, y.p, L.cout, n, hi, wi, s);
-    const size_t npx = (size_t)n * hi * wi * 4;
-    dim3 grid((unsigned)((npx + 127) / 128), L.cout / 16);
-    upconv2_kernel<T><<<grid, 128, (size_t)4 * L.cin * 16 * 4, s>>>(
-        x, L.cin, (const float*)net->wf32.p + net->wf_off[l], (const float*)net->params.p + L.boff,
-        y, L.cout, n, hi, wi);
-    NRV_CHECK_LAUNCH();
-    return NRV_OK;
+    } else {
+        const size_t npx = (size_t)n * hi * wi * 4;
+        dim3 grid((unsigned)((npx + 127) / 128), L.cout / 16);
+        upconv2_kernel<T><<<grid, 128, (size_t)4 * L.cin * 16 * 4, s>>>(
+            x, L.cin, (const float*)net->wf32.p + net->wf_off[l], (const float*)net->params.p + L.boff,
+            y, L.cout, n, hi, wi);
+        NRV_CHECK_LAUNCH();
+        return NRV_OK;
+    }
 }
 
 template <typename T>

@@ -1,8 +1,9 @@
 // SIMT kernels of the post-processing U-Net (Sec. 3.3): the small memory-bound layers
 // (pooling, head) of every precision, and the BF16 convolutions of shapes that the
-// tensor-core path does not cover (the FP32 network's are in f32.cu).  Tensors are views {ptr, channels, layout} in NHWC or in
-// the row-planar layout of the tensor-core path (see TView); storage is float
-// or bfloat16, arithmetic always FP32 with FMA.
+// tensor-core path does not cover (the FP32 network's are in f32.cu).  Tensors are
+// views {ptr, channels, layout} in NHWC or in the row-planar layout of the
+// tensor-core path (see TView); storage is float or bfloat16, arithmetic always
+// FP32 with FMA.
 #pragma once
 #include "internal.h"
 

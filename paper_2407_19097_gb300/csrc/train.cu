@@ -830,36 +830,38 @@ struct Bwd {
                 clear_error();
             }
         }
-        if constexpr (sizeof(T) == 4)
+        if constexpr (sizeof(T) == 4) {
             return f32_conv3(gpre.p, net->layers[l].cout, nullptr, 0,
                              (const float*)net->wtf32.p + net->wf_off[l], nullptr, 0, mask.p, out.p,
                              net->layers[l].cin, g.n, g.h[level], g.w[level], s);
-        // this translation unit has its own instance of the kernel template
-        static bool attr = false;
-        if (!attr) {
-            NRV_CHECK_CUDA(cudaFuncSetAttribute(conv3_simt_kernel<T>,
-                                                cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                9 * 128 * 16 * 4));
-            attr = true;
+        } else {
+            // this translation unit has its own instance of the kernel template
+            static bool attr = false;
+            if (!attr) {
+                NRV_CHECK_CUDA(cudaFuncSetAttribute(conv3_simt_kernel<T>,
+                                                    cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                    9 * 128 * 16 * 4));
+                attr = true;
+            }
+            const Layer& L = net->layers[l];
+            Conv3Args<T> a;
+            a.x1 = gpre;
+            a.c1 = L.cout;
+            a.x2 = TView<const T>{nullptr, 0};
+            a.c2 = 0;
+            a.w = (const float*)net->wtf32.p + net->wf_off[l];
+            a.bias = nullptr;
+            a.y = out;
+            a.cout = L.cin;
+            a.n = g.n; a.h = g.h[level]; a.w_ = g.w[level];
+            a.relu = 0;
+            a.mask = mask;
+            const size_t npx = g.px(level);
+            dim3 grid((unsigned)((npx + 127) / 128), L.cin / 16);
+            conv3_simt_kernel<T><<<grid, 128, (size_t)9 * L.cout * 16 * 4, s>>>(a);
+            NRV_CHECK_LAUNCH();
+            return NRV_OK;
         }
-        const Layer& L = net->layers[l];
-        Conv3Args<T> a;
-        a.x1 = gpre;
-        a.c1 = L.cout;
-        a.x2 = TView<const T>{nullptr, 0};
-        a.c2 = 0;
-        a.w = (const float*)net->wtf32.p + net->wf_off[l];
-        a.bias = nullptr;
-        a.y = out;
-        a.cout = L.cin;
-        a.n = g.n; a.h = g.h[level]; a.w_ = g.w[level];
-        a.relu = 0;
-        a.mask = mask;
-        const size_t npx = g.px(level);
-        dim3 grid((unsigned)((npx + 127) / 128), L.cin / 16);
-        conv3_simt_kernel<T><<<grid, 128, (size_t)9 * L.cout * 16 * 4, s>>>(a);
-        NRV_CHECK_LAUNCH();
-        return NRV_OK;
     }
 
     // weight and bias gradient of transposed conv l: x at level_in, gout one level up
@@ -916,7 +918,6 @@ struct Bwd {
     // ReLU output) is not positive
     nrv_status dgrad_up(int l, TView<const T> gout, TView<const T> xm, TView<T> gx, int level_in) {
         const Layer& L = net->layers[l];
-        const size_t npx = g.px(level_in);
         if (sizeof(T) == 2 && gout.planar && gx.planar && !gx.coff && gx.ld == L.cin && xm.planar &&
             !xm.coff && xm.ld == L.cin) {
             // BF16: on the tensor cores
@@ -925,16 +926,18 @@ struct Bwd {
             if (st != NRV_ERR_UNSUPPORTED) return st;
             clear_error();
         }
-        if constexpr (sizeof(T) == 4)
+        if constexpr (sizeof(T) == 4) {
             return f32_upconv_dgrad(gout.p + gout.coff, gout.ld, L.cout,
                                     (const float*)net->wtf32.p + net->wf_off[l], xm.p, gx.p, L.cin, g.n,
                                     g.h[level_in], g.w[level_in], s);
-        dim3 grid((unsigned)((npx + 127) / 128), L.cin / 16);
-        upconv2_dgrad_kernel<T><<<grid, 128, (size_t)4 * 16 * L.cout * 4, s>>>(
-            gout, L.cout, (const float*)net->wf32.p + net->wf_off[l], L.cin, xm, gx, g.n,
-            g.h[level_in], g.w[level_in]);
-        NRV_CHECK_LAUNCH();
-        return NRV_OK;
+        } else {
+            dim3 grid((unsigned)((g.px(level_in) + 127) / 128), L.cin / 16);
+            upconv2_dgrad_kernel<T><<<grid, 128, (size_t)4 * 16 * L.cout * 4, s>>>(
+                gout, L.cout, (const float*)net->wf32.p + net->wf_off[l], L.cin, xm, gx, g.n,
+                g.h[level_in], g.w[level_in]);
+            NRV_CHECK_LAUNCH();
+            return NRV_OK;
+        }
     }
 
     nrv_status pool_bwd(TView<const T> gp, TView<const T> gs, int e, TView<T> ge, int level) {
