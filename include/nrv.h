@@ -195,7 +195,9 @@ typedef struct {
  * Keys and planes are bit-exact: the projection is the fixed FP32 sequence
  *   c = ((m0*x + m1*y) + m2*z) + m3 per row (no fused multiply-add),
  *   ndc = c.xy / c.w (IEEE division).
- * n_views in 1..8; gbufs has n_views entries.  Errors: NRV_ERR_ARG. */
+ * n_views in 1..8; gbufs has n_views entries.  Views whose planes share memory are
+ * resolved in order (the last one's pixels stay); every d_key is its own.
+ * Errors: NRV_ERR_ARG. */
 nrv_status nrv_rasterize(nrv_scene* scene, const nrv_view* views, int n_views,
                          const nrv_gbuffer* gbufs, nrv_stream stream);
 

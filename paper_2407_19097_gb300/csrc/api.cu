@@ -229,6 +229,26 @@ static nrv_status raster_views(nrv_scene* s, const nrv_view* views, int n, uint6
                              s->chunks.p);
 }
 
+// Do planes of two of the views share memory?  (A caller may pass one scratch plane for several.)
+static bool planes_overlap(const ResolveArgs* a, int n) {
+    uintptr_t lo[24], hi[24];
+    int of[24], m = 0;
+    for (int i = 0; i < n; ++i) {
+        const size_t px = (size_t)a[i].width * a[i].height;
+        const void* p[3] = {a[i].depth, a[i].mask, a[i].gattr};
+        const size_t bytes[3] = {4 * px, px, 4 * px * a[i].n_words};
+        for (int k = 0; k < 3; ++k) {
+            if (!p[k]) continue;
+            lo[m] = (uintptr_t)p[k];
+            hi[m] = lo[m] + bytes[k];
+            for (int j = 0; j < m; ++j)
+                if (of[j] != i && lo[j] < hi[m] && lo[m] < hi[j]) return true;
+            of[m++] = i;
+        }
+    }
+    return false;
+}
+
 extern "C" nrv_status nrv_rasterize(nrv_scene* s, const nrv_view* views, int n,
                                     const nrv_gbuffer* gb, nrv_stream stream) {
     clear_error();
@@ -261,7 +281,11 @@ extern "C" nrv_status nrv_rasterize(nrv_scene* s, const nrv_view* views, int n,
         a.mask = gb[i].d_mask;
         a.gattr = gb[i].d_attr;
     }
-    return nr ? launch_resolve(ra, nr, st) : NRV_OK;
+    if (nr == 0) return NRV_OK;
+    if (!planes_overlap(ra, nr)) return launch_resolve(ra, nr, st);
+    // shared planes hold the last view's pixels where the views overlap: one after the other
+    for (int i = 0; i < nr; ++i) NRV_TRY(launch_resolve(&ra[i], 1, st));
+    return NRV_OK;
 }
 
 extern "C" nrv_status nrv_pack(const nrv_gbuffer* gb, int h, int w, const nrv_pack_desc* d,

@@ -114,3 +114,29 @@ def test_losses_on_two_streams(kind):
     for i, (ref, d) in enumerate(refs):
         assert torch.equal(outs[i], ref.expand(rounds, 1)), i
         assert torch.equal(grads[i], d), i
+
+
+def test_views_that_share_planes():
+    """One set of planes passed for all views of a call holds the last view's, as when the views are
+    resolved one after the other."""
+    import torch
+    import nrv_inputs as I
+    from gpu_util import gpu_raster, upload_scene
+    from paper_2407_19097_gb300 import nrv
+    sc = I.terrain_scene(300, seed=7)
+    scene, dev = upload_scene(sc), torch_dev()
+    views = I.orbit_views(sc, [(640, 480)] * 6, seed=3)
+    k = scene.n_words
+    keys = [torch.empty((480, 640), dtype=torch.int64, device=dev) for _ in views]
+    depth = torch.empty((480, 640), dtype=torch.int32, device=dev)
+    mask = torch.empty((480, 640), dtype=torch.uint8, device=dev)
+    attr = torch.empty((k, 480, 640), dtype=torch.int32, device=dev)
+    refs = gpu_raster(scene, views)
+    assert not np.array_equal(refs[0][1], refs[-1][1])
+    for _ in range(20):
+        nrv.rasterize(scene, views, keys, [depth] * 6, [mask] * 6, [attr] * 6)
+        torch.cuda.synchronize()
+        for kt, ref in zip(keys, refs):
+            assert np.array_equal(kt.cpu().numpy().view(np.uint64), ref[0])
+        for t, ref in zip((depth, mask, attr), refs[-1][1:]):
+            assert np.array_equal(t.cpu().numpy().view(ref.dtype), ref)
