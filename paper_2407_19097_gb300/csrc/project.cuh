@@ -35,13 +35,15 @@ __device__ __forceinline__ f2 f2_fma(f2 a, f2 b, f2 c) {
     asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
     return r;
 }
-// (.ftz: the depths it is used for, 2^-60 .. 2^125, and their reciprocals are normal; without
-// it every call carries a scaling for subnormal arguments, a tenth of the pass's instructions)
+// (of the gated network's epilogue)
 __device__ __forceinline__ float ex2_approx(float x) {
     float r;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
     return r;
 }
+// (.ftz: the depths it is used for, 2^-60 .. 2^125, and their reciprocals are normal; without
+// it every call carries a scaling for subnormal arguments, a tenth of the pass's instructions.  The
+// gate's denominators are at least 1.)
 __device__ __forceinline__ float rcp_approx(float v) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));

@@ -23,10 +23,12 @@
 
 namespace nrv {
 
-// Programmatic dependent launch inside the chunk-culling render pass (unless NRV_PDL=0): each
-// of its kernels is launched while the previous one drains and waits (griddepcontrol.wait)
-// for it to complete before reading anything it wrote; the kernel before the pass lets it
-// start early.  Both instructions do nothing for a plain launch.
+// Programmatic dependent launch inside the render and resolve passes (unless NRV_PDL=0): each
+// of their kernels is launched while the previous one drains and waits (griddepcontrol.wait)
+// for it to complete before reading anything it wrote.  The clear before them is a plain launch
+// that lets the next one start at once, so what a kernel reads ahead of its wait (positions, the
+// table of views) was complete before the clear began.  Both instructions do nothing for a plain
+// launch.
 __device__ __forceinline__ void pdl_wait_and_release() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -1945,8 +1945,9 @@ static nrv_status tc_launch(const Net* net, const TcLayerCfg& c, const uint8_t* 
     P.nissue = (4 * c.n_slice <= 256 && c.nks / c.rows >= 2 && c.kind != UPCONV2) ? 2 : 1;
     P.stream = c.stream && conv && !mask ? 1 : 0;
     if (P.stream) {
-        // one issuer; a ring of nb blocks in 128 TMEM columns for 16-column slices (four CTAs
-        // per SM), 256 otherwise; groups of grp rows, gm groups in flight, gm * grp + 2 <= nb
+        // one issuer; a ring of nb blocks in 256 TMEM columns (two CTAs per SM): sixteen blocks of
+        // 16 columns in groups of four rows, eight of 32 in groups of two; gm groups in flight,
+        // gm * grp + 2 <= nb
         P.nissue = 1;
         P.nb = 256 / c.n_slice;
         P.grp = (P.nb - 2) / 3;
